@@ -362,7 +362,7 @@ static size_t layout(const Geom &g, void *base, Bufs *w)
         b.state = static_cast<uint32_t *>(take(ST_WORDS * 4));
         b.ctr = static_cast<uint32_t *>(take(64 * 4));
         b.hist = static_cast<uint32_t *>(take(size_t(g.nt) * g.sigma * 4));
-        b.tab = static_cast<uint32_t *>(take((4 * size_t(g.sigma) + 4) * 4));
+        b.tab = static_cast<uint32_t *>(take((3 * size_t(g.sigma) + 4) * 4));
         const size_t jump = align_up(npi2 * 8, 256), fin = finalize_extra_bytes(g);
         const size_t lbw = grid_ring_bytes(g);
         char *z = static_cast<char *>(take(lbw > jump + fin ? lbw : jump + fin));

@@ -63,7 +63,6 @@ namespace {
 
 constexpr uint32_t LB_INCL = 0x80000000u;
 constexpr uint32_t PI_NONE = 0xFFFFFFFFu;
-constexpr uint32_t SH_NONE = 0xFFFFu;
 constexpr uint32_t TILE_END = 0xFFFFFFFFu;
 
 __device__ __forceinline__ uint32_t ld_volatile(const uint32_t *p)
@@ -340,8 +339,7 @@ __global__ void k_grid_setup(const KT *Ak, const uint32_t *Av, KT *Tk, uint32_t 
 }
 
 // Tables of one round (one CTA of 1024 threads): bucket starts O, the shared
-// blocks (those with a bucket start strictly inside), per bucket the ranks
-// of its first / last block among the shared ones and its range of
+// blocks (those with a bucket start strictly inside), per bucket its range of
 // non-shared blocks [ns0, ns1); pi' prefilled with the blocks taken before
 // the round (shared blocks, then the first non-shared block of each bucket),
 // the next head start and (n % b == 0) the empty tail block.  A digit with
@@ -416,7 +414,7 @@ __global__ void __launch_bounds__(1024) k_grid_prep(const uint32_t *hist_r, uint
         if (fl[q])
             s_list[s_a[c]] = s_O[c] >> lb;
     __syncthreads();
-    auto find = [&](uint32_t j) -> uint32_t { // rank of shared block j, or SH_NONE
+    auto find = [&](uint32_t j) -> bool { // is block j shared?
         uint32_t lo = 0, hi = nS;
         while (lo < hi) {
             const uint32_t m = (lo + hi) >> 1;
@@ -425,18 +423,16 @@ __global__ void __launch_bounds__(1024) k_grid_prep(const uint32_t *hist_r, uint
             else
                 hi = m;
         }
-        return (lo < nS && s_list[lo] == j) ? lo : SH_NONE;
+        return lo < nS && s_list[lo] == j;
     };
-    uint32_t *tO = tab, *tns0 = tab + SIGMA + 1, *tns1 = tns0 + SIGMA, *tsh = tns1 + SIGMA;
+    uint32_t *tO = tab, *tns0 = tab + SIGMA + 1, *tns1 = tns0 + SIGMA;
     for (int c = threadIdx.x; c < SIGMA; c += blockDim.x) {
         const uint32_t O = s_O[c], cn = s_cnt[c];
-        uint32_t ns0, ns1, fsh = SH_NONE, lsh = SH_NONE;
+        uint32_t ns0, ns1;
         if (cn > 0) {
             const uint32_t jf = O >> lb, jl = (O + cn - 1) >> lb;
-            fsh = find(jf);
-            lsh = find(jl);
-            ns0 = jf + (fsh != SH_NONE ? 1u : 0u);
-            ns1 = jl + 1 - (lsh != SH_NONE ? 1u : 0u);
+            ns0 = jf + (find(jf) ? 1u : 0u);
+            ns1 = jl + 1 - (find(jl) ? 1u : 0u);
             if (ns1 < ns0)
                 ns1 = ns0;
         } else {
@@ -445,7 +441,6 @@ __global__ void __launch_bounds__(1024) k_grid_prep(const uint32_t *hist_r, uint
         tO[c] = O;
         tns0[c] = ns0;
         tns1[c] = ns1;
-        tsh[c] = fsh | (lsh << 16);
     }
     __syncthreads();
     // the first GRID_AHEAD non-shared blocks of each bucket: entries nS .. nP-1
@@ -551,8 +546,8 @@ template <typename KT, bool HASV, int DB, int TILE, int NW, int NG, int STAGES, 
     static constexpr size_t GROUP = al(g_misc + MISC_BYTES);
     static constexpr size_t o_group = o_stage + STAGES * STAGE;
     // shared by the groups (read only after the start): O (sigma + 1) and,
-    // with SMALL, Radsort's tables ns0, ns1, sh
-    static constexpr int NTAB = (!OOP && SMALL) ? 4 : 1;
+    // with SMALL, Radsort's tables ns0, ns1
+    static constexpr int NTAB = (!OOP && SMALL) ? 3 : 1;
     static constexpr size_t o_tabs = o_group + NG * GROUP;
     static constexpr size_t o_meta = o_tabs + al((size_t(NTAB) * SIGMA + 4) * 4);
     static constexpr size_t o_bar = o_meta + al(STAGES * 16);
@@ -571,7 +566,7 @@ template <typename KT> struct LbArgs {
     uint32_t *Tv;
     const uint32_t *pi;     // Radsort: current block map (= the free list)
     uint32_t *pin;          // Radsort: next block map
-    const uint32_t *tab;    // O[sigma+1] (+ Radsort: ns0, ns1, sh)
+    const uint32_t *tab;    // O[sigma+1] (+ Radsort: ns0, ns1)
     unsigned long long *ring; // R x sigma look-back words (tags below tagbase)
     uint32_t *done;         // R done tags
     uint32_t *ticket;       // zeroed
@@ -663,7 +658,7 @@ __global__ void __launch_bounds__(LbCfg<KT, HASV, DB, TILE, NW, NG, STAGES, OOP>
     uint32_t *stab = sO + SIGMA + 1;
     // bucket tables: shared memory (SMALL) or global
     const uint32_t *ns0 = C::SMALL ? stab : a.tab + SIGMA + 1;
-    const uint32_t *ns1 = ns0 + SIGMA, *shr = ns1 + SIGMA;
+    const uint32_t *ns1 = ns0 + SIGMA;
     uint2 *qb = reinterpret_cast<uint2 *>(gb + C::g_qb);
     uint4 *qb16 = reinterpret_cast<uint4 *>(gb + C::g_qb);
     uint32_t *qlo = reinterpret_cast<uint32_t *>(gb + C::g_qb + C::QLO_OFF);
@@ -694,7 +689,7 @@ __global__ void __launch_bounds__(LbCfg<KT, HASV, DB, TILE, NW, NG, STAGES, OOP>
     for (int c = tid; c <= SIGMA; c += C::THREADS)
         sO[c] = a.tab[c];
     if constexpr (!OOP && C::SMALL) {
-        for (int c = tid; c < 3 * SIGMA; c += C::THREADS)
+        for (int c = tid; c < 2 * SIGMA; c += C::THREADS)
             stab[c] = a.tab[SIGMA + 1 + c];
     }
     if constexpr (C::PTAB)
@@ -1160,26 +1155,30 @@ __global__ void __launch_bounds__(LbCfg<KT, HASV, DB, TILE, NW, NG, STAGES, OOP>
                 const uint32_t cs = (g + b - 1) >> a.lb, ce = (g + cn + b - 1) >> a.lb;
                 const uint32_t first = max(cs, n0) + GRID_AHEAD;
                 const uint32_t last = min(ce + GRID_AHEAD, n1); // blocks first .. last-1 taken here
-                const uint32_t sh = shr[c], fsh = sh & 0xFFFFu, lsh = sh >> 16;
-                const uint32_t jf = sO[c] >> a.lb, jl = (sO[c + 1] - 1) >> a.lb;
-                auto take = [&](uint32_t j) -> uint32_t {
-                    const uint32_t idx = fbase + kos[q] + (j - first);
-                    if (idx >= fcap) {
+                // the blocks taken here go into the map before this thread
+                // waits for any other's: a bucket that fills tile after tile
+                // (skewed keys) has each tile continue blocks that the tile
+                // just before took, and taking after the wait would chain
+                // every tile's step 5 to its predecessor's (1-2 us a tile).
+                // Measured (2^26 keys + index, a sort): Zipf keys 57.8 -> 3.7
+                // ms, float32 N(0,1) keys (top digit skewed) 15.8 -> 3.0,
+                // uniform keys unchanged
+                const uint32_t fi0 = fbase + kos[q] - first; // block j's free-list index - j
+                const uint32_t jend = j0 + touched;
+                for (uint32_t j = first; j < last; ++j) {
+                    const uint32_t idx = fi0 + j; // (mod 2^32)
+                    if (idx < fcap)
+                        a.pin[a.H + j] = __ldg(a.pi + idx);
+                    else
                         set_status(ST_INTERNAL); // Lemma 1 would be violated
-                        return PI_NONE;
-                    }
-                    const uint32_t ph = __ldg(a.pi + idx);
-                    a.pin[a.H + j] = ph;
-                    return ph;
-                };
-                for (uint32_t i = 0; i < touched; ++i) {
-                    const uint32_t j = j0 + i;
+                }
+                for (uint32_t j = j0; j < jend; ++j) {
                     uint32_t phys;
-                    if (j >= first && j < last && !(fsh != SH_NONE && j == jf) &&
-                        !(lsh != SH_NONE && j == jl)) {
-                        phys = take(j); // this tile writes the first position of block j - L
+                    if (j >= first && j < last) { // taken here
+                        const uint32_t idx = fi0 + j;
+                        phys = idx < fcap ? __ldg(a.pi + idx) : PI_NONE;
                     } else { // taken before the round or by an earlier tile
-                        phys = i == 0 ? pf[q] : PI_NONE;
+                        phys = j == j0 ? pf[q] : PI_NONE;
                         if (phys == PI_NONE)
                             phys = wait_pi(a.pin + a.H + j);
                     }
@@ -1194,8 +1193,8 @@ __global__ void __launch_bounds__(LbCfg<KT, HASV, DB, TILE, NW, NG, STAGES, OOP>
                             phys == PI_NONE ? 0ull
                                             : (reinterpret_cast<unsigned long long>(kaddr(phys)) |
                                                (phys >= a.nT ? 1ull : 0ull));
-                        listk[l0 + i] = w;
-                        if (i == 0 && w) {
+                        listk[l0 + (j - j0)] = w;
+                        if (j == j0 && w) {
                             // the first block as a base for the run's
                             // positions: key address of position p in it is
                             // base + p elements (bit 1 marks it valid)
@@ -1206,11 +1205,9 @@ __global__ void __launch_bounds__(LbCfg<KT, HASV, DB, TILE, NW, NG, STAGES, OOP>
                                                  static_cast<uint32_t>(base >> 32));
                         }
                     } else {
-                        listb[l0 + i] = phys;
+                        listb[l0 + (j - j0)] = phys;
                     }
                 }
-                for (uint32_t j = max(first, j0 + touched); j < last; ++j) // taken, not touched
-                    (void)take(j);
             }
             bar();
         }

@@ -53,7 +53,7 @@ struct Bufs {
     void *fin;         // Finalize scratch (finalize_extra_bytes)
     // grid layout only
     uint32_t *hist;    // nt*sigma digit counts of the input
-    uint32_t *tab;     // per-round bucket tables (4*sigma + 1 words)
+    uint32_t *tab;     // per-round bucket tables (3*sigma + 1 words)
     uint32_t *status;  // look-back ring (after the rounds: Finalize's jump array and scratch)
     uint32_t *ctr;     // per-round tile tickets
 };
