@@ -656,10 +656,16 @@ static radsort_status sort_common(void *keys, uint32_t *values, size_t n, int ke
         const size_t need = scratch_bytes(n, key_bytes, hasv, digit_bits);
         void *ws = workspace;
         bool own = false;
-        if (ws) {
-            if (workspace_bytes < need || !aligned16(ws))
-                return workspace_bytes < need ? RADSORT_ENOMEM : RADSORT_EINVAL;
-        } else {
+        if (ws && (workspace_bytes < need || !aligned16(ws)))
+            return workspace_bytes < need ? RADSORT_ENOMEM : RADSORT_EINVAL;
+        if (n <= small_sort_max(key_bytes, hasv)) { // one launch, in shared memory (8-bit digits whatever the width)
+            Scope sc(1, -1, st);
+            const cudaError_t e = launch_small_sort(keys, values, static_cast<uint32_t>(n), key_bytes,
+                                                    (flags & RADSORT_KEY_FLOAT32) != 0, st);
+            if (e != cudaErrorNotSupported)
+                return cuda_status(e);
+        }
+        if (!ws) {
             cudaError_t e = cudaMallocAsync(&ws, need, st);
             if (e != cudaSuccess)
                 return cuda_status(e);
@@ -1703,7 +1709,7 @@ radsort_status radsort_device_status(void *stream)
     if (e != cudaSuccess)
         return cuda_status(e);
     const unsigned v = take_status_round() | take_status_finalize() | take_status_oop() | take_status_seg() |
-                       take_status_perm();
+                       take_status_perm() | take_status_small();
     if (v & ST_TIMEOUT)
         return RADSORT_ETIMEOUT;
     if (v & ST_INTERNAL)

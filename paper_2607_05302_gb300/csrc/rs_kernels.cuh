@@ -108,6 +108,10 @@ cudaError_t launch_lsd_oop(void *keys, uint32_t *vals, void *keys_alt, uint32_t 
 cudaError_t launch_lsd_oop_ws(void *keys, uint32_t *vals, void *keys_alt, uint32_t *vals_alt,
                               size_t n, int kb, int db, void *scratch, cudaStream_t st);
 size_t lsd_oop_scratch_bytes(size_t n, int kb, int db, bool hasv);
+// a short array (n <= small_sort_max) sorted in one launch in a cluster's
+// shared memory; flt: keys are float32 bits, transformed on the way
+uint32_t small_sort_max(int kb, bool hasv);
+cudaError_t launch_small_sort(void *keys, uint32_t *vals, uint32_t n, int kb, bool flt, cudaStream_t st);
 // batched segmented sort of the small and medium segments
 constexpr uint32_t SEG_MED = 1u << 18;
 uint32_t seg_small_max(int db);
@@ -162,6 +166,7 @@ unsigned take_status_round();
 unsigned take_status_finalize();
 unsigned take_status_oop();
 unsigned take_status_perm();
+unsigned take_status_small();
 
 // permuted representation kept between calls (grid layout; g.n is the
 // current element count, g.npi the block count of the original array)
