@@ -96,10 +96,11 @@ typedef struct {
                             nonzero with layout AUTO selects the chunk layout */
     uint32_t layout;     /* RADSORT_LAYOUT_* */
     uint32_t shape;      /* grid layout, tile shape of the round kernel:
-                            0 or 1, one CTA of 16 consumer warps per SM on the
-                            largest tiles; 2 (8-bit digits), two groups of 8
-                            warps on smaller tiles (4096 or 8192 elements),
-                            for arrays of few tiles per SM */
+                            0 or 1, one CTA of 16 ranking warps per SM on the
+                            largest tiles; 2 (8-bit digits), two CTAs of 8
+                            per SM (8-byte keys with values: one) on smaller
+                            tiles (4096 or 8192 elements), for arrays of few
+                            tiles per SM */
     uint32_t reserved[4];
 } radsort_plan;
 

@@ -148,6 +148,12 @@ __device__ __forceinline__ void named_bar(int id, int nthreads)
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 
+// Arrival without waiting at named barrier `id` (its other threads wait).
+__device__ __forceinline__ void bar_arrive(int id, int nthreads)
+{
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
+}
+
 // Mask of the lanes whose digit equals this lane's, among lanes with
 // `valid` set: one ballot per digit bit (warp-level multisplit).  All 32
 // lanes must call it.

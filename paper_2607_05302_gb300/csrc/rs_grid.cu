@@ -39,19 +39,21 @@
 // number of CTAs, and after the last round every block but the array's tail
 // is full: Finalize is a block permutation plus one tail copy.
 //
-// Round kernel (both layouts): a producer warp takes tiles in ticket order
-// and streams them into a ring of shared-memory stages with bulk copies
-// (TMA) that complete on mbarriers; the consumer warps rank each tile's
-// digits stably, publish the tile's per-digit counts, reorder the tile by
-// digit in shared memory, resolve the global per-digit offsets by look-back,
-// and store each digit run into its output blocks (Radsort) or contiguously
-// (out of place).  Look-back words live in a ring of R tiles x sigma 64-bit
-// words: (tag << 32) | value, the tag naming the round and the tile, the
-// value the tile's count or 0x80000000 | inclusive prefix (n < 2^31).  Tile t
+// Round kernels (k_lb_round8, k_lb_round11; both layouts): a producer warp
+// takes tiles in ticket order and streams them into a ring of shared-memory
+// stages with bulk copies (TMA) that complete on mbarriers; other warps rank
+// each tile's digits stably, publish the tile's per-digit counts, reorder the
+// tile by digit in shared memory, resolve the global per-digit offsets by
+// look-back, and store each digit run into its output blocks (Radsort) or
+// contiguously (out of place).  Look-back words live in a ring of R tiles x
+// sigma 64-bit words: (tag << 32) | value, the tag naming the round and the
+// tile, the value the tile's count or 0x80000000 | inclusive prefix (n < 2^31).  Tile t
 // reuses the slot of tile t - R only after every tile up to t - R + 1 has
 // finished its look-back (per-slot done tags that the producer checks).  A
 // reader that finds a slot already reused starts its look-back over: tile
 // t - R + 1 is inclusive by then, so the new walk stops above the reused slot.
+#include <type_traits>
+
 #include "rs_common.cuh"
 #include "rs_kernels.cuh"
 
@@ -474,82 +476,53 @@ __global__ void __launch_bounds__(1024) k_grid_prep(const uint32_t *hist_r, uint
         pin[i] = pi[i];
 }
 
-// ---------------------------------------------------------------- round kernel
-template <typename KT, bool HASV, int DB, int TILE, int NW, int NG, int STAGES, bool OOP> struct LbCfg {
-    static constexpr int SIGMA = 1 << DB;
-    // NG consumer groups of NW warps each; a group takes every NG-th tile and
-    // works through it on its own (its own named barrier, tables and lists),
-    // so the latency-bound phases of one group (look-back, block lists,
-    // stores) overlap the shared-memory-bound phases of another
-    static constexpr int NT = NW * 32;            // consumer threads per group
-    static constexpr int THREADS = NG * NT + 32;  // + one producer warp
+// ---------------------------------------------------------------- round kernel, 11-bit digits
+template <typename KT, bool HASV, int TILE, bool OOP> struct LbCfg {
+    static constexpr int DB = 11, SIGMA = 1 << DB, STAGES = 2, NW = 16;
+    static constexpr int NT = NW * 32;            // consumer threads
+    static constexpr int THREADS = NT + 32;       // + one producer warp
+    static constexpr int MINB = 1;                // CTAs per SM
     static constexpr int MAXM = TILE / 64;   // blocks per tile (b >= 64)
     static constexpr int R = TILE / NW;      // tile elements ranked per warp
     static constexpr int ITEMS = R / 32;     // elements per consumer thread
     static_assert(R % 32 == 0, "warp range must be a multiple of 32");
-    static_assert(THREADS <= 1024, "one CTA holds at most 1024 threads");
-    // stage s serves group s % NG only: a group waits on the phases of its
-    // own stages, in order (a stage shared by two groups could let one group
-    // see an earlier phase of the other's fill as its own)
-    static_assert(STAGES % NG == 0, "stages split evenly between the groups");
     // threads per bucket in the column passes (each sums NW / TPB warp rows):
-    // measured with 16 warps, one thread per bucket is fastest for sigma =
-    // 256 (round 1.86 -> 1.83 ms at 2^28); for sigma = 2048 two were 5%
-    // faster at 2^26 but at 2^30 u64 left some rounds 3x slower, four do not
-    static constexpr int TPB = NW >= 16 ? (DB <= 8 ? 1 : 4) : (NT >= (1 << DB) ? 1 : 2);
+    // two were 5% faster at 2^26 but at 2^30 u64 left some rounds 3x slower,
+    // four do not
+    static constexpr int TPB = 4;
     static_assert(NW % TPB == 0, "rows split evenly");
     // more than 16 elements per thread: digits are recomputed from the keys
     // and warp ranks kept as 16-bit halves, to stay within the registers
     static constexpr bool LEAN = ITEMS > 16;
-    // CTAs per SM the configuration is built for (registers are capped to fit)
-    static constexpr int MINB = (NG * NW <= 8 && DB <= 8) ? 2 : 1;
-    // sigma <= 256: a per-warp table of 32-bit lane masks by digit, built
-    // with shared-memory atomicOr; sigma = 2048: one ballot per digit bit.
-    // Either way a per-warp 16-bit row keeps the running count of each
-    // digit, later the warp's start per digit in the reordered tile.
-    static constexpr bool PTAB = DB <= 8;
+    // one ballot per digit bit finds the lanes with the same digit; a
+    // per-warp 16-bit row keeps the running count of each digit, later the
+    // warp's start per digit in the reordered tile
     static constexpr bool PAIR = HASV && sizeof(KT) == 4;
     static constexpr int HROW = SIGMA + 2;
-    // sigma <= 256: bucket tables and block lists (key / value pointers) in
-    // shared memory; sigma = 2048: tables read from global memory, block
-    // lists of block indices
-    static constexpr bool SMALL = DB <= 8;
     static constexpr size_t al(size_t x) { return (x + 127) & ~size_t(127); }
     // 16 bytes of slack per array: the lead of a misaligned source (out of place)
     static constexpr size_t KBYTES = al(size_t(TILE) * sizeof(KT) + 16);
     static constexpr size_t STAGE = al(KBYTES + (HASV ? size_t(TILE) * 4 + 16 : 0));
-    static constexpr size_t o_stage = 0;
-    // per group: warp rows, mask tables, per-bucket words (tcnt, bstart,
-    // gpos), run offsets, block list, counters and scan scratch
+    // warp rows, per-bucket words (tcnt, bstart, gpos), run offsets, block
+    // list, counters and scan scratch
     static constexpr size_t HIST_BYTES = al(size_t(NW) * HROW * 2);
-    static constexpr size_t TAB_BYTES = PTAB ? al(size_t(NW) * 2 * SIGMA * 4) : 0;
     static constexpr size_t BK_BYTES = al(size_t(3) * SIGMA * 4);
     // touched blocks per tile: at most TILE/b + 2 per bucket with elements
     static constexpr int LIST = MAXM + 2 * (SIGMA < TILE ? SIGMA : TILE) + 2;
-    // Radsort with sigma <= 256: per bucket a 16-byte run descriptor (offset,
-    // end of the run's first block, that block's base address) and the list
-    // slot of its first block; otherwise 8 bytes (offset, list slot)
-    static constexpr bool QB16 = !OOP && SMALL;
-    static constexpr size_t QLO_OFF = al(size_t(SIGMA) * (QB16 ? 16 : 8));
-    static constexpr size_t QB_BYTES = QLO_OFF + (QB16 ? al(size_t(SIGMA) * 4) : 0);
-    static constexpr size_t LK_BYTES = OOP ? 0 : al(size_t(LIST) * (SMALL ? 8 : 4));
-    // sigma = 2048: the per-bucket run offsets and the block list live in
-    // the warp-row region, which the tile no longer needs once reordered
-    static constexpr bool ALIAS = !SMALL && QB_BYTES + LK_BYTES <= HIST_BYTES;
-    static constexpr size_t MISC_BYTES = 512;
-    static constexpr size_t g_hist = 0;
-    static constexpr size_t g_tab = g_hist + HIST_BYTES;
-    static constexpr size_t g_bk = g_tab + TAB_BYTES;
-    static constexpr size_t g_qb = ALIAS ? g_hist : g_bk + BK_BYTES;
-    static constexpr size_t g_lk = g_qb + QB_BYTES;
-    static constexpr size_t g_misc = ALIAS ? g_bk + BK_BYTES : g_lk + LK_BYTES;
-    static constexpr size_t GROUP = al(g_misc + MISC_BYTES);
-    static constexpr size_t o_group = o_stage + STAGES * STAGE;
-    // shared by the groups (read only after the start): O (sigma + 1) and,
-    // with SMALL, Radsort's tables ns0, ns1
-    static constexpr int NTAB = (!OOP && SMALL) ? 3 : 1;
-    static constexpr size_t o_tabs = o_group + NG * GROUP;
-    static constexpr size_t o_meta = o_tabs + al((size_t(NTAB) * SIGMA + 4) * 4);
+    // per bucket (offset, list slot of its first block)
+    static constexpr size_t QB_BYTES = al(size_t(SIGMA) * 8);
+    static constexpr size_t LK_BYTES = OOP ? 0 : al(size_t(LIST) * 4);
+    // the per-bucket run offsets and the block list live in the warp-row
+    // region, which the tile no longer needs once reordered
+    static_assert(QB_BYTES + LK_BYTES <= HIST_BYTES, "run offsets and block list fit the warp rows");
+    static constexpr size_t o_stage = 0;
+    static constexpr size_t o_hist = STAGES * STAGE;
+    static constexpr size_t o_bk = o_hist + HIST_BYTES;
+    static constexpr size_t o_qb = o_hist;
+    static constexpr size_t o_lk = o_qb + QB_BYTES;
+    static constexpr size_t o_misc = o_bk + BK_BYTES;
+    static constexpr size_t o_tabs = o_misc + 512; // O (sigma + 1)
+    static constexpr size_t o_meta = o_tabs + al((size_t(SIGMA) + 4) * 4);
     static constexpr size_t o_bar = o_meta + al(STAGES * 16);
     static constexpr size_t SMEM = o_bar + al(2 * STAGES * 8);
     static_assert(SMEM <= 227 * 1024, "shared memory budget");
@@ -616,7 +589,18 @@ __device__ __forceinline__ uint32_t look_back(const unsigned long long *ring, ui
                 set_status(ST_TIMEOUT);
                 return excl;
             }
-            __nanosleep(32);
+            // wait for that tile's word alone: reloading the whole window
+            // loads the L2 with polls (round kernel at 2^28: 1.58 ms, so 1.53)
+            while (x >= 0) {
+                const unsigned long long w = ld_volatile64(ring + size_t(x & rmask) * SIGMA + c);
+                if (static_cast<uint32_t>(w >> 32) >= tagbase + uint32_t(x))
+                    break;
+                if (++spins > SPIN_LIMIT || ((spins & 1023u) == 0 && wait_failed())) {
+                    set_status(ST_TIMEOUT);
+                    return excl;
+                }
+                __nanosleep(64);
+            }
         }
     }
     return excl;
@@ -636,45 +620,28 @@ __device__ __forceinline__ uint32_t wait_pi(const uint32_t *p)
     return PI_NONE;
 }
 
-template <typename KT, bool HASV, int DB, int TILE, int NW, int NG, int STAGES, bool OOP>
-__global__ void __launch_bounds__(LbCfg<KT, HASV, DB, TILE, NW, NG, STAGES, OOP>::THREADS,
-                                   LbCfg<KT, HASV, DB, TILE, NW, NG, STAGES, OOP>::MINB)
-    k_lb_round(LbArgs<KT> a)
+template <typename KT, bool HASV, int TILE, bool OOP>
+__global__ void __launch_bounds__(LbCfg<KT, HASV, TILE, OOP>::THREADS, 1) k_lb_round11(LbArgs<KT> a)
 {
-    using C = LbCfg<KT, HASV, DB, TILE, NW, NG, STAGES, OOP>;
-    constexpr int SIGMA = C::SIGMA, NT = C::NT;
+    using C = LbCfg<KT, HASV, TILE, OOP>;
+    constexpr int SIGMA = C::SIGMA, NT = C::NT, NW = C::NW, STAGES = C::STAGES, DB = C::DB;
     extern __shared__ __align__(128) unsigned char sm[];
     if (!OOP && a.state[ST_SKIP])
         return; // the digit is constant: the round is the identity
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    // this warp's consumer group (the producer warp maps past the last one)
-    const int grp = warp / NW < NG ? warp / NW : 0;
-    unsigned char *gb = sm + C::o_group + size_t(grp) * C::GROUP;
-    uint16_t *hist = reinterpret_cast<uint16_t *>(gb + C::g_hist);
-    unsigned *ptab = reinterpret_cast<unsigned *>(gb + C::g_tab);
-    uint32_t *bk = reinterpret_cast<uint32_t *>(gb + C::g_bk);
+    uint16_t *hist = reinterpret_cast<uint16_t *>(sm + C::o_hist);
+    uint32_t *bk = reinterpret_cast<uint32_t *>(sm + C::o_bk);
     uint32_t *tcnt = bk, *bstart = bk + SIGMA, *gpos = bk + 2 * SIGMA;
     uint32_t *sO = reinterpret_cast<uint32_t *>(sm + C::o_tabs); // sigma + 1 entries
-    uint32_t *stab = sO + SIGMA + 1;
-    // bucket tables: shared memory (SMALL) or global
-    const uint32_t *ns0 = C::SMALL ? stab : a.tab + SIGMA + 1;
-    const uint32_t *ns1 = ns0 + SIGMA;
-    uint2 *qb = reinterpret_cast<uint2 *>(gb + C::g_qb);
-    uint4 *qb16 = reinterpret_cast<uint4 *>(gb + C::g_qb);
-    uint32_t *qlo = reinterpret_cast<uint32_t *>(gb + C::g_qb + C::QLO_OFF);
-    // list entries: the key block pointer tagged with its array (SMALL), or
-    // the block index
-    unsigned long long *listk = reinterpret_cast<unsigned long long *>(gb + C::g_lk);
-    uint32_t *listb = reinterpret_cast<uint32_t *>(gb + C::g_lk);
-    // byte distance from a key block to its value block, in T and in A
-    const long long dvT = reinterpret_cast<const char *>(a.Tv) - reinterpret_cast<const char *>(a.Tk);
-    const long long dvA = reinterpret_cast<const char *>(a.Av) - reinterpret_cast<const char *>(a.Ak);
+    const uint32_t *ns0 = a.tab + SIGMA + 1, *ns1 = ns0 + SIGMA;
+    uint2 *qb = reinterpret_cast<uint2 *>(sm + C::o_qb);
+    uint32_t *listb = reinterpret_cast<uint32_t *>(sm + C::o_lk); // block indices
     uint32_t *meta = reinterpret_cast<uint32_t *>(sm + C::o_meta);
     uint64_t *full = reinterpret_cast<uint64_t *>(sm + C::o_bar);
     uint64_t *empty = full + STAGES;
-    // the group's [1..3] a tile's list slots, blocks taken and blocks taken
-    // by earlier tiles, [8..] scan scratch
-    uint32_t *misc = reinterpret_cast<uint32_t *>(gb + C::g_misc);
+    // [1..3] a tile's list slots, blocks taken and blocks taken by earlier
+    // tiles, [8..] scan scratch
+    uint32_t *misc = reinterpret_cast<uint32_t *>(sm + C::o_misc);
 
     const uint32_t b = 1u << a.lb;
     const uint32_t mask = SIGMA - 1;
@@ -688,16 +655,6 @@ __global__ void __launch_bounds__(LbCfg<KT, HASV, DB, TILE, NW, NG, STAGES, OOP>
     }
     for (int c = tid; c <= SIGMA; c += C::THREADS)
         sO[c] = a.tab[c];
-    if constexpr (!OOP && C::SMALL) {
-        for (int c = tid; c < 2 * SIGMA; c += C::THREADS)
-            stab[c] = a.tab[SIGMA + 1 + c];
-    }
-    if constexpr (C::PTAB)
-        for (int g = 0; g < NG; ++g) {
-            unsigned *pt = reinterpret_cast<unsigned *>(sm + C::o_group + size_t(g) * C::GROUP + C::g_tab);
-            for (int i = tid; i < 2 * NW * SIGMA; i += C::THREADS)
-                pt[i] = 0u;
-        }
     __syncthreads();
 
     auto kaddr = [&](uint32_t blk) -> KT * {
@@ -707,7 +664,7 @@ __global__ void __launch_bounds__(LbCfg<KT, HASV, DB, TILE, NW, NG, STAGES, OOP>
         return blk < a.nT ? a.Tv + (size_t(blk) << a.lb) : a.Av + (size_t(blk - a.nT) << a.lb);
     };
 
-    if (warp == NG * NW) {
+    if (warp == NW) {
         // ================================================================ producer
         uint32_t k = 0;
         uint32_t wm = 0; // tiles below wm have finished their look-back
@@ -742,22 +699,11 @@ __global__ void __launch_bounds__(LbCfg<KT, HASV, DB, TILE, NW, NG, STAGES, OOP>
                 }
             }
             if (t >= a.ntiles) {
-                // every group stops at its next tile: NG end marks, each in
-                // the next stage in fill order
                 if (lane == 0) {
                     mt[0] = TILE_END;
                     mbar_arrive(&full[s]);
                 }
                 ++k;
-                bool ok = true;
-                for (int g = 1; g < NG && ok; ++g, ++k) {
-                    const int s2 = k % STAGES;
-                    ok = mbar_wait(&empty[s2], ((k / STAGES) & 1u) ^ 1u);
-                    if (ok && lane == 0) {
-                        meta[s2 * 4] = TILE_END;
-                        mbar_arrive(&full[s2]);
-                    }
-                }
                 break;
             }
             unsigned char *st = sm + C::o_stage + size_t(s) * C::STAGE;
@@ -867,14 +813,13 @@ __global__ void __launch_bounds__(LbCfg<KT, HASV, DB, TILE, NW, NG, STAGES, OOP>
     }
 
     // ==================================================================== consumers
-    // thread and warp index within the group
-    const int ctid = tid - grp * NT, cw = warp - grp * NW;
+    const int ctid = tid, cw = warp;
     uint32_t *tmp = misc + 8;
-    auto bar = [grp] { named_bar(1 + grp, NT); };
+    auto bar = [] { named_bar(1, NT); };
     const uint32_t nP = OOP ? 0u : a.state[ST_NS]; // free-list entries taken before the round
     const uint32_t M = uint32_t(TILE) >> a.lb;
 
-    for (uint32_t k = grp;; k += NG) { // fills grp, grp + NG, ...
+    for (uint32_t k = 0;; ++k) { // fill k
         const int s = k % STAGES;
         if (!mbar_wait(&full[s], (k / STAGES) & 1u))
             break;
@@ -926,34 +871,7 @@ __global__ void __launch_bounds__(LbCfg<KT, HASV, DB, TILE, NW, NG, STAGES, OOP>
         uint16_t *hw = hist + cw * C::HROW;
         for (int c = lane; c < SIGMA; c += 32)
             hw[c] = 0;
-        if constexpr (C::PTAB) {
-            // row by row: lanes with the same digit OR their bit into the
-            // digit's mask word, read back the mask and the warp's running
-            // count; the lowest of those lanes advances the count and clears
-            // the word.  Rows alternate between two mask tables, so the
-            // clearing of one row and the ORs of the next never meet (a
-            // table is all zero again two rows later)
-            unsigned *pt0 = ptab + cw * 2 * SIGMA;
-            __syncwarp();
-#pragma unroll
-            for (int it = 0; it < C::ITEMS; ++it) {
-                unsigned *pt = pt0 + (it & 1) * SIGMA;
-                const uint32_t d = dig(it);
-                const bool v = d < SIGMA;
-                if (v)
-                    atomicOr(&pt[d], 1u << lane);
-                __syncwarp();
-                const unsigned pm = v ? pt[d] : 0u;
-                const uint32_t base = v ? hw[d] : 0u;
-                set_rk(it, base + __popc(pm & lt));
-                __syncwarp();
-                if (v && (__ffs(pm) - 1) == lane) {
-                    hw[d] = static_cast<uint16_t>(base + __popc(pm));
-                    pt[d] = 0u;
-                }
-            }
-            __syncwarp();
-        } else {
+        {
             // a few rows at a time: their peer masks (independent ballots),
             // then row by row the lowest lane of each digit group reads and
             // advances the running count and passes the old count to its
@@ -1056,8 +974,7 @@ __global__ void __launch_bounds__(LbCfg<KT, HASV, DB, TILE, NW, NG, STAGES, OOP>
             }
         }
 
-        if constexpr (C::ALIAS)
-            bar(); // every warp has read its row before qb and the list overwrite it
+        bar(); // every warp has read its row before qb and the list overwrite it
 
         // ---- 4. global offset of each bucket's run (look-back); Radsort:
         // blocks touched, blocks taken here and by earlier tiles, list slots
@@ -1140,14 +1057,7 @@ __global__ void __launch_bounds__(LbCfg<KT, HASV, DB, TILE, NW, NG, STAGES, OOP>
                     continue;
                 const uint32_t g = gpos[c], cn = tcnt[c];
                 const uint32_t l0 = l0s[q], j0 = g >> a.lb;
-                if constexpr (C::QB16) {
-                    // the run's first block is filled in below; an element
-                    // past it reads its block from the list
-                    qb16[c] = make_uint4(g - bstart[c], 0u, 0u, 0u);
-                    qlo[c] = l0 - j0;
-                } else {
-                    qb[c] = make_uint2(g - bstart[c], l0 - j0);
-                }
+                qb[c] = make_uint2(g - bstart[c], l0 - j0);
                 if (!cn || g + cn > sO[c + 1] || g + cn < g)
                     continue; // (a corrupted run was reported in step 4)
                 const uint32_t touched = ((g + cn - 1) >> a.lb) - j0 + 1;
@@ -1186,27 +1096,7 @@ __global__ void __launch_bounds__(LbCfg<KT, HASV, DB, TILE, NW, NG, STAGES, OOP>
                         set_status(ST_INTERNAL);
                         phys = PI_NONE;
                     }
-                    if constexpr (C::SMALL) {
-                        // one word per entry: the key block pointer, bit 0 set
-                        // for a block of A (the value pointer follows from it)
-                        const unsigned long long w =
-                            phys == PI_NONE ? 0ull
-                                            : (reinterpret_cast<unsigned long long>(kaddr(phys)) |
-                                               (phys >= a.nT ? 1ull : 0ull));
-                        listk[l0 + (j - j0)] = w;
-                        if (j == j0 && w) {
-                            // the first block as a base for the run's
-                            // positions: key address of position p in it is
-                            // base + p elements (bit 1 marks it valid)
-                            const unsigned long long base =
-                                ((w & ~1ull) - (static_cast<unsigned long long>(j0) << a.lb) * sizeof(KT)) |
-                                (w & 1ull) | 2ull;
-                            qb16[c] = make_uint4(g - bstart[c], (j0 + 1) << a.lb, static_cast<uint32_t>(base),
-                                                 static_cast<uint32_t>(base >> 32));
-                        }
-                    } else {
-                        listb[l0 + (j - j0)] = phys;
-                    }
+                    listb[l0 + (j - j0)] = phys;
                 }
             }
             bar();
@@ -1230,36 +1120,6 @@ __global__ void __launch_bounds__(LbCfg<KT, HASV, DB, TILE, NW, NG, STAGES, OOP>
                         vv = tv[i];
                 }
                 const uint32_t dg = digit_of(kv, a.shift, mask);
-                if constexpr (C::QB16) {
-                    // Radsort, sigma <= 256: most runs lie in one block, whose
-                    // base address the run descriptor holds; the rest read
-                    // their block from the list
-                    const uint4 qd = qb16[dg];
-                    const uint32_t pos = i + qd.x;
-                    unsigned long long w;
-                    uint32_t idx;
-                    if (pos < qd.y) {
-                        w = (static_cast<unsigned long long>(qd.w) << 32) | qd.z;
-                        idx = pos;
-                    } else {
-                        const uint32_t l = (pos >> a.lb) + qlo[dg];
-                        w = l < TT ? listk[l] : 0ull;
-                        idx = pos & (b - 1);
-                    }
-                    if (w) {
-                        KT *pk = reinterpret_cast<KT *>(w & ~3ull) + idx;
-                        *pk = kv;
-                        if (HASV) {
-                            uint32_t *pv;
-                            if constexpr (sizeof(KT) == 4)
-                                pv = reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(pk) + ((w & 1ull) ? dvA : dvT));
-                            else
-                                pv = ((w & 1ull) ? a.Av + (pk - a.Ak) : a.Tv + (pk - a.Tk));
-                            *pv = vv;
-                        }
-                    }
-                    continue;
-                }
                 const uint2 qd = qb[dg];
                 const uint32_t pos = i + qd.x;
                 if constexpr (OOP) {
@@ -1270,27 +1130,11 @@ __global__ void __launch_bounds__(LbCfg<KT, HASV, DB, TILE, NW, NG, STAGES, OOP>
                     }
                 } else {
                     const uint32_t l = (pos >> a.lb) + qd.y, off = pos & (b - 1);
-                    if constexpr (C::SMALL) {
-                        const unsigned long long w = l < TT ? listk[l] : 0ull;
-                        if (w) {
-                            KT *pk = reinterpret_cast<KT *>(w & ~1ull);
-                            pk[off] = kv;
-                            if (HASV) {
-                                uint32_t *pv;
-                                if constexpr (sizeof(KT) == 4)
-                                    pv = reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(pk) + ((w & 1ull) ? dvA : dvT));
-                                else
-                                    pv = ((w & 1ull) ? a.Av + (pk - a.Ak) : a.Tv + (pk - a.Tk));
-                                pv[off] = vv;
-                            }
-                        }
-                    } else {
-                        const uint32_t blk = l < TT ? listb[l] : PI_NONE;
-                        if (blk != PI_NONE) {
-                            kaddr(blk)[off] = kv;
-                            if (HASV)
-                                vaddr(blk)[off] = vv;
-                        }
+                    const uint32_t blk = l < TT ? listb[l] : PI_NONE;
+                    if (blk != PI_NONE) {
+                        kaddr(blk)[off] = kv;
+                        if (HASV)
+                            vaddr(blk)[off] = vv;
                     }
                 }
             }
@@ -1304,70 +1148,785 @@ __global__ void __launch_bounds__(LbCfg<KT, HASV, DB, TILE, NW, NG, STAGES, OOP>
     }
 }
 
-// ---------------------------------------------------------------- launch helpers
-template <typename KT, bool HASV, int DB, int TILE, int NW, int NG, int STAGES, bool OOP>
-static int lb_ctas(size_t ntiles)
+// ---------------------------------------------------------------- round kernel, 8-bit digits
+// One CTA per SM: NW ranking warps, 8 look-back warps and a producer warp, on
+// tiles of TILE elements in two shared-memory stages.  What bounds it is
+// shared memory (the random-digit accesses of the ranking and the reorder,
+// each 3.4 wavefronts a row of 32 elements) and instruction issue, both near
+// 60% busy; DRAM is at 40% of its peak.  Hence
+//  * the ranking works on half-warps.  Each half-warp ranks its own run of
+//    TILE / (2 NW) elements, 16 a row, with one word per digit: the count so
+//    far in the high half, the lanes of this row in the low half.  A row is
+//    one atomicOr, one read and one write by the last lane of each digit
+//    group; a word per warp needs mask and count apart (two reads, two
+//    writes).  Ranking a tile of 10240: 5600 -> 3450 cycles.
+//  * the look-back and the block lists (5-6 L2 round trips, 4.6 us a tile) run
+//    on their own warps, one thread per bucket.  The ranking warps rank and
+//    count tile k before they store tile k - 1, so tile k's look-back has that
+//    store, the reorder of tile k and the ranking of tile k + 1 to complete
+//    in, and no one waits for it.
+//  * no barrier ends a tile: a warp that has stored and reordered its part
+//    ranks the next tile.
+// Measured (a round, uniform keys, ms; before: 16 ranking warps that did all
+// of it in turn, per-warp masks and counts): 2^28 u32 + u32 1.79 -> 1.46, u32
+// alone 1.48 -> 0.92; 2^27 u64 + u32 1.26 -> 1.06, u64 alone 0.88 -> 0.69;
+// 2^26 u32 + u32 Zipf 0.83 -> 0.62.  The look-back walks over 64-bit words, 8
+// in flight; smaller words with flags, or groups of tiles with a prefix each,
+// read less but need two dependent round trips where the walk needs one, and
+// were slower (1.9 to 3 ms at 2^28 u32 + u32).
+template <typename KT, bool HASV, int TILE, int NW, bool OOP> struct Lb8Cfg {
+    static constexpr int SIGMA = 256, STAGES = 2;
+    static constexpr int NT = NW * 32;             // ranking threads
+    static constexpr int NA = SIGMA;               // look-back threads, one per bucket
+    static constexpr int THREADS = NT + NA + 128;  // + the producer's warpgroup (one warp works)
+    static constexpr int SROWS = 2 * NW;           // half-warps
+    static constexpr int R = TILE / SROWS;         // elements ranked per half-warp
+    static constexpr int ITEMS = R / 16;           // elements per ranking thread
+    static_assert(TILE % (NW * 64) == 0 && R % 16 == 0 && ITEMS % 2 == 0, "whole rows, an even number");
+    static constexpr int PARTS = NT / SIGMA;       // threads per bucket in the column pass
+    static constexpr int RPT = SROWS / PARTS;      // rows each of them sums
+    static_assert(PARTS * SIGMA == NT && (PARTS == 1 || PARTS == 2), "one or two threads per bucket");
+    static constexpr int MAXM = TILE / 64;         // blocks per tile (b >= 64)
+    static constexpr bool PAIR = HASV && sizeof(KT) == 4;
+    // touched blocks per tile: at most TILE/b + 2 per bucket with elements
+    static constexpr int LIST = MAXM + 2 * SIGMA + 2;
+    static constexpr size_t al(size_t x) { return (x + 127) & ~size_t(127); }
+    // 16 bytes of slack per array: the lead of a misaligned source (out of
+    // place).  The values start 64 bytes past a multiple of 128, so that one
+    // half-warp reading keys and the other values meet in no bank
+    static constexpr size_t KBYTES = al(size_t(TILE) * sizeof(KT) + 16 + 64) - 64;
+    static constexpr size_t STAGE = al(KBYTES + (HASV ? size_t(TILE) * 4 + 16 : 0));
+    static constexpr size_t o_tab = STAGES * STAGE;                  // SROWS x SIGMA words
+    // what the look-back warps read or write of a tile while the ranking
+    // warps work on the next one is there twice (even and odd tiles)
+    static constexpr size_t o_part = o_tab + size_t(SROWS) * SIGMA * 4; // 2 x PARTS x SIGMA
+    static constexpr size_t o_bst = o_part + 2 * size_t(PARTS) * SIGMA * 4; // 2 x SIGMA
+    static constexpr size_t o_tot = o_bst + 2 * size_t(SIGMA) * 4;   // 8 x 16 bytes, then 8 words
+    static constexpr size_t QD = size_t(SIGMA) * 16;                 // run descriptors
+    static constexpr size_t LISTB = OOP ? 0 : al(size_t(LIST) * 8);
+    static constexpr size_t o_qd = o_tot + 256;                      // 2 x QD
+    static constexpr size_t o_qlo = o_qd + 2 * QD;                   // 2 x SIGMA
+    static constexpr size_t o_list = o_qlo + 2 * size_t(SIGMA) * 4;  // 2 x LISTB
+    static constexpr size_t o_tabs = o_list + 2 * LISTB;             // O, ns0, ns1
+    static constexpr size_t o_misc = o_tabs + al((3 * size_t(SIGMA) + 4) * 4);
+    static constexpr size_t o_meta = o_misc + 64;
+    static constexpr size_t o_bar = o_meta + STAGES * 16;
+    static constexpr size_t SMEM = al(o_bar + STAGES * 8);
+    static_assert(SMEM <= 227 * 1024, "shared memory budget");
+    static constexpr int MINB = NW <= 8 && 2 * (SMEM + 1024) <= 228 * 1024 ? 2 : 1; // CTAs per SM
+    // registers a thread: a CTA is launched with 72 (896 threads), 48 (two of
+    // 640) or 96 (one of 640) and deals them out anew
+    static constexpr int MAIN_REGS = NW == 16 ? 88 : MINB == 2 ? 64 : 120;
+    static constexpr int AUX_REGS = NW == 16 ? 56 : MINB == 2 ? 40 : 72;
+    static constexpr int PROD_REGS = NW == 16 ? 40 : MINB == 2 ? 32 : 72;
+};
+
+// Moves registers between the warps of a CTA (all four warps of a warpgroup
+// execute it; the shares add up to what the CTA was launched with).
+template <int N> __device__ __forceinline__ void reg_dec()
 {
-    using C = LbCfg<KT, HASV, DB, TILE, NW, NG, STAGES, OOP>;
-    static DeviceOnce attr; // per template instance
-    if (attr.run([] {
-            return cudaFuncSetAttribute(k_lb_round<KT, HASV, DB, TILE, NW, NG, STAGES, OOP>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, int(C::SMEM));
-        }) != cudaSuccess)
-        return -1;
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lb_round<KT, HASV, DB, TILE, NW, NG, STAGES, OOP>,
-                                                  C::THREADS, C::SMEM);
-    if (per_sm < 1)
-        per_sm = 1;
-    size_t grid = size_t(num_sms()) * per_sm;
-    if (grid > ntiles)
-        grid = ntiles;
-    return grid < 1 ? 1 : static_cast<int>(grid);
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N));
+}
+template <int N> __device__ __forceinline__ void reg_inc()
+{
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
 }
 
-// Calls f.template operator()<KT, HASV, DB, TILE, NW, NG, STAGES>() for the configuration.
+// named barriers of k_lb_round8
+enum { LB8_MAIN = 1, LB8_AUX = 2, LB8_CNT = 3, LB8_SCAN = 4, LB8_LIST = 5, LB8_FREE = 6 };
+
+template <typename KT, bool HASV, int TILE, int NW, bool OOP>
+__global__ void __launch_bounds__(Lb8Cfg<KT, HASV, TILE, NW, OOP>::THREADS, Lb8Cfg<KT, HASV, TILE, NW, OOP>::MINB)
+    k_lb_round8(LbArgs<KT> a)
+{
+    using C = Lb8Cfg<KT, HASV, TILE, NW, OOP>;
+    constexpr int SIGMA = C::SIGMA, NT = C::NT, ITEMS = C::ITEMS;
+    extern __shared__ __align__(128) unsigned char sm[];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (!OOP && a.state[ST_SKIP])
+        return; // the digit is constant: the round is the identity
+    uint32_t *tab = reinterpret_cast<uint32_t *>(sm + C::o_tab);
+    uint32_t *part2 = reinterpret_cast<uint32_t *>(sm + C::o_part);
+    uint32_t *bst2 = reinterpret_cast<uint32_t *>(sm + C::o_bst);
+    uint4 *tot4 = reinterpret_cast<uint4 *>(sm + C::o_tot);
+    uint32_t *wsum = reinterpret_cast<uint32_t *>(sm + C::o_tot + 128);
+    uint32_t *sO = reinterpret_cast<uint32_t *>(sm + C::o_tabs); // sigma + 1 entries
+    uint32_t *misc = reinterpret_cast<uint32_t *>(sm + C::o_misc); // [0..1]: list entries of the tile
+    uint32_t *meta = reinterpret_cast<uint32_t *>(sm + C::o_meta);
+    uint64_t *full = reinterpret_cast<uint64_t *>(sm + C::o_bar);
+    const uint32_t b = 1u << a.lb;
+
+    if (tid == 0) {
+        for (int s = 0; s < C::STAGES; ++s) {
+            mbar_init(&full[s], 1);
+            meta[s * 4] = TILE_END;
+        }
+        misc[0] = misc[1] = 0;
+        fence_mbar_init();
+    }
+    for (int c = tid; c < (OOP ? SIGMA + 1 : 3 * SIGMA + 1); c += C::THREADS)
+        sO[c] = a.tab[c];
+    for (int i = tid; i < C::SROWS * SIGMA; i += C::THREADS)
+        tab[i] = 0u;
+    __syncthreads();
+
+    if (warp >= NW + SIGMA / 32) {
+        // ============================================================ producer
+        reg_dec<C::PROD_REGS>();
+        if (warp > NW + SIGMA / 32)
+            return;
+        auto kaddr = [&](uint32_t blk) -> KT * {
+            return blk < a.nT ? a.Tk + (size_t(blk) << a.lb) : a.Ak + (size_t(blk - a.nT) << a.lb);
+        };
+        auto vaddr = [&](uint32_t blk) -> uint32_t * {
+            return blk < a.nT ? a.Tv + (size_t(blk) << a.lb) : a.Av + (size_t(blk - a.nT) << a.lb);
+        };
+        // fill fk (this CTA's tile fk) goes to stage fk % 2
+        uint32_t ft = 0, fphys = 0, wm = 0; // drawn ticket; its block `lane`; tiles below wm have looked back
+        auto draw = [&]() {
+            uint32_t t = 0;
+            if (lane == 0)
+                t = atomicAdd(a.ticket, 1u);
+            ft = __shfl_sync(0xffffffffu, t, 0);
+            if constexpr (!OOP) {
+                if (ft < a.ntiles) {
+                    const uint32_t cnt = min(uint32_t(TILE), a.n - ft * uint32_t(TILE));
+                    const uint32_t nb = (cnt + b - 1) >> a.lb;
+                    fphys = uint32_t(lane) < nb ? a.pi[a.H + ft * (uint32_t(TILE) >> a.lb) + lane] : 0u;
+                }
+            }
+        };
+        // the ring slot of tile ft held tile ft - R: wait until every tile up
+        // to ft - R + 1 has finished its look-back
+        auto ring_free = [&]() {
+            if (ft >= a.ntiles || ft <= a.rmask)
+                return;
+            const uint32_t need = ft - a.rmask + 1; // tiles below it
+            unsigned spins = 0;
+            while (wm < need) {
+                const uint32_t z = wm + lane;
+                const bool ok = z >= need || ld_volatile(a.done + (z & a.rmask)) >= a.tagbase + z;
+                const unsigned bal = __ballot_sync(0xffffffffu, ok);
+                const uint32_t adv = bal == 0xffffffffu ? 32u : uint32_t(__ffs(~bal) - 1);
+                wm = min(need, wm + adv);
+                if (wm < need && adv < 32u) {
+                    if (++spins > SPIN_LIMIT || ((spins & 1023u) == 0 && wait_failed())) {
+                        set_status(ST_TIMEOUT);
+                        return;
+                    }
+                    __nanosleep(64);
+                }
+            }
+        };
+        auto issue = [&](int fk) {
+            const int s = fk % C::STAGES;
+            uint32_t *mt = meta + s * 4;
+            if (ft >= a.ntiles) { // the end mark
+                if (lane == 0) {
+                    mt[0] = TILE_END;
+                    mbar_arrive(&full[s]);
+                }
+                return;
+            }
+            unsigned char *st = sm + size_t(s) * C::STAGE;
+            KT *stk = reinterpret_cast<KT *>(st);
+            uint32_t *stv = reinterpret_cast<uint32_t *>(st + C::KBYTES);
+            const uint32_t e0 = ft * uint32_t(TILE);
+            const uint32_t cnt = min(uint32_t(TILE), a.n - e0);
+            uint32_t leadk = 0, leadv = 0;
+            if constexpr (OOP) {
+                // the 16-byte-aligned middle by bulk copies, the ragged ends
+                // (under 16 bytes each) by plain loads
+                const uintptr_t ka = reinterpret_cast<uintptr_t>(a.ik + e0);
+                const uintptr_t kz = ka + uintptr_t(cnt) * sizeof(KT);
+                const uintptr_t ka16 = (ka + 15) & ~uintptr_t(15), kz16 = kz & ~uintptr_t(15);
+                leadk = static_cast<uint32_t>((ka & 15) / sizeof(KT));
+                const bool kmid = ka16 < kz16;
+                const uint32_t khead = kmid ? static_cast<uint32_t>((ka16 - ka) / sizeof(KT)) : cnt;
+                const uint32_t ktail = kmid ? static_cast<uint32_t>((kz16 - ka) / sizeof(KT)) : cnt;
+                uint32_t bytes = kmid ? static_cast<uint32_t>(kz16 - ka16) : 0u;
+                uintptr_t va16 = 0, vz16 = 0;
+                uint32_t vhead = 0, vtail = 0;
+                bool vmid = false;
+                if (HASV) {
+                    const uintptr_t va = reinterpret_cast<uintptr_t>(a.iv + e0);
+                    const uintptr_t vz = va + uintptr_t(cnt) * 4;
+                    va16 = (va + 15) & ~uintptr_t(15);
+                    vz16 = vz & ~uintptr_t(15);
+                    leadv = static_cast<uint32_t>((va & 15) / 4);
+                    vmid = va16 < vz16;
+                    vhead = vmid ? static_cast<uint32_t>((va16 - va) / 4) : cnt;
+                    vtail = vmid ? static_cast<uint32_t>((vz16 - va) / 4) : cnt;
+                    bytes += vmid ? static_cast<uint32_t>(vz16 - va16) : 0u;
+                }
+                if (lane == 0 && bytes)
+                    asm volatile("mbarrier.expect_tx.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&full[s])),
+                                 "r"(bytes)
+                                 : "memory");
+                __syncwarp();
+                if (lane == 0 && kmid)
+                    bulk_g2s(stk + leadk + khead, reinterpret_cast<const void *>(ka16),
+                             static_cast<uint32_t>(kz16 - ka16), &full[s]);
+                if (HASV && lane == 1 && vmid)
+                    bulk_g2s(stv + leadv + vhead, reinterpret_cast<const void *>(va16),
+                             static_cast<uint32_t>(vz16 - va16), &full[s]);
+                for (uint32_t e = lane; e < khead; e += 32)
+                    stk[leadk + e] = a.ik[e0 + e];
+                for (uint32_t e = ktail + lane; e < cnt; e += 32)
+                    stk[leadk + e] = a.ik[e0 + e];
+                if (HASV) {
+                    for (uint32_t e = lane; e < vhead; e += 32)
+                        stv[leadv + e] = a.iv[e0 + e];
+                    for (uint32_t e = vtail + lane; e < cnt; e += 32)
+                        stv[leadv + e] = a.iv[e0 + e];
+                }
+            } else {
+                // blocks ft*M .. of the logical data: block i at stage offset
+                // i*b (a block index outside the block store is reported and
+                // skipped)
+                const uint32_t nb = (cnt + b - 1) >> a.lb;
+                const uint32_t i0 = a.H + ft * (uint32_t(TILE) >> a.lb);
+                uint32_t tot = 0;
+                for (uint32_t base = 0; base < nb; base += 32) {
+                    const uint32_t i = base + lane;
+                    uint32_t bytes = 0;
+                    if (i < nb && (base ? a.pi[i0 + i] : fphys) < a.npi) {
+                        const uint32_t len = min(b, cnt - i * b);
+                        bytes = ((len * uint32_t(sizeof(KT)) + 15u) & ~15u) + (HASV ? ((len * 4u + 15u) & ~15u) : 0u);
+                    }
+                    tot += warp_sum(bytes);
+                }
+                if (lane == 0 && tot)
+                    asm volatile("mbarrier.expect_tx.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&full[s])),
+                                 "r"(tot)
+                                 : "memory");
+                __syncwarp();
+                for (uint32_t i = lane; i < nb; i += 32) {
+                    const uint32_t len = min(b, cnt - i * b);
+                    const uint32_t phys = i < 32 ? fphys : a.pi[i0 + i];
+                    if (phys >= a.npi) {
+                        set_status(ST_INTERNAL);
+                        continue;
+                    }
+                    bulk_g2s(stk + size_t(i) * b, kaddr(phys), (len * uint32_t(sizeof(KT)) + 15u) & ~15u, &full[s]);
+                    if (HASV)
+                        bulk_g2s(stv + size_t(i) * b, vaddr(phys), (len * 4u + 15u) & ~15u, &full[s]);
+                }
+            }
+            __syncwarp();
+            if (lane == 0) {
+                mt[0] = ft;
+                mt[1] = cnt;
+                mt[2] = leadk;
+                mt[3] = leadv;
+            }
+            __syncwarp();
+            if (lane == 0)
+                mbar_arrive(&full[s]); // release: the plain stores above are visible
+        };
+        // The ticket of fill k + 1 is drawn when tile k is counted, not before:
+        // every look-back waits for the tiles drawn earlier, and a CTA that
+        // drew two tiles in a row at its start held up all between them
+        draw();
+        ring_free();
+        issue(0);
+        int k = 0; // fill k is issued
+        while (ft < a.ntiles) {
+            named_bar(LB8_CNT, C::NT + C::NA + 32);
+            draw();
+            ring_free();
+            if (k >= 1)
+                named_bar(LB8_FREE, NT + 32); // tile k - 1 is stored: the stage of fill k + 1 is free
+            issue(++k);
+        }
+        named_bar(LB8_CNT, C::NT + C::NA + 32); // (the end mark's)
+        // every issued copy lands before this CTA exits (only after a wait
+        // that ran out can one still be in flight)
+        if (lane == 0)
+            for (int f = k > 0 ? k - 1 : 0; f <= k; ++f)
+                mbar_wait(&full[f % C::STAGES], (f / C::STAGES) & 1u);
+        return;
+    }
+
+    if (warp >= NW) {
+        // ============================================================ look-back warps
+        reg_dec<C::AUX_REGS>();
+        const int c = tid - NT, aw = warp - NW; // this thread's bucket, its warp among the 8
+        const uint32_t *ns0 = sO + SIGMA + 1, *ns1 = ns0 + SIGMA;
+        const uint32_t Oc = sO[c], Oe = sO[c + 1];
+        const uint32_t n0 = OOP ? 0u : ns0[c], n1 = OOP ? 0u : ns1[c];
+        const uint32_t nP = OOP ? 0u : a.state[ST_NS]; // free-list entries taken before the round
+        auto kaddr = [&](uint32_t blk) -> KT * {
+            return blk < a.nT ? a.Tk + (size_t(blk) << a.lb) : a.Ak + (size_t(blk - a.nT) << a.lb);
+        };
+
+        for (uint32_t k = 0;; ++k) { // fill k
+            named_bar(LB8_CNT, C::NT + C::NA + 32); // the tile's counts per bucket are in part
+            const uint32_t *part = part2 + (k & 1) * C::PARTS * SIGMA, *bst = bst2 + (k & 1) * SIGMA;
+            uint4 *qd16 = reinterpret_cast<uint4 *>(sm + C::o_qd + (k & 1) * C::QD);        // Radsort
+            uint32_t *qoff = reinterpret_cast<uint32_t *>(sm + C::o_qd + (k & 1) * C::QD);  // out of place
+            uint32_t *qlo = reinterpret_cast<uint32_t *>(sm + C::o_qlo) + (k & 1) * SIGMA;
+            unsigned long long *list = reinterpret_cast<unsigned long long *>(sm + C::o_list + (k & 1) * C::LISTB);
+            const uint32_t t = meta[(k % C::STAGES) * 4];
+            if (t == TILE_END)
+                break;
+            const uint32_t cnt = meta[(k % C::STAGES) * 4 + 1];
+            // elements past the tile's end were ranked as digit 255
+            uint32_t cn = part[c] + (C::PARTS == 2 ? part[SIGMA + c] : 0u);
+            if (c == SIGMA - 1)
+                cn -= uint32_t(TILE) - cnt;
+            // ---- the count published, the bucket's prefix over the tiles before
+            unsigned long long *slot = a.ring + size_t(t & a.rmask) * SIGMA + c;
+            st_volatile64(slot, lbw(a.tagbase + t, t == 0 ? (LB_INCL | cn) : cn));
+            uint32_t excl = 0;
+            if (t > 0) {
+                excl = look_back<SIGMA>(a.ring, a.rmask, a.tagbase, t, c);
+                st_volatile64(slot, lbw(a.tagbase + t, LB_INCL | (excl + cn)));
+            }
+            __syncwarp();
+            const uint32_t g = Oc + excl;
+            __syncwarp();
+            if constexpr (OOP) {
+                named_bar(LB8_AUX, C::NA);
+                if (c == 0) // this tile reads no more look-back words
+                    st_volatile(a.done + (t & a.rmask), a.tagbase + t);
+                named_bar(LB8_SCAN, C::NT + C::NA); // bucket starts in the tile
+                qoff[c] = g - bst[c];
+            } else {
+                // the run lies inside the bucket's output range unless the
+                // look-back words were corrupted: then it is reported and its
+                // blocks are left alone
+                if (g + cn > Oe || g + cn < g) {
+                    set_status(ST_INTERNAL);
+                    cn = 0;
+                }
+                // ---- blocks touched, blocks taken here and by earlier tiles
+                const uint32_t e = g + cn, j0 = g >> a.lb;
+                const uint32_t touched = cn ? ((e - 1) >> a.lb) - j0 + 1 : 0u;
+                const uint32_t cs = (g + b - 1) >> a.lb, ce = (e + b - 1) >> a.lb;
+                // block j in [n0 + L, n1) is taken by the writer of the first
+                // position of block j - L: by earlier tiles for j - L < cs,
+                // here for cs <= j - L < ce
+                const uint32_t mb = min(cs + GRID_AHEAD, n1), e0 = n0 + GRID_AHEAD;
+                const uint32_t before = mb > e0 ? mb - e0 : 0u;
+                const uint32_t first = max(cs, n0) + GRID_AHEAD, last = min(ce + GRID_AHEAD, n1);
+                const uint32_t take = last > first ? last - first : 0u;
+                // the map entry of the first block touched (taken before
+                // this tile, if it touches any)
+                const uint32_t pf = cn ? ld_volatile(a.pin + a.H + j0) : PI_NONE;
+                // (and of the second, where it is not taken here)
+                const uint32_t pf2 = touched > 1 && j0 + 1 < first ? ld_volatile(a.pin + a.H + j0 + 1) : PI_NONE;
+                const uint32_t it_ = warp_incl_scan(touched), ik = warp_incl_scan(take), sb = warp_sum(before);
+                if (lane == 31)
+                    tot4[aw] = make_uint4(it_, ik, sb, 0u);
+                named_bar(LB8_AUX, C::NA);
+                if (c == 0) // this tile reads no more look-back words
+                    st_volatile(a.done + (t & a.rmask), a.tagbase + t);
+                uint32_t l0 = it_ - touched, ko = ik - take, TT = 0, fbase = nP;
+#pragma unroll
+                for (int w = 0; w < SIGMA / 32; ++w) {
+                    const uint4 x = tot4[w];
+                    if (w < aw) {
+                        l0 += x.x;
+                        ko += x.y;
+                    }
+                    TT += x.x;
+                    fbase += x.z;
+                }
+                // ---- the physical block of every block this tile touches,
+                // and the blocks it takes beyond those.  Those go into the map
+                // before this thread waits for any other's: a bucket that
+                // fills tile after tile (skewed keys) has each tile continue
+                // blocks that the tile just before took, and taking after the
+                // wait would chain every tile to its predecessor (1-2 us a
+                // tile).  Measured (2^26 keys + index, a sort): Zipf keys 57.8
+                // -> 3.7 ms, float32 N(0,1) keys (top digit skewed) 15.8 ->
+                // 3.0, uniform keys unchanged
+                // free-list entries consumed so far (Lemma 1), within the list
+                const uint32_t fcap = min(a.H + (t + 1) * (uint32_t(TILE) >> a.lb), a.npi);
+                const uint32_t fi0 = fbase + ko - first; // block j's free-list index - j (mod 2^32)
+                for (uint32_t j = first; j < last; ++j) {
+                    const uint32_t idx = fi0 + j;
+                    if (idx < fcap)
+                        a.pin[a.H + j] = __ldg(a.pi + idx);
+                    else
+                        set_status(ST_INTERNAL); // Lemma 1 would be violated
+                }
+                __syncwarp();
+                named_bar(LB8_SCAN, C::NT + C::NA); // bucket starts in the tile
+                // the run's first block is filled in below; an element past
+                // it reads its block from the list
+                uint4 qd = make_uint4(g - bst[c], 0u, 0u, 0u);
+                for (uint32_t i = 0; i < touched; ++i) {
+                    const uint32_t j = j0 + i;
+                    uint32_t phys;
+                    if (j >= first && j < last) { // taken here
+                        const uint32_t idx = fi0 + j;
+                        phys = idx < fcap ? __ldg(a.pi + idx) : PI_NONE;
+                    } else { // taken before the round or by an earlier tile
+                        phys = i == 0 ? pf : i == 1 ? pf2 : PI_NONE;
+                        if (phys == PI_NONE)
+                            phys = wait_pi(a.pin + a.H + j);
+                    }
+                    if (phys != PI_NONE && phys >= a.npi) {
+                        set_status(ST_INTERNAL);
+                        phys = PI_NONE;
+                    }
+                    // one word per entry: the key block pointer, bit 0 set
+                    // for a block of A (the value pointer follows from it)
+                    const unsigned long long w =
+                        phys == PI_NONE ? 0ull
+                                        : (reinterpret_cast<unsigned long long>(kaddr(phys)) |
+                                           (phys >= a.nT ? 1ull : 0ull));
+                    list[l0 + i] = w;
+                    if (i == 0 && w) {
+                        // the first block as a base for the run's positions:
+                        // the key address of position p in it is base + p
+                        // elements (bit 1 marks it valid)
+                        const unsigned long long base =
+                            ((w & ~1ull) - (static_cast<unsigned long long>(j0) << a.lb) * sizeof(KT)) | (w & 1ull) |
+                            2ull;
+                        qd.y = (j0 + 1) << a.lb;
+                        qd.z = static_cast<uint32_t>(base);
+                        qd.w = static_cast<uint32_t>(base >> 32);
+                    }
+                }
+                qd16[c] = qd;
+                qlo[c] = l0 - j0;
+                if (c == 0)
+                    misc[k & 1] = TT;
+            }
+            __syncwarp();
+            bar_arrive(LB8_LIST, C::NT + C::NA);
+        }
+        return;
+    }
+
+    // ================================================================ ranking warps
+    reg_inc<C::MAIN_REGS>();
+    const int h = lane >> 4, l16 = lane & 15;
+    const uint32_t ltm = (1u << l16) - 1u, gtm = 0xFFFFu & ~((2u << l16) - 1u);
+    uint32_t *row = tab + (2 * warp + h) * SIGMA; // this half-warp's words
+    const uint32_t eh = uint32_t((2 * warp + h) * C::R + l16); // its first element in the tile
+    auto dig = [&](KT key) -> uint32_t { return static_cast<uint32_t>(key >> a.shift) & 255u; };
+
+    // Tile k is ranked and counted before tile k - 1 is stored, so that a
+    // tile's look-back and block lists have the store before it, its own
+    // reorder and the next tile's ranking to complete in.
+    uint32_t pcnt = 0; // elements of tile k - 1
+    for (uint32_t k = 0;; ++k) { // fill k
+        const int s = k % C::STAGES;
+        // (a wait that runs out is reported; the tile is then worked through
+        // with what is there, so that every barrier is met)
+        (void)mbar_wait(&full[s], (k / C::STAGES) & 1u);
+        __syncwarp();
+        const uint32_t *mt = meta + s * 4;
+        const bool end = mt[0] == TILE_END;
+        const uint32_t cnt = mt[1], leadk = mt[2], leadv = mt[3];
+        unsigned char *st = sm + size_t(s) * C::STAGE;
+        KT *tk = reinterpret_cast<KT *>(st);
+        uint32_t *tv = reinterpret_cast<uint32_t *>(st + C::KBYTES);
+
+        KT key[ITEMS];
+        uint32_t val[HASV ? ITEMS : 1];
+        uint32_t rk[ITEMS / 2]; // ranks within the half-warp, two 16-bit ones each
+        if (!end) {
+            // ---- 1. this thread's elements into registers
+            if constexpr (C::PAIR) {
+                // one half-warp reads keys while the other reads values: the two
+                // halves' runs start in the same bank
+                const uint32_t *p0 = (h ? tv + leadv : tk + leadk) + eh, *p1 = (h ? tk + leadk : tv + leadv) + eh;
+#pragma unroll
+                for (int it = 0; it < ITEMS; ++it) {
+                    const uint32_t x = p0[it * 16], y = p1[it * 16];
+                    key[it] = h ? y : x;
+                    val[it] = h ? x : y;
+                }
+            } else {
+                // (4-byte words: the second half-warp reads the rows of a pair in
+                // the other order)
+#pragma unroll
+                for (int it = 0; it < ITEMS; it += 2) {
+                    const KT *pk = tk + leadk + eh + it * 16;
+                    if constexpr (sizeof(KT) == 4) {
+                        const KT x = pk[h * 16], y = pk[16 - h * 16];
+                        key[it] = h ? y : x;
+                        key[it + 1] = h ? x : y;
+                    } else {
+                        key[it] = pk[0];
+                        key[it + 1] = pk[16];
+                    }
+                    if constexpr (HASV) {
+                        const uint32_t *pv = tv + leadv + eh + it * 16;
+                        const uint32_t x = pv[h * 16], y = pv[16 - h * 16];
+                        val[it] = h ? y : x;
+                        val[it + 1] = h ? x : y;
+                    }
+                }
+            }
+            if (cnt < uint32_t(TILE)) {
+                // elements past the end rank as the last ones of digit 255
+#pragma unroll
+                for (int it = 0; it < ITEMS; ++it)
+                    if (eh + it * 16 >= cnt)
+                        key[it] = ~KT(0);
+            }
+            // ---- stable rank within the half-warp: lanes with the same digit OR
+            // their bit into the digit's word and read it back; the last of them
+            // writes the new count (its rank + 1) with the lane bits cleared
+#pragma unroll
+            for (int it = 0; it < ITEMS; ++it) {
+                uint32_t *w = row + dig(key[it]);
+                atomicOr(w, 1u << l16);
+                __syncwarp();
+                const uint32_t v = *reinterpret_cast<volatile uint32_t *>(w);
+                const uint32_t r = (v >> 16) + __popc(v & ltm);
+                __syncwarp();
+                if (!(v & gtm))
+                    *reinterpret_cast<volatile uint32_t *>(w) = (r + 1u) << 16;
+                __syncwarp();
+                if (it & 1)
+                    rk[it >> 1] |= r << 16;
+                else
+                    rk[it >> 1] = r;
+            }
+            named_bar(LB8_MAIN, NT);
+
+            // ---- 2. tile counts per bucket, for the look-back warps, and their
+            // exclusive scan (bucket starts in the reordered tile); then each
+            // half-warp's start per bucket: the ranks are relative to it
+            {
+                const int c = tid & (SIGMA - 1), p = tid / SIGMA;
+                uint32_t *col = tab + p * C::RPT * SIGMA + c;
+                uint32_t *part = part2 + (k & 1) * C::PARTS * SIGMA, *bst = bst2 + (k & 1) * SIGMA;
+                uint32_t hc[C::RPT / 2], sum = 0;
+#pragma unroll
+                for (int r = 0; r < C::RPT; r += 2) {
+                    const uint32_t x = col[r * SIGMA] >> 16, y = col[(r + 1) * SIGMA] & 0xFFFF0000u;
+                    hc[r >> 1] = x | y;
+                    sum += x + (y >> 16);
+                }
+                part[p * SIGMA + c] = sum;
+                bar_arrive(LB8_CNT, C::NT + C::NA + 32);
+                uint32_t tot = sum, below = 0;
+                if constexpr (C::PARTS == 2) {
+                    named_bar(LB8_MAIN, NT);
+                    const uint32_t o = part[(p ^ 1) * SIGMA + c];
+                    tot += o;
+                    below = p ? o : 0u;
+                }
+                const uint32_t inc = warp_incl_scan(tot);
+                if (lane == 31 && p == 0)
+                    wsum[warp] = inc;
+                named_bar(LB8_MAIN, NT);
+                uint32_t base = inc - tot;
+#pragma unroll
+                for (int w = 0; w < SIGMA / 32 - 1; ++w)
+                    base += w < (warp & 7) ? wsum[w] : 0u;
+                if (p == 0)
+                    bst[c] = base;
+                uint32_t run = base + below;
+#pragma unroll
+                for (int r = 0; r < C::RPT; ++r) {
+                    col[r * SIGMA] = run;
+                    run += (r & 1) ? hc[r >> 1] >> 16 : hc[r >> 1] & 0xFFFFu;
+                }
+            }
+        } else {
+            bar_arrive(LB8_CNT, C::NT + C::NA + 32);
+        }
+        if (k == 0)
+            named_bar(LB8_MAIN, NT);
+        else
+            named_bar(LB8_LIST, C::NT + C::NA); // tile k - 1 is reordered, its run descriptors are there
+        if (!end)
+            bar_arrive(LB8_SCAN, C::NT + C::NA);
+
+        // ---- 3. store tile k - 1, every bucket run, U elements a thread at a time
+        if (k > 0) {
+            unsigned char *pst = sm + size_t(s ^ 1) * C::STAGE;
+            const KT *pk = reinterpret_cast<const KT *>(pst);
+            const uint32_t *pv = reinterpret_cast<const uint32_t *>(pst + C::KBYTES);
+            const uint2 *pp = reinterpret_cast<const uint2 *>(pst);
+            const unsigned char *qdb = sm + C::o_qd + ((k - 1) & 1) * C::QD;
+            const uint4 *qd16 = reinterpret_cast<const uint4 *>(qdb);        // Radsort
+            const uint32_t *qoff = reinterpret_cast<const uint32_t *>(qdb);  // out of place
+            const uint32_t *qlo = reinterpret_cast<const uint32_t *>(sm + C::o_qlo) + ((k - 1) & 1) * SIGMA;
+            const unsigned long long *list =
+                reinterpret_cast<const unsigned long long *>(sm + C::o_list + ((k - 1) & 1) * C::LISTB);
+            constexpr int SI = TILE / NT, U = SI % 5 == 0 ? 5 : 4;
+            static_assert(SI % U == 0, "whole batches");
+            const uint32_t TT = OOP ? 0u : misc[(k - 1) & 1];
+            // byte distance from a key block to its value block, in T and in A
+            const long long dvT = reinterpret_cast<const char *>(a.Tv) - reinterpret_cast<const char *>(a.Tk);
+            const long long dvA = reinterpret_cast<const char *>(a.Av) - reinterpret_cast<const char *>(a.Ak);
+#pragma unroll 1
+            for (int k0 = 0; k0 < SI; k0 += U) {
+                KT kv[U];
+                uint32_t vv[U], idx[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const uint32_t i = tid + (k0 + u) * NT;
+                    if constexpr (C::PAIR) {
+                        const uint2 pr = pp[i];
+                        kv[u] = pr.x;
+                        vv[u] = pr.y;
+                    } else {
+                        kv[u] = pk[i];
+                        vv[u] = HASV ? pv[i] : 0u;
+                    }
+                }
+                if constexpr (OOP) {
+#pragma unroll
+                    for (int u = 0; u < U; ++u)
+                        idx[u] = tid + (k0 + u) * NT + qoff[dig(kv[u])];
+#pragma unroll
+                    for (int u = 0; u < U; ++u)
+                        if (tid + (k0 + u) * NT < pcnt && idx[u] < a.n) {
+                            a.ok[idx[u]] = kv[u];
+                            if (HASV)
+                                a.ov[idx[u]] = vv[u];
+                        }
+                } else {
+                    // most runs lie in one block, whose base address the run
+                    // descriptor holds; the rest read their block from the list,
+                    // behind one branch for the warp: a branch per element keeps
+                    // the reads of the next ones from overlapping
+                    unsigned long long w[U];
+                    uint32_t late = 0;
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const uint32_t i = tid + (k0 + u) * NT;
+                        const uint4 qd = qd16[dig(kv[u])];
+                        idx[u] = i + qd.x;
+                        w[u] = i < pcnt ? (static_cast<unsigned long long>(qd.w) << 32) | qd.z : 0ull;
+                        if (i < pcnt && idx[u] >= qd.y)
+                            late |= 1u << u;
+                    }
+                    if (__any_sync(0xffffffffu, late)) {
+#pragma unroll
+                        for (int u = 0; u < U; ++u)
+                            if ((late >> u) & 1u) {
+                                const uint32_t l = (idx[u] >> a.lb) + qlo[dig(kv[u])];
+                                w[u] = l < TT ? list[l] : 0ull;
+                                idx[u] &= b - 1;
+                            }
+                    }
+#pragma unroll
+                    for (int u = 0; u < U; ++u)
+                        if (w[u]) {
+                            KT *dk = reinterpret_cast<KT *>(w[u] & ~3ull) + idx[u];
+                            *dk = kv[u];
+                            if (HASV) {
+                                uint32_t *dv;
+                                if constexpr (sizeof(KT) == 4)
+                                    dv = reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(dk) +
+                                                                      ((w[u] & 1ull) ? dvA : dvT));
+                                else
+                                    dv = ((w[u] & 1ull) ? a.Av + (dk - a.Ak) : a.Tv + (dk - a.Tk));
+                                *dv = vv[u];
+                            }
+                        }
+                }
+            }
+            // the stage was read and rewritten with generic accesses; it is
+            // refilled with bulk copies (async proxy)
+            fence_proxy_async_smem();
+            bar_arrive(LB8_FREE, NT + 32);
+        }
+        if (end)
+            break;
+        pcnt = cnt;
+
+        // ---- 4. reorder the tile by digit, in place in its stage buffer
+        // (every element is in registers since the barriers above)
+        uint2 *tp = reinterpret_cast<uint2 *>(st); // (key, value) pairs after the reorder
+#pragma unroll
+        for (int it = 0; it < ITEMS; ++it) {
+            const uint32_t pos = row[dig(key[it])] + ((it & 1) ? rk[it >> 1] >> 16 : rk[it >> 1] & 0xFFFFu);
+            if (pos >= uint32_t(TILE)) { // only a broken scan gets here
+                set_status(ST_INTERNAL);
+                continue;
+            }
+            if constexpr (C::PAIR) {
+                tp[pos] = make_uint2(static_cast<uint32_t>(key[it]), val[it]);
+            } else {
+                tk[pos] = key[it];
+                if (HASV)
+                    tv[pos] = val[it];
+            }
+        }
+        // this warp's words for the next tile
+        __syncwarp();
+        {
+            uint4 *z = reinterpret_cast<uint4 *>(tab + 2 * warp * SIGMA);
+#pragma unroll
+            for (int i = 0; i < 2 * SIGMA / 128; ++i)
+                z[i * 32 + lane] = make_uint4(0u, 0u, 0u, 0u);
+        }
+    }
+}
+
+// ---------------------------------------------------------------- launch helpers
+// The round kernel of a configuration: 8-bit digits with NW ranking warps, or
+// 11-bit digits (NW ignored).
+template <typename KT, bool HASV, int DB, int TILE, int NW, bool OOP> struct LbKernel {
+    using C = std::conditional_t<DB == 8, Lb8Cfg<KT, HASV, DB == 8 ? TILE : 4096, NW, OOP>,
+                                 LbCfg<KT, HASV, DB == 8 ? 4096 : TILE, OOP>>;
+    static auto kernel()
+    {
+        if constexpr (DB == 8)
+            return k_lb_round8<KT, HASV, TILE, NW, OOP>;
+        else
+            return k_lb_round11<KT, HASV, TILE, OOP>;
+    }
+    // CTAs of a launch over ntiles tiles (-1: the kernel cannot be set up)
+    static int ctas(size_t ntiles)
+    {
+        static DeviceOnce attr; // per template instance
+        if (attr.run([] {
+                return cudaFuncSetAttribute(kernel(), cudaFuncAttributeMaxDynamicSharedMemorySize, int(C::SMEM));
+            }) != cudaSuccess)
+            return -1;
+        size_t grid = size_t(num_sms()) * C::MINB;
+        if (grid > ntiles)
+            grid = ntiles;
+        return grid < 1 ? 1 : static_cast<int>(grid);
+    }
+};
+
+// Calls f.template operator()<KT, HASV, DB, TILE, NW>() for the configuration.
 template <typename F> static cudaError_t lb_dispatch(int kb, int db, bool hasv, F &&f)
 {
     using u64 = unsigned long long;
     // The largest tiles that two stages and the tables leave room for
     // (per-tile costs scale with sigma, not with the tile), each a multiple
     // of 2048 so that blocks of up to 2048 elements fit whole; 11-bit digits
-    // keep their run offsets and block list in the warp rows (ALIAS).
-    // One group of 16 consumer warps and two stages throughout.  Measured at
-    // 2^30 u32 keys + values, 8-bit digits (round kernel): tiles of 10240,
-    // 7.29 ms; tiles of 4096, 10.7 ms; two groups of 8 warps on tiles of
-    // 4096 with two stages each, 8.21 ms; two groups on 8192 / 6144 with one
-    // stage each, 9.34 / 9.93 ms.  Per-tile work over the sigma buckets
-    // (column sums, scan, look-back, block lists) costs about 6800 cycles a
-    // tile whatever its size, so the largest tile wins even though a second
-    // group overlaps some of it.
+    // keep their run offsets and block list in the warp rows.
     if (kb == 4) {
         if (db == 8)
-            return hasv ? f.template operator()<uint32_t, true, 8, 10240, 16, 1, 2>()
-                        : f.template operator()<uint32_t, false, 8, 16384, 16, 1, 2>();
-        return hasv ? f.template operator()<uint32_t, true, 11, 8192, 16, 1, 2>()
-                    : f.template operator()<uint32_t, false, 11, 16384, 16, 1, 2>();
+            return hasv ? f.template operator()<uint32_t, true, 8, 10240, 16>()
+                        : f.template operator()<uint32_t, false, 8, 16384, 16>();
+        return hasv ? f.template operator()<uint32_t, true, 11, 8192, 16>()
+                    : f.template operator()<uint32_t, false, 11, 16384, 16>();
     }
     if (db == 8)
-        return hasv ? f.template operator()<u64, true, 8, 6144, 16, 1, 2>()
-                    : f.template operator()<u64, false, 8, 10240, 16, 1, 2>();
-    return hasv ? f.template operator()<u64, true, 11, 4096, 16, 1, 2>()
-                : f.template operator()<u64, false, 11, 8192, 16, 1, 2>();
+        return hasv ? f.template operator()<u64, true, 8, 6144, 16>()
+                    : f.template operator()<u64, false, 8, 10240, 16>();
+    return hasv ? f.template operator()<u64, true, 11, 4096, 16>() : f.template operator()<u64, false, 11, 8192, 16>();
 }
 
 // Radsort rounds with a tile shape: 0 or 1, the configuration above; 2 (8-bit
-// digits), two groups of 8 warps on smaller tiles with two stages each, which
-// the autotuner may pick where the arrays hold few tiles per SM
+// digits), two CTAs of 8 ranking warps per SM on smaller tiles, which the
+// autotuner may pick where the arrays hold few tiles per SM
 template <typename F> static cudaError_t lb_dispatch_shape(int kb, int db, bool hasv, int shape, F &&f)
 {
     using u64 = unsigned long long;
     if (shape == 2 && db == 8) {
         if (kb == 4)
-            return hasv ? f.template operator()<uint32_t, true, 8, 4096, 8, 2, 4>()
-                        : f.template operator()<uint32_t, false, 8, 8192, 8, 2, 4>();
-        return hasv ? f.template operator()<u64, true, 8, 4096, 8, 2, 2>()
-                    : f.template operator()<u64, false, 8, 4096, 8, 2, 4>();
+            return hasv ? f.template operator()<uint32_t, true, 8, 4096, 8>()
+                        : f.template operator()<uint32_t, false, 8, 8192, 8>();
+        return hasv ? f.template operator()<u64, true, 8, 4096, 8>() : f.template operator()<u64, false, 8, 4096, 8>();
     }
     return lb_dispatch(kb, db, hasv, f);
 }
@@ -1380,7 +1939,7 @@ uint32_t lb_tile(int kb, int db, bool hasv, int shape)
 {
     uint32_t r = 0;
     lb_dispatch_shape(kb, db, hasv, shape,
-                      [&]<typename KT, bool HASV, int DB, int TILE, int NW, int NG, int STAGES>() {
+                      [&]<typename KT, bool HASV, int DB, int TILE, int NW>() {
                           r = TILE;
                           return cudaSuccess;
                       });
@@ -1473,10 +2032,10 @@ cudaError_t launch_grid_round(const Geom &g, const Bufs &w, const uint32_t *pi, 
 {
     const uint32_t n = static_cast<uint32_t>(g.n);
     return lb_dispatch_shape(g.kb, g.db, g.hasv, g.shape,
-                             [&]<typename KT, bool HASV, int DB, int TILE, int NW, int NG, int STAGES>() {
-        using C = LbCfg<KT, HASV, DB, TILE, NW, NG, STAGES, false>;
+                             [&]<typename KT, bool HASV, int DB, int TILE, int NW>() {
+        using K = LbKernel<KT, HASV, DB, TILE, NW, false>;
         const size_t ntiles = (g.n + TILE - 1) / TILE;
-        const int grid = lb_ctas<KT, HASV, DB, TILE, NW, NG, STAGES, false>(ntiles);
+        const int grid = K::ctas(ntiles);
         if (grid < 0)
             return cudaErrorInvalidValue;
         LbArgs<KT> a{};
@@ -1501,7 +2060,7 @@ cudaError_t launch_grid_round(const Geom &g, const Bufs &w, const uint32_t *pi, 
         a.npi = g.npi;
         a.lb = g.lb;
         a.shift = static_cast<uint32_t>(round * g.db);
-        k_lb_round<KT, HASV, DB, TILE, NW, NG, STAGES, false><<<grid, C::THREADS, C::SMEM, st>>>(a);
+        K::kernel()<<<grid, K::C::THREADS, K::C::SMEM, st>>>(a);
         g_launches += 1;
         return cudaGetLastError();
     });
@@ -1557,9 +2116,9 @@ cudaError_t launch_lsd_oop_ws(void *keys, uint32_t *vals, void *keys_alt, uint32
         g_launches += 1;
     }
     if (e == cudaSuccess)
-        e = lb_dispatch(kb, db, vals != nullptr, [&]<typename KT, bool HASV, int DB, int TILE, int NW, int NG, int STAGES>() {
-        using C = LbCfg<KT, HASV, DB, TILE, NW, NG, STAGES, true>;
-        const int grid = lb_ctas<KT, HASV, DB, TILE, NW, NG, STAGES, true>(ntiles);
+        e = lb_dispatch(kb, db, vals != nullptr, [&]<typename KT, bool HASV, int DB, int TILE, int NW>() {
+        using K = LbKernel<KT, HASV, DB, TILE, NW, true>;
+        const int grid = K::ctas(ntiles);
         if (grid < 0)
             return cudaErrorInvalidValue;
         KT *src = static_cast<KT *>(keys), *dst = static_cast<KT *>(keys_alt);
@@ -1579,7 +2138,7 @@ cudaError_t launch_lsd_oop_ws(void *keys, uint32_t *vals, void *keys_alt, uint32
             a.n = nn;
             a.ntiles = static_cast<uint32_t>(ntiles);
             a.shift = static_cast<uint32_t>(r * DB);
-            k_lb_round<KT, HASV, DB, TILE, NW, NG, STAGES, true><<<grid, C::THREADS, C::SMEM, st>>>(a);
+            K::kernel()<<<grid, K::C::THREADS, K::C::SMEM, st>>>(a);
             g_launches += 1;
             std::swap(src, dst);
             std::swap(vs, vd);
