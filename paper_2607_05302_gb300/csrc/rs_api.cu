@@ -359,10 +359,11 @@ static size_t layout(const Geom &g, void *base, Bufs *w)
         b.aux = static_cast<uint32_t *>(take(2 * npi2 * 4));
         b.P = static_cast<uint2 *>(take(8));
         b.E = static_cast<unsigned long long *>(take(2 * 8));
+        b.tab = static_cast<uint32_t *>(take(grid_tab_words(g) * 4));
+        // (one memset clears from here to the end of the look-back words)
         b.state = static_cast<uint32_t *>(take(ST_WORDS * 4));
         b.ctr = static_cast<uint32_t *>(take(64 * 4));
         b.hist = static_cast<uint32_t *>(take(size_t(g.nt) * g.sigma * 4));
-        b.tab = static_cast<uint32_t *>(take((3 * size_t(g.sigma) + 4) * 4));
         const size_t jump = align_up(npi2 * 8, 256), fin = finalize_extra_bytes(g);
         const size_t lbw = grid_ring_bytes(g);
         char *z = static_cast<char *>(take(lbw > jump + fin ? lbw : jump + fin));
@@ -434,16 +435,13 @@ static cudaError_t run_rounds(const Geom &g, Bufs &w, int rounds, cudaStream_t s
     cudaError_t e;
     if (g.grid) {
         uint32_t *pc = w.aux, *pn = w.aux + npi2;
-        e = cudaMemsetAsync(w.state, 0, ST_WORDS * 4, st);
-        if (e == cudaSuccess)
-            e = cudaMemsetAsync(w.ctr, 0, 64 * 4, st);
-        if (e == cudaSuccess) {
+        {
             Scope sc(0, -1, st);
             e = launch_grid_setup(g, w, pc, st);
         }
         for (int r = 0; r < rounds && e == cudaSuccess; ++r) {
-            {   // the tables of this digit and the parts of the next map
-                // known before the round (head start, shared blocks)
+            {   // the parts of the next map known before the round (head
+                // start, shared blocks, each bucket's first blocks)
                 Scope sc(2, r, st);
                 e = launch_grid_prep(g, w, pc, pn, r, st);
             }
@@ -1555,8 +1553,8 @@ radsort_status radsort_perm_open(void *keys, uint32_t *values, size_t n, int key
     h->hist_ok = true; // setup takes the histograms of the input
     h->finalized = false;
     cudaStream_t st = as_stream(stream);
-    cudaError_t e = cudaMemsetAsync(h->w.state, 0, ST_WORDS * 4, st);
-    if (e == cudaSuccess) {
+    cudaError_t e;
+    {
         Scope sc(0, -1, st);
         e = launch_grid_setup(g, h->w, h->pc, st);
     }
@@ -1583,6 +1581,8 @@ radsort_status radsort_perm_rounds(radsort_perm *h, int first, int count, void *
     if (e == cudaSuccess && !h->hist_ok) {
         Scope sc(0, -1, st);
         e = launch_block_hist(g, h->w, h->pc, st);
+        if (e == cudaSuccess)
+            e = launch_grid_tables(g, h->w, nullptr, false, st);
         if (e == cudaSuccess)
             h->hist_ok = true;
     }

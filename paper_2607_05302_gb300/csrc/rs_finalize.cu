@@ -204,45 +204,6 @@ __global__ void k_fz_jump(unsigned long long *jump, uint32_t npi, int mode, uint
         atomicAdd(&changes[round], 1u);
 }
 
-// The same pointer jumping for a small permutation (n_pi <= FZ_SMALL_NPI):
-// one CTA with the entries in shared memory, steps until one changes
-// nothing (windows at least double each step, so 33 steps bound it), in one
-// launch instead of one per (JUMP_STEPS + 1)-fold growth.
-constexpr uint32_t FZ_SMALL_NPI = 12288;
-
-__global__ void __launch_bounds__(1024) k_fz_jump_small(unsigned long long *jump, uint32_t npi, int mode)
-{
-    extern __shared__ unsigned long long sj[];
-    for (uint32_t x = threadIdx.x; x < npi; x += blockDim.x)
-        sj[x] = jump[x];
-    __syncthreads();
-    for (int step = 0; step < 34; ++step) {
-        bool changed = false;
-        for (uint32_t x = threadIdx.x; x < npi; x += blockDim.x) {
-            const unsigned long long e = sj[x];
-            const uint32_t v = hi32(e);
-            if (v == ABS)
-                continue;
-            const uint32_t nx = lo32(e);
-            if (nx >= npi)
-                continue; // only a broken entry points out of the permutation
-            const unsigned long long f = sj[nx];
-            const uint32_t fv = hi32(f);
-            if (fv == ABS)
-                continue;
-            const unsigned long long ne = pk(lo32(f), mode == 0 ? min(v, fv) : v + fv);
-            if (ne != e) {
-                sj[x] = ne;
-                changed = true;
-            }
-        }
-        if (!__syncthreads_or(changed))
-            break;
-    }
-    for (uint32_t x = threadIdx.x; x < npi; x += blockDim.x)
-        jump[x] = sj[x];
-}
-
 // classify each moving block in pi's top bits: moving / on a cycle / the
 // cycle's minimum position
 __global__ void k_fz_classify(FinArgs a)
@@ -344,6 +305,142 @@ __global__ void k_fz_order(FinArgs a)
     }
 }
 
+// Everything up to the order array for a small permutation (n_pi <=
+// FZ_SMALL_NPI): one CTA with the map and the entries in shared memory, one
+// launch.  The steps are those of the kernels above; each jumping pass stops
+// at the step that changes nothing (windows at least double each step, so 34
+// steps bound it).  What bounds it is latency: with nine launches
+// (the jumping in one CTA already) Finalize took 74 us at 2^20 elements of 8
+// bytes and 101 at 2^22, with this one 45 and 67.
+constexpr uint32_t FZ_SMALL_NPI = 12288;
+
+__global__ void __launch_bounds__(1024) k_fz_plan_small(FinArgs a, uint32_t clear)
+{
+    extern __shared__ unsigned long long sj[]; // n_pi entries, then the map (n_pi words)
+    uint32_t *sp = reinterpret_cast<uint32_t *>(sj + a.npi);
+    __shared__ uint32_t s_order, s_rec;
+    const uint32_t tid = threadIdx.x, nt = blockDim.x, npi = a.npi;
+    const uint32_t NL = a.state[ST_F] - a.H, R = NL - a.nA;
+    for (uint32_t i = tid; i < clear; i += nt) // counters and flags of the moves
+        a.ctr[i] = 0u;
+    if (tid == 0)
+        s_order = s_rec = 0;
+    auto reset = [&]() {
+        for (uint32_t x = tid; x < npi; x += nt)
+            sj[x] = pk(x, ABS);
+        __syncthreads();
+    };
+    auto jump = [&](bool sum) {
+        for (int step = 0; step < 34; ++step) {
+            bool changed = false;
+            for (uint32_t x = tid; x < npi; x += nt) {
+                const unsigned long long e = ld64(&sj[x]);
+                const uint32_t v = hi32(e), nx = lo32(e);
+                if (v == ABS || nx >= npi)
+                    continue; // (only a broken entry points out of the permutation)
+                const unsigned long long f = ld64(&sj[nx]);
+                const uint32_t fv = hi32(f);
+                if (fv == ABS)
+                    continue;
+                const unsigned long long ne = pk(lo32(f), sum ? v + fv : min(v, fv));
+                if (ne != e) {
+                    st64(&sj[x], ne);
+                    changed = true;
+                }
+            }
+            if (!__syncthreads_or(changed))
+                break;
+        }
+    };
+    reset();
+    for (uint32_t q = tid; q < NL; q += nt) { // edges
+        const uint32_t x = a.pi[a.H + q], t = target_of(q, a.nA, a.nT);
+        sp[q] = x;
+        if (x < npi && x != t)
+            sj[x] = pk(t, x);
+    }
+    __syncthreads();
+    jump(false);
+    for (uint32_t q = tid; q < NL; q += nt) { // moving, on a cycle, the cycle's minimum
+        const uint32_t x = sp[q];
+        if (x >= npi || x == target_of(q, a.nA, a.nT))
+            continue;
+        const unsigned long long e = sj[x];
+        const bool cyc = lo32(e) < npi && hi32(sj[lo32(e)]) != ABS;
+        sp[q] = x | F_MOVE | (cyc ? F_CYC : 0u) | (cyc && hi32(e) == x ? F_MIN : 0u);
+    }
+    __syncthreads();
+    reset();
+    for (uint32_t q = tid; q < NL; q += nt) { // rank edges
+        const uint32_t v = sp[q];
+        if ((v & F_MOVE) && !(v & F_MIN))
+            sj[v & POS_MASK] = pk(target_of(q, a.nA, a.nT), 1u);
+    }
+    __syncthreads();
+    jump(true);
+    for (uint32_t q = tid; q < NL; q += nt) { // chains
+        const uint32_t v = sp[q];
+        if (!(v & F_MOVE))
+            continue;
+        const uint32_t x = v & POS_MASK;
+        const bool cyc = (v & F_CYC) != 0;
+        uint32_t h, r;
+        if (cyc) {
+            if (!(v & F_MIN))
+                continue;
+            h = x;
+            r = hi32(sj[target_of(q, a.nA, a.nT)]);
+        } else {
+            if (!((x < a.nT && x >= R) || x >= a.nT + a.nA))
+                continue;
+            const unsigned long long e = sj[x];
+            h = lo32(e);
+            r = hi32(e);
+        }
+        const uint32_t len = r + 1;
+        const uint32_t base = atomicAdd(&s_order, len);
+        uint32_t defer = 0;
+        if (cyc && base / a.K != (base + len - 1) / a.K) {
+            const uint32_t ri = atomicAdd(&s_rec, 1u);
+            if (ri < a.nrec_cap) {
+                const uint32_t slot = ri < a.nslots ? ri : SLOT_NONE;
+                a.rec[ri] = make_uint4(base, len, slot, 0);
+                defer = slot == SLOT_NONE ? H_DEFER : 0u;
+            } else {
+                set_status(ST_INTERNAL);
+            }
+        }
+        if (h < npi)
+            st64(&sj[h], pk(base, len | H_HEAD | (cyc ? H_CYC : 0u) | defer));
+    }
+    __syncthreads();
+    if (tid == 0) {
+        a.ctr[C_ORDER] = s_order;
+        a.ctr[C_REC] = s_rec;
+    }
+    for (uint32_t x = tid; x < npi; x += nt) { // order
+        const unsigned long long e = sj[x];
+        const uint32_t v = hi32(e);
+        if (v == ABS)
+            continue;
+        uint32_t base, info, r;
+        if (v & H_HEAD) {
+            base = lo32(e);
+            info = v;
+            r = 0;
+        } else {
+            const unsigned long long hd = lo32(e) < npi ? sj[lo32(e)] : 0ull;
+            base = lo32(hd);
+            info = hi32(hd);
+            r = v;
+        }
+        const uint32_t len = info & H_LEN;
+        if (base + r < npi)
+            a.pi[base + r] = x | (r == 0 ? O_FIRST : 0u) | (r + 1 == len ? O_LAST : 0u) |
+                             ((info & H_CYC) ? O_CYC : 0u) | ((info & H_DEFER) ? O_DEFER : 0u);
+    }
+}
+
 // record of the straddling cycle that contains order index g (linear search;
 // straddling cycles are few: random-like permutations have O(log n) cycles)
 __device__ uint4 find_rec(const FinArgs &a, uint32_t g)
@@ -417,7 +514,7 @@ __global__ void __launch_bounds__(FIN_T) k_fz_move(FinArgs a)
             const uint32_t o = a.pi[g];
             uint32_t kind = 0, src = 0, slot = SLOT_NONE, save = SLOT_NONE;
             if (o & O_DEFER) {
-                kind = 0; // the whole cycle is moved by k_fz_move_deferred
+                kind = 0; // the whole cycle is moved after the strides
             } else if (o & O_LAST) {
                 if (o & O_CYC) {
                     const uint4 r = find_rec(a, g);
@@ -514,17 +611,14 @@ __global__ void __launch_bounds__(FIN_T) k_fz_move(FinArgs a)
     }
     if (threadIdx.x < 32)
         bulk_wait_all();
-}
-
-// straddling cycles beyond the slot capacity: one CTA moves a whole cycle,
-// K-1 blocks at a time, holding the head block in shared memory
-template <typename KT>
-__global__ void __launch_bounds__(FIN_T) k_fz_move_deferred(FinArgs a)
-{
-    extern __shared__ __align__(16) unsigned char fsm[];
-    const BlockIO<KT> io(a);
-    const uint32_t nr = min(a.ctr[C_REC], a.nrec_cap);
-    const uint32_t KB = a.K - 1;
+    // straddling cycles beyond the slot capacity (no stride touches their
+    // blocks): one CTA moves a whole cycle, K-1 blocks at a time, holding the
+    // head block in shared memory
+    const uint32_t nr = min(a.ctr[C_REC], a.nrec_cap), KB = a.K - 1;
+    if (nr <= a.nslots)
+        return;
+    fence_proxy_async_smem();
+    __syncthreads();
     for (uint32_t ri = blockIdx.x; ri < nr; ri += gridDim.x) {
         const uint4 r = a.rec[ri];
         if (r.z != SLOT_NONE)
@@ -942,7 +1036,10 @@ cudaError_t fin_impl(const Geom &g, const Bufs &w, uint32_t *pi, unsigned long l
     a.K = L.K;
     a.W = L.W;
 
-    cudaError_t e = cudaMemsetAsync(base, 0, L.rec, st);
+    cudaError_t e = cudaSuccess;
+    const bool small = g.npi <= FZ_SMALL_NPI;
+    if (!small || !g.grid) // (a small permutation's plan clears what the moves need)
+        e = cudaMemsetAsync(base, 0, L.rec, st);
     if (e != cudaSuccess)
         return e;
     if (!g.grid) {
@@ -951,43 +1048,40 @@ cudaError_t fin_impl(const Geom &g, const Bufs &w, uint32_t *pi, unsigned long l
             return e;
     }
     const int sms = num_sms();
-    int grid = static_cast<int>((g.npi + FIN_T - 1) / FIN_T);
-    if (grid > sms * 8)
-        grid = sms * 8;
-    if (grid < 1)
-        grid = 1;
-    // launches until every window reaches n_pi (growth (JUMP_STEPS+1)-fold
-    // each), plus one that sees no change
-    int rounds = 1;
-    for (unsigned long long w = JUMP_STEPS + 1; w < g.npi; w *= JUMP_STEPS + 1)
-        ++rounds;
-    rounds += 1;
-    static DeviceOnce jattr;
-    const cudaError_t ej = jattr.run([] {
-        return cudaFuncSetAttribute(k_fz_jump_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    int(FZ_SMALL_NPI * 8));
-    });
-    if (ej != cudaSuccess)
-        return ej;
-    const bool small = g.npi <= FZ_SMALL_NPI;
-    k_fz_reset<<<grid, FIN_T, 0, st>>>(a.jump, g.npi);
-    k_fz_edges<<<grid, FIN_T, 0, st>>>(a);
-    uint32_t *chg = a.ctr + C_WORDS; // per-round change counters (cleared with the flags)
-    if (small)
-        k_fz_jump_small<<<1, 1024, size_t(g.npi) * 8, st>>>(a.jump, g.npi, 0);
-    else
+    if (small) {
+        static DeviceOnce jattr;
+        const cudaError_t ej = jattr.run([] {
+            return cudaFuncSetAttribute(k_fz_plan_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        int(FZ_SMALL_NPI * 12));
+        });
+        if (ej != cudaSuccess)
+            return ej;
+        k_fz_plan_small<<<1, 1024, size_t(g.npi) * 12, st>>>(a, static_cast<uint32_t>(L.rec / 4));
+        g_launches += 1;
+    } else {
+        int grid = static_cast<int>((g.npi + FIN_T - 1) / FIN_T);
+        if (grid > sms * 8)
+            grid = sms * 8;
+        // launches until every window reaches n_pi (growth (JUMP_STEPS+1)-fold
+        // each), plus one that sees no change
+        int rounds = 1;
+        for (unsigned long long w = JUMP_STEPS + 1; w < g.npi; w *= JUMP_STEPS + 1)
+            ++rounds;
+        rounds += 1;
+        k_fz_reset<<<grid, FIN_T, 0, st>>>(a.jump, g.npi);
+        k_fz_edges<<<grid, FIN_T, 0, st>>>(a);
+        uint32_t *chg = a.ctr + C_WORDS; // per-round change counters (cleared with the flags)
         for (int r = 0; r < rounds; ++r)
             k_fz_jump<<<grid, FIN_T, 0, st>>>(a.jump, g.npi, 0, chg, r);
-    k_fz_classify<<<grid, FIN_T, 0, st>>>(a);
-    k_fz_reset<<<grid, FIN_T, 0, st>>>(a.jump, g.npi);
-    k_fz_rank_edges<<<grid, FIN_T, 0, st>>>(a);
-    if (small)
-        k_fz_jump_small<<<1, 1024, size_t(g.npi) * 8, st>>>(a.jump, g.npi, 1);
-    else
+        k_fz_classify<<<grid, FIN_T, 0, st>>>(a);
+        k_fz_reset<<<grid, FIN_T, 0, st>>>(a.jump, g.npi);
+        k_fz_rank_edges<<<grid, FIN_T, 0, st>>>(a);
         for (int r = 0; r < rounds; ++r)
             k_fz_jump<<<grid, FIN_T, 0, st>>>(a.jump, g.npi, 1, chg + 64, r);
-    k_fz_chains<<<grid, FIN_T, 0, st>>>(a);
-    k_fz_order<<<grid, FIN_T, 0, st>>>(a);
+        k_fz_chains<<<grid, FIN_T, 0, st>>>(a);
+        k_fz_order<<<grid, FIN_T, 0, st>>>(a);
+        g_launches += 7 + 2 * rounds;
+    }
     const size_t bbytes = size_t(g.b) * (g.kb + (g.hasv ? 4 : 0));
     const size_t msm = bbytes * L.K;
     const size_t kcap = L.W + 2 * (16 / g.kb) * (MAXSEG + 1), vcap = L.W + 8 * (MAXSEG + 1);
@@ -995,9 +1089,6 @@ cudaError_t fin_impl(const Geom &g, const Bufs &w, uint32_t *pi, unsigned long l
     static DeviceOnce attr;
     const cudaError_t ea = attr.run([] {
         cudaError_t e = cudaFuncSetAttribute(k_fz_move<KT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 << 10);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_fz_move_deferred<KT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     160 << 10);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_fz_compact<KT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      160 << 10);
@@ -1008,14 +1099,15 @@ cudaError_t fin_impl(const Geom &g, const Bufs &w, uint32_t *pi, unsigned long l
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fz_move<KT>, FIN_T, msm);
     k_fz_move<KT><<<sms * (per_sm > 0 ? per_sm : 1), FIN_T, msm, st>>>(a);
-    k_fz_move_deferred<KT><<<sms, FIN_T, msm, st>>>(a);
+    g_launches += 1;
     if (g.grid) {
         // every block but the last is full: only the tail (now in scratch
         // block 0) remains to be copied behind A's last block
         const uint32_t tail = static_cast<uint32_t>(g.n - size_t(g.nA) * g.b);
         if (tail)
             k_fz_tail<KT><<<(tail + FIN_T - 1) / FIN_T, FIN_T, 0, st>>>(a, tail);
-        g_launches += 10 + 2 * (small ? 1 : rounds);
+        if (tail)
+            g_launches += 1;
         return cudaGetLastError();
     }
     uint4 *wplan = reinterpret_cast<uint4 *>(base + L.wplan);
@@ -1023,7 +1115,7 @@ cudaError_t fin_impl(const Geom &g, const Bufs &w, uint32_t *pi, unsigned long l
     k_fz_winplan<<<(L.nwin + FIN_T - 1) / FIN_T, FIN_T, 0, st>>>(a, wplan, wsegs);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fz_compact<KT>, FIN_T, csm);
     k_fz_compact<KT><<<sms * (per_sm > 0 ? per_sm : 1), FIN_T, csm, st>>>(a, wplan, wsegs);
-    g_launches += 11 + 2 * (small ? 1 : rounds);
+    g_launches += 2;
     return cudaGetLastError();
 }
 

@@ -315,73 +315,68 @@ template <int DB> __global__ void __launch_bounds__(1024) k_offsets(const uint32
 }
 
 // ---------------------------------------------------------------- grid layout: setup, tables
-// pi = [scratch 0 .. H) ++ [A's blocks] ++ [scratch block H: the input
-// tail]; the tail is copied there; P holds the one partial block.
-template <typename KT>
-__global__ void k_grid_setup(const KT *Ak, const uint32_t *Av, KT *Tk, uint32_t *Tv, uint32_t n,
-                             uint32_t b, uint32_t H, uint32_t nA, uint32_t npi, uint32_t *pi,
-                             uint2 *P, uint32_t *state)
-{
-    const uint32_t nT = H + 1;
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < npi; i += gridDim.x * blockDim.x)
-        pi[i] = i < H ? i : (i < H + nA ? nT + (i - H) : H);
-    const uint32_t tail = n - nA * b;
-    for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < tail; j += gridDim.x * blockDim.x) {
-        Tk[size_t(H) * b + j] = Ak[size_t(nA) * b + j];
-        if (Av)
-            Tv[size_t(H) * b + j] = Av[size_t(nA) * b + j];
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        P[0] = make_uint2(H + nA, tail);
-        state[ST_F] = H + nA + 1;
-        state[ST_NP] = 1;
-        state[ST_FPREV] = H + nA + 1;
-        state[ST_LOFFTOT] = 0;
-    }
-}
+// Tables of one round, in words of Bufs::tab (GRID_TAB_WORDS a round): bucket
+// starts O (sigma + 1), each bucket's range of non-shared blocks [ns0, ns1),
+// the free-list index of its first one, the shared blocks (those with a bucket
+// start strictly inside) in order, and a header.
+enum { TAB_SKIP = 0, TAB_TAKEN = 1, TAB_NS = 2 }; // identity round; free-list entries taken before it; shared blocks
+template <int SIGMA> struct GridTab {
+    static constexpr int O = 0, NS0 = SIGMA + 1, NS1 = NS0 + SIGMA, FREE = NS1 + SIGMA, SHARED = FREE + SIGMA,
+                         HDR = SHARED + SIGMA, WORDS = HDR + 3;
+};
 
-// Tables of one round (one CTA of 1024 threads): bucket starts O, the shared
-// blocks (those with a bucket start strictly inside), per bucket its range of
-// non-shared blocks [ns0, ns1); pi' prefilled with the blocks taken before
-// the round (shared blocks, then the first non-shared block of each bucket),
-// the next head start and (n % b == 0) the empty tail block.  A digit with
-// one non-empty bucket leaves the sequence unchanged: pi' = pi and the round
-// is skipped.
-template <int DB>
-__global__ void __launch_bounds__(1024) k_grid_prep(const uint32_t *hist_r, uint32_t n, uint32_t lb,
-                                                     uint32_t H, uint32_t nA, uint32_t npi,
-                                                     const uint32_t *pi, uint32_t *pin,
-                                                     uint32_t *tab, uint32_t *state, uint32_t clear)
+// The tables of rounds r0 .. r0 + nr - 1 from the digit counts alone, one CTA
+// of 1024 threads each; the other CTAs (setup) write the first map,
+// pi = [scratch 0 .. H) ++ [A's blocks] ++ [scratch block H: the input tail],
+// and copy that tail.  A digit with one non-empty bucket leaves the sequence
+// unchanged: its round is skipped.
+template <typename KT, int DB>
+__global__ void __launch_bounds__(1024)
+    k_grid_tables(const uint32_t *hist, uint32_t *tab, uint32_t r0, uint32_t nr, uint32_t n, uint32_t lb, uint32_t H,
+                  uint32_t nA, uint32_t npi, const KT *Ak, const uint32_t *Av, KT *Tk, uint32_t *Tv, uint32_t *pi,
+                  uint2 *P, uint32_t *state)
 {
     constexpr int SIGMA = 1 << DB;
+    using T = GridTab<SIGMA>;
+    const uint32_t b = 1u << lb;
+    if (blockIdx.x >= nr) { // setup (Alg. 4)
+        const uint32_t id = (blockIdx.x - nr) * blockDim.x + threadIdx.x, step = (gridDim.x - nr) * blockDim.x;
+        const uint32_t nT = H + 1, tail = n - nA * b;
+        for (uint32_t i = id; i < npi; i += step)
+            pi[i] = i < H ? i : (i < H + nA ? nT + (i - H) : H);
+        for (uint32_t j = id; j < tail; j += step) {
+            Tk[size_t(H) * b + j] = Ak[size_t(nA) * b + j];
+            if (Av)
+                Tv[size_t(H) * b + j] = Av[size_t(nA) * b + j];
+        }
+        if (id == 0) {
+            P[0] = make_uint2(H + nA, tail);
+            state[ST_F] = H + nA + 1;
+            state[ST_NP] = 1;
+            state[ST_FPREV] = H + nA + 1;
+            state[ST_LOFFTOT] = 0;
+        }
+        return;
+    }
     // s_a: scan buffer; s_list: bucket of the k-th bucket start strictly
     // inside a block, later the k-th shared block
     __shared__ uint32_t s_O[SIGMA + 1], s_cnt[SIGMA], s_a[SIGMA], s_list[SIGMA], s_tmp[40];
-    __shared__ int s_skip;
-    const uint32_t b = 1u << lb;
+    const uint32_t *hist_r = hist + size_t(r0 + blockIdx.x) * SIGMA;
+    uint32_t *t = tab + size_t(r0 + blockIdx.x) * T::WORDS;
     auto bar = [] { __syncthreads(); };
-    // a small map is cleared here rather than by a memset launch
-    for (uint32_t i = threadIdx.x; i < clear; i += blockDim.x)
-        pin[H + i] = 0xFFFFFFFFu;
-    if (threadIdx.x == 0)
-        s_skip = 0;
-    __syncthreads();
+    bool one = false;
     for (int c = threadIdx.x; c < SIGMA; c += blockDim.x) {
         const uint32_t v = hist_r[c];
         s_cnt[c] = v;
         s_O[c] = v;
-        if (v == n)
-            s_skip = 1;
+        one |= v == n;
     }
-    __syncthreads();
-    block_scan<SIGMA, 1024>(s_O, s_tmp, bar, threadIdx.x);
-    if (s_skip) {
-        for (uint32_t i = threadIdx.x; i < npi; i += blockDim.x)
-            pin[i] = pi[i];
+    if (__syncthreads_or(one)) {
         if (threadIdx.x == 0)
-            state[ST_SKIP] = 1;
+            t[T::HDR + TAB_SKIP] = 1;
         return;
     }
+    block_scan<SIGMA, 1024>(s_O, s_tmp, bar, threadIdx.x);
     if (threadIdx.x == 0)
         s_O[SIGMA] = n;
     // bucket starts strictly inside a block, in order
@@ -416,7 +411,7 @@ __global__ void __launch_bounds__(1024) k_grid_prep(const uint32_t *hist_r, uint
         if (fl[q])
             s_list[s_a[c]] = s_O[c] >> lb;
     __syncthreads();
-    auto find = [&](uint32_t j) -> bool { // is block j shared?
+    auto shared = [&](uint32_t j) -> bool { // is block j shared?
         uint32_t lo = 0, hi = nS;
         while (lo < hi) {
             const uint32_t m = (lo + hi) >> 1;
@@ -427,53 +422,110 @@ __global__ void __launch_bounds__(1024) k_grid_prep(const uint32_t *hist_r, uint
         }
         return lo < nS && s_list[lo] == j;
     };
-    uint32_t *tO = tab, *tns0 = tab + SIGMA + 1, *tns1 = tns0 + SIGMA;
-    for (int c = threadIdx.x; c < SIGMA; c += blockDim.x) {
+    uint32_t ahead[(SIGMA + 1023) / 1024];
+    q = 0;
+    for (int c = threadIdx.x; c < SIGMA; c += blockDim.x, ++q) {
         const uint32_t O = s_O[c], cn = s_cnt[c];
         uint32_t ns0, ns1;
         if (cn > 0) {
             const uint32_t jf = O >> lb, jl = (O + cn - 1) >> lb;
-            ns0 = jf + (find(jf) ? 1u : 0u);
-            ns1 = jl + 1 - (find(jl) ? 1u : 0u);
+            ns0 = jf + (shared(jf) ? 1u : 0u);
+            ns1 = jl + 1 - (shared(jl) ? 1u : 0u);
             if (ns1 < ns0)
                 ns1 = ns0;
         } else {
             ns0 = ns1 = (O + b - 1) >> lb;
         }
-        tO[c] = O;
-        tns0[c] = ns0;
-        tns1[c] = ns1;
+        t[T::O + c] = O;
+        t[T::NS0 + c] = ns0;
+        t[T::NS1 + c] = ns1;
+        if (uint32_t(c) < nS)
+            t[T::SHARED + c] = s_list[c];
+        ahead[q] = min(GRID_AHEAD, ns1 - ns0);
     }
     __syncthreads();
     // the first GRID_AHEAD non-shared blocks of each bucket: entries nS .. nP-1
-    for (int c = threadIdx.x; c < SIGMA; c += blockDim.x)
-        s_a[c] = min(GRID_AHEAD, tns1[c] - tns0[c]);
+    q = 0;
+    for (int c = threadIdx.x; c < SIGMA; c += blockDim.x, ++q)
+        s_a[c] = ahead[q];
     __syncthreads();
     const uint32_t nF = block_scan<SIGMA, 1024>(s_a, s_tmp, bar, threadIdx.x);
-    for (int c = threadIdx.x; c < SIGMA; c += blockDim.x) {
-        const uint32_t k = min(GRID_AHEAD, tns1[c] - tns0[c]);
-        for (uint32_t i = 0; i < k; ++i)
-            pin[H + tns0[c] + i] = pi[nS + s_a[c] + i];
-    }
+    for (int c = threadIdx.x; c < SIGMA; c += blockDim.x)
+        t[T::FREE + c] = nS + s_a[c];
     if (threadIdx.x == 0) {
-        tO[SIGMA] = n;
-        state[ST_SKIP] = 0;
-        state[ST_NS] = nS + nF;
+        t[T::O + SIGMA] = n;
+        t[T::HDR + TAB_SKIP] = 0;
+        t[T::HDR + TAB_TAKEN] = nS + nF;
+        t[T::HDR + TAB_NS] = nS;
     }
-    // pi': shared blocks take free-list entries 0 .. nS-1; the entries after
-    // the last data block taken form the next head start
-    const uint32_t NB = (n + b - 1) >> lb;
-    for (uint32_t k = threadIdx.x; k < nS; k += blockDim.x)
-        pin[H + s_list[k]] = pi[k];
-    for (uint32_t i = threadIdx.x; i < H; i += blockDim.x)
-        pin[i] = pi[NB + i];
-    if (threadIdx.x == 0 && NB == nA)
-        pin[H + nA] = pi[NB + H]; // the empty tail block
-    // the round reads free-list entries 0 .. H + nA only; blocks past them
-    // (free blocks left behind when the sequence was cut short, Alg. 8) keep
-    // their map entries
-    for (uint32_t i = H + nA + 1 + threadIdx.x; i < npi; i += blockDim.x)
-        pin[i] = pi[i];
+}
+
+// pi' before a round, an entry per thread: the next head start (the H
+// free-list entries after the last one taken), the blocks taken before the
+// round (shared block k takes entry k, then the first non-shared blocks of
+// each bucket theirs), the empty tail block when b divides n, and unset
+// entries for the blocks that the round takes.  An identity round copies pi.
+// Latency bounds it: one CTA that made the round's tables and wrote the map
+// took 10-12 us a round (and a memset before it past 65536 blocks); the tables
+// of all rounds in one launch at setup and this kernel take 8 + 4 x 6 us of a
+// sort of 2^20 where that took 45.
+template <int DB>
+__global__ void __launch_bounds__(256)
+    k_grid_fill(const uint32_t *tab, uint32_t n, uint32_t lb, uint32_t H, uint32_t nA, uint32_t npi,
+                const uint32_t *pi, uint32_t *pin)
+{
+    constexpr int SIGMA = 1 << DB;
+    using T = GridTab<SIGMA>;
+    __shared__ uint32_t s_O[SIGMA + 1], s_list[SIGMA];
+    const uint32_t skip = tab[T::HDR + TAB_SKIP], nS = skip ? 0u : tab[T::HDR + TAB_NS];
+    if (!skip) {
+        for (int c = threadIdx.x; c <= SIGMA; c += blockDim.x)
+            s_O[c] = tab[T::O + c];
+        for (uint32_t k = threadIdx.x; k < nS; k += blockDim.x)
+            s_list[k] = tab[T::SHARED + k];
+    }
+    __syncthreads();
+    const uint32_t b = 1u << lb, NB = (n + b - 1) >> lb;
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < npi; i += gridDim.x * blockDim.x) {
+        // (the round reads free-list entries 0 .. H + nA only; blocks past
+        // them, free blocks left behind when the sequence was cut short,
+        // Alg. 8, keep their map entries)
+        uint32_t from = i; // pi entry that pi'[i] is
+        if (!skip && i < H) {
+            from = NB + i;
+        } else if (!skip && i <= H + nA) {
+            const uint32_t j = i - H;
+            if (j >= NB) {
+                from = NB + H;
+            } else {
+                const uint32_t p = j << lb;
+                uint32_t lo = 0, hi = SIGMA; // the bucket of position p: the last with O <= p
+                while (hi - lo > 1) {
+                    const uint32_t m = (lo + hi) >> 1;
+                    if (s_O[m] <= p)
+                        lo = m;
+                    else
+                        hi = m;
+                }
+                const uint32_t next = s_O[lo + 1];
+                if (next < n && next - p < b) { // shared
+                    uint32_t l = 0, h = nS;
+                    while (l < h) {
+                        const uint32_t m = (l + h) >> 1;
+                        if (s_list[m] < j)
+                            l = m + 1;
+                        else
+                            h = m;
+                    }
+                    from = l;
+                } else {
+                    const uint32_t ns0 = tab[T::NS0 + lo];
+                    from = j - ns0 < GRID_AHEAD ? tab[T::FREE + lo] + (j - ns0) : PI_NONE;
+                }
+            }
+        }
+        pin[i] = from == PI_NONE ? PI_NONE : pi[from];
+    }
 }
 
 // ---------------------------------------------------------------- round kernel, 11-bit digits
@@ -545,17 +597,16 @@ template <typename KT> struct LbArgs {
     uint32_t *ticket;       // zeroed
     uint32_t rmask;         // R - 1 (R a power of two)
     uint32_t tagbase;       // tag of tile t: tagbase + t (grows with the round)
-    const uint32_t *state;  // Radsort: ST_NS, ST_SKIP
+    const uint32_t *hdr;    // Radsort: the tables' header
     uint32_t n, ntiles, H, nT, npi, lb, shift;
 };
 
 // Exclusive prefix of bucket c before tile t: sum of the counts of the tiles
 // back to the nearest inclusive prefix, LBW words in flight per step.
-template <int SIGMA>
+template <int SIGMA, int LBW = 8>
 __device__ __forceinline__ uint32_t look_back(const unsigned long long *ring, uint32_t rmask,
                                               uint32_t tagbase, uint32_t t, int c)
 {
-    constexpr int LBW = 8;
     uint32_t excl = 0;
     int x = static_cast<int>(t) - 1;
     unsigned spins = 0;
@@ -626,7 +677,7 @@ __global__ void __launch_bounds__(LbCfg<KT, HASV, TILE, OOP>::THREADS, 1) k_lb_r
     using C = LbCfg<KT, HASV, TILE, OOP>;
     constexpr int SIGMA = C::SIGMA, NT = C::NT, NW = C::NW, STAGES = C::STAGES, DB = C::DB;
     extern __shared__ __align__(128) unsigned char sm[];
-    if (!OOP && a.state[ST_SKIP])
+    if (!OOP && a.hdr[TAB_SKIP])
         return; // the digit is constant: the round is the identity
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     uint16_t *hist = reinterpret_cast<uint16_t *>(sm + C::o_hist);
@@ -816,7 +867,7 @@ __global__ void __launch_bounds__(LbCfg<KT, HASV, TILE, OOP>::THREADS, 1) k_lb_r
     const int ctid = tid, cw = warp;
     uint32_t *tmp = misc + 8;
     auto bar = [] { named_bar(1, NT); };
-    const uint32_t nP = OOP ? 0u : a.state[ST_NS]; // free-list entries taken before the round
+    const uint32_t nP = OOP ? 0u : a.hdr[TAB_TAKEN]; // free-list entries taken before the round
     const uint32_t M = uint32_t(TILE) >> a.lb;
 
     for (uint32_t k = 0;; ++k) { // fill k
@@ -1243,7 +1294,7 @@ __global__ void __launch_bounds__(Lb8Cfg<KT, HASV, TILE, NW, OOP>::THREADS, Lb8C
     constexpr int SIGMA = C::SIGMA, NT = C::NT, ITEMS = C::ITEMS;
     extern __shared__ __align__(128) unsigned char sm[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    if (!OOP && a.state[ST_SKIP])
+    if (!OOP && a.hdr[TAB_SKIP])
         return; // the digit is constant: the round is the identity
     uint32_t *tab = reinterpret_cast<uint32_t *>(sm + C::o_tab);
     uint32_t *part2 = reinterpret_cast<uint32_t *>(sm + C::o_part);
@@ -1455,7 +1506,7 @@ __global__ void __launch_bounds__(Lb8Cfg<KT, HASV, TILE, NW, OOP>::THREADS, Lb8C
         const uint32_t *ns0 = sO + SIGMA + 1, *ns1 = ns0 + SIGMA;
         const uint32_t Oc = sO[c], Oe = sO[c + 1];
         const uint32_t n0 = OOP ? 0u : ns0[c], n1 = OOP ? 0u : ns1[c];
-        const uint32_t nP = OOP ? 0u : a.state[ST_NS]; // free-list entries taken before the round
+        const uint32_t nP = OOP ? 0u : a.hdr[TAB_TAKEN]; // free-list entries taken before the round
         auto kaddr = [&](uint32_t blk) -> KT * {
             return blk < a.nT ? a.Tk + (size_t(blk) << a.lb) : a.Ak + (size_t(blk - a.nT) << a.lb);
         };
@@ -1976,53 +2027,60 @@ size_t grid_ring_bytes(const Geom &g)
 }
 
 // ---------------------------------------------------------------- grid-layout Radsort
+size_t grid_tab_words(const Geom &g)
+{
+    return size_t(g.nt) * (g.db == 8 ? GridTab<256>::WORDS : GridTab<2048>::WORDS);
+}
+
+cudaError_t launch_grid_tables(const Geom &g, const Bufs &w, uint32_t *pi, bool setup, cudaStream_t st)
+{
+    const uint32_t n = static_cast<uint32_t>(g.n), nr = static_cast<uint32_t>(g.nt);
+    int blocks = setup ? static_cast<int>((g.npi + 1023) / 1024) : 0;
+    if (blocks > 1024)
+        blocks = 1024;
+    auto go = [&]<typename KT, int DB>() {
+        k_grid_tables<KT, DB><<<nr + blocks, 1024, 0, st>>>(w.hist, w.tab, 0u, nr, n, g.lb, g.H, g.nA, g.npi,
+                                                           static_cast<const KT *>(w.Ak), w.Av,
+                                                           static_cast<KT *>(w.Tk), w.Tv, pi, w.P, w.state);
+    };
+    using u64 = unsigned long long;
+    if (g.kb == 4)
+        g.db == 8 ? go.template operator()<uint32_t, 8>() : go.template operator()<uint32_t, 11>();
+    else
+        g.db == 8 ? go.template operator()<u64, 8>() : go.template operator()<u64, 11>();
+    g_launches += 1;
+    return cudaGetLastError();
+}
+
 cudaError_t launch_grid_setup(const Geom &g, const Bufs &w, uint32_t *pi, cudaStream_t st)
 {
-    // all digit histograms from the input keys, before any block moves; the
-    // look-back ring starts with no tags
-    cudaError_t e = cudaMemsetAsync(w.hist, 0, size_t(g.nt) * g.sigma * 4, st);
-    if (e == cudaSuccess)
-        e = cudaMemsetAsync(w.status, 0, grid_ring_bytes(g), st);
+    // cleared: the state, the tickets, the histograms (all digits' counts from
+    // the input keys, before any block moves) and the look-back ring (no
+    // tags), which lie in this order
+    char *z0 = reinterpret_cast<char *>(w.state);
+    cudaError_t e = cudaMemsetAsync(z0, 0, reinterpret_cast<char *>(w.status) + grid_ring_bytes(g) - z0, st);
     if (e != cudaSuccess)
         return e;
     e = launch_digit_hist(w.Ak, static_cast<uint32_t>(g.n), g.kb, g.db, w.hist, st);
     if (e != cudaSuccess)
         return e;
-    const uint32_t n = static_cast<uint32_t>(g.n);
-    int blocks = static_cast<int>((g.npi + 255) / 256);
-    if (blocks > 4096)
-        blocks = 4096;
-    if (g.kb == 4)
-        k_grid_setup<uint32_t><<<blocks, 256, 0, st>>>(static_cast<const uint32_t *>(w.Ak), w.Av,
-                                                       static_cast<uint32_t *>(w.Tk), w.Tv, n, g.b,
-                                                       g.H, g.nA, g.npi, pi, w.P, w.state);
-    else
-        k_grid_setup<unsigned long long><<<blocks, 256, 0, st>>>(
-            static_cast<const unsigned long long *>(w.Ak), w.Av, static_cast<unsigned long long *>(w.Tk),
-            w.Tv, n, g.b, g.H, g.nA, g.npi, pi, w.P, w.state);
-    g_launches += 2;
-    return cudaGetLastError();
+    return launch_grid_tables(g, w, pi, true, st);
 }
 
 cudaError_t launch_grid_prep(const Geom &g, const Bufs &w, const uint32_t *pi, uint32_t *pin,
                              int round, cudaStream_t st)
 {
-    const uint32_t NB = static_cast<uint32_t>((g.n + g.b - 1) / g.b);
-    // the new map's data entries start unset: cleared by the prep kernel
-    // itself when there are few of them, else by a memset
-    const uint32_t clear = NB <= 65536 ? NB : 0u;
-    if (!clear) {
-        cudaError_t e = cudaMemsetAsync(pin + g.H, 0xFF, size_t(NB) * 4, st);
-        if (e != cudaSuccess)
-            return e;
-    }
     const uint32_t n = static_cast<uint32_t>(g.n);
+    int blocks = static_cast<int>((g.npi + 255) / 256);
+    const int cap = num_sms() * (g.db == 8 ? 8 : 2);
+    if (blocks > cap)
+        blocks = cap;
     if (g.db == 8)
-        k_grid_prep<8><<<1, 1024, 0, st>>>(w.hist + size_t(round) * g.sigma, n, g.lb, g.H, g.nA, g.npi,
-                                           pi, pin, w.tab, w.state, clear);
+        k_grid_fill<8><<<blocks, 256, 0, st>>>(w.tab + size_t(round) * GridTab<256>::WORDS, n, g.lb, g.H, g.nA, g.npi,
+                                               pi, pin);
     else
-        k_grid_prep<11><<<1, 1024, 0, st>>>(w.hist + size_t(round) * g.sigma, n, g.lb, g.H, g.nA,
-                                            g.npi, pi, pin, w.tab, w.state, clear);
+        k_grid_fill<11><<<blocks, 256, 0, st>>>(w.tab + size_t(round) * GridTab<2048>::WORDS, n, g.lb, g.H, g.nA,
+                                                g.npi, pi, pin);
     g_launches += 1;
     return cudaGetLastError();
 }
@@ -2045,14 +2103,14 @@ cudaError_t launch_grid_round(const Geom &g, const Bufs &w, const uint32_t *pi, 
         a.Tv = w.Tv;
         a.pi = pi;
         a.pin = pin;
-        a.tab = w.tab;
+        a.tab = w.tab + size_t(round) * GridTab<(1 << DB)>::WORDS;
+        a.hdr = a.tab + GridTab<(1 << DB)>::HDR;
         const uint32_t R = ring_rows(ntiles, g.sigma);
         a.ring = reinterpret_cast<unsigned long long *>(w.status);
         a.done = reinterpret_cast<uint32_t *>(a.ring + size_t(R) * g.sigma);
         a.rmask = R - 1;
         a.tagbase = uint32_t(round + 1) << 24;
         a.ticket = w.ctr + round;
-        a.state = w.state;
         a.n = n;
         a.ntiles = static_cast<uint32_t>(ntiles);
         a.H = g.H;

@@ -53,7 +53,7 @@ struct Bufs {
     void *fin;         // Finalize scratch (finalize_extra_bytes)
     // grid layout only
     uint32_t *hist;    // nt*sigma digit counts of the input
-    uint32_t *tab;     // per-round bucket tables (3*sigma + 1 words)
+    uint32_t *tab;     // bucket tables of every round (grid_tab_words)
     uint32_t *status;  // look-back ring (after the rounds: Finalize's jump array and scratch)
     uint32_t *ctr;     // per-round tile tickets
 };
@@ -63,7 +63,7 @@ struct Bufs {
 constexpr uint32_t GRID_AHEAD = 2;
 
 // indices into Bufs::state
-enum { ST_F = 0, ST_NP = 1, ST_FPREV = 2, ST_LOFFTOT = 3, ST_NS = 4, ST_SKIP = 5, ST_WORDS = 8 };
+enum { ST_F = 0, ST_NP = 1, ST_FPREV = 2, ST_LOFFTOT = 3, ST_WORDS = 8 };
 
 // setup (Alg. 4) + chunk bounds of round 0
 cudaError_t launch_setup(const Geom &g, const Bufs &w, uint32_t *pi, cudaStream_t st);
@@ -76,8 +76,11 @@ enum FixMode { FIX_EVEN = 0, FIX_SPLIT = 1, FIX_PER_CHUNK = 2 };
 cudaError_t launch_fixup(const Geom &g, const Bufs &w, const uint32_t *pi_old, uint32_t *pi_new,
                          const uint32_t *UC, const uint32_t *lo_old, uint32_t *lo_new, int mode,
                          cudaStream_t st);
-// grid layout: digit histograms + setup; per round the tables and the
-// prefilled next map (prep), then sortPhase
+// grid layout: digit histograms, every round's tables and setup; per round
+// the prefilled next map (prep), then sortPhase.  launch_grid_tables without
+// setup: the tables alone, from the histograms of the current sequence
+size_t grid_tab_words(const Geom &g);
+cudaError_t launch_grid_tables(const Geom &g, const Bufs &w, uint32_t *pi, bool setup, cudaStream_t st);
 cudaError_t launch_grid_setup(const Geom &g, const Bufs &w, uint32_t *pi, cudaStream_t st);
 cudaError_t launch_grid_prep(const Geom &g, const Bufs &w, const uint32_t *pi, uint32_t *pin,
                              int round, cudaStream_t st);
