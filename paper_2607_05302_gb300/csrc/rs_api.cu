@@ -1025,7 +1025,7 @@ radsort_status seg_plan(const uint64_t *offh, size_t nseg, int kb, bool hasv, in
     sp->level = sp->ip ? level : 0;
     sp->med_ctas = !med_max ? 0
                    : sp->ip ? static_cast<uint32_t>(nmed < ip_ctas ? nmed : ip_ctas)
-                            : seg_med_ctas(med_max, kb, hasv,
+                            : seg_med_ctas(med_max, kb, hasv, db,
                                            static_cast<size_t>(SEG_MED_SHARE * double(n) * (kb + (hasv ? 4 : 0))));
     sp->base = (seg_scratch_bytes(kb, hasv, nseg, med_max, sp->med_ctas, sp->ip) + 255) / 256 * 256;
     sp->large = large;

@@ -101,6 +101,10 @@ __device__ __forceinline__ void fence_proxy_async_smem()
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
+// The same for memory in general: before bulk copies that read global memory
+// written with plain stores.
+__device__ __forceinline__ void fence_proxy_async_all() { asm volatile("fence.proxy.async;" ::: "memory"); }
+
 // 1-D bulk copy global -> shared through the TMA engine; completion is
 // signalled on `bar` as transaction bytes.  dst, src and bytes must be
 // multiples of 16.
@@ -167,6 +171,36 @@ template <int DB> __device__ __forceinline__ unsigned peer_mask(uint32_t d, bool
         m &= on ? bal : ~bal;
     }
     return m;
+}
+
+// Stable ranks of a half-warp's elements, ITEMS rows of 16: row holds a zeroed
+// word per digit, the count so far in its high half and the lanes of the
+// present row in its low half.  Lanes with the same digit OR their bit into the
+// digit's word and read it back; the last of them writes the new count (its
+// rank + 1) with the lane bits cleared.  digit(it): this lane's digit in row
+// it; real(it): whether it has an element there (missing ones come last).
+// rk: two 16-bit ranks a word.  All 32 lanes call it, each half with its row.
+template <int ITEMS, typename D, typename V>
+__device__ __forceinline__ void rank_half_warp(uint32_t *row, D &&digit, V &&real, uint32_t (&rk)[(ITEMS + 1) / 2])
+{
+    const uint32_t l16 = threadIdx.x & 15u, ltm = (1u << l16) - 1u, gtm = 0xFFFFu & ~((2u << l16) - 1u);
+#pragma unroll
+    for (int it = 0; it < ITEMS; ++it) {
+        uint32_t *w = row + digit(it);
+        if (real(it))
+            atomicOr(w, 1u << l16);
+        __syncwarp();
+        const uint32_t v = *reinterpret_cast<volatile uint32_t *>(w);
+        const uint32_t r = (v >> 16) + __popc(v & ltm);
+        __syncwarp();
+        if (real(it) && !(v & gtm))
+            *reinterpret_cast<volatile uint32_t *>(w) = (r + 1u) << 16;
+        __syncwarp();
+        if (it & 1)
+            rk[it >> 1] |= r << 16;
+        else
+            rk[it >> 1] = r;
+    }
 }
 
 // ---------------------------------------------------------------- keys

@@ -1656,7 +1656,6 @@ __global__ void __launch_bounds__(Lb8Cfg<KT, HASV, TILE, NW, OOP>::THREADS, Lb8C
     // ================================================================ ranking warps
     reg_inc<C::MAIN_REGS>();
     const int h = lane >> 4, l16 = lane & 15;
-    const uint32_t ltm = (1u << l16) - 1u, gtm = 0xFFFFu & ~((2u << l16) - 1u);
     uint32_t *row = tab + (2 * warp + h) * SIGMA; // this half-warp's words
     const uint32_t eh = uint32_t((2 * warp + h) * C::R + l16); // its first element in the tile
     auto dig = [&](KT key) -> uint32_t { return static_cast<uint32_t>(key >> a.shift) & 255u; };
@@ -1722,25 +1721,8 @@ __global__ void __launch_bounds__(Lb8Cfg<KT, HASV, TILE, NW, OOP>::THREADS, Lb8C
                     if (eh + it * 16 >= cnt)
                         key[it] = ~KT(0);
             }
-            // ---- stable rank within the half-warp: lanes with the same digit OR
-            // their bit into the digit's word and read it back; the last of them
-            // writes the new count (its rank + 1) with the lane bits cleared
-#pragma unroll
-            for (int it = 0; it < ITEMS; ++it) {
-                uint32_t *w = row + dig(key[it]);
-                atomicOr(w, 1u << l16);
-                __syncwarp();
-                const uint32_t v = *reinterpret_cast<volatile uint32_t *>(w);
-                const uint32_t r = (v >> 16) + __popc(v & ltm);
-                __syncwarp();
-                if (!(v & gtm))
-                    *reinterpret_cast<volatile uint32_t *>(w) = (r + 1u) << 16;
-                __syncwarp();
-                if (it & 1)
-                    rk[it >> 1] |= r << 16;
-                else
-                    rk[it >> 1] = r;
-            }
+            // ---- stable rank within the half-warp
+            rank_half_warp<ITEMS>(row, [&](int it) { return dig(key[it]); }, [](int) { return true; }, rk);
             named_bar(LB8_MAIN, NT);
 
             // ---- 2. tile counts per bucket, for the look-back warps, and their

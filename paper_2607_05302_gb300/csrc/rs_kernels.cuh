@@ -118,7 +118,7 @@ cudaError_t launch_small_sort(void *keys, uint32_t *vals, uint32_t n, int kb, bo
 // batched segmented sort of the small and medium segments
 constexpr uint32_t SEG_MED = 1u << 18;
 uint32_t seg_small_max(int db);
-uint32_t seg_med_ctas(uint32_t med_max, int kb, bool hasv, size_t budget);
+uint32_t seg_med_ctas(uint32_t med_max, int kb, bool hasv, int db, size_t budget);
 uint32_t seg_ip_ctas();
 // a long segment with an unaligned start, in the low-memory plan: its first
 // h < 4 elements set aside (save), the rest sorted, then merged back

@@ -16,6 +16,8 @@
 // processed by one persistent launch that takes segments from an atomic
 // work counter.  Nothing reads device memory on the host, so the whole call
 // is stream-ordered and can be captured in a CUDA graph.
+#include <type_traits>
+
 #include "rs_common.cuh"
 #include "rs_kernels.cuh"
 
@@ -219,7 +221,7 @@ template <int BYTES> __device__ __forceinline__ void cp_async_elem(void *smem, c
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
-// medium segments: out-of-place LSD between the segment and this CTA's
+// medium segments, 11-bit digits: out-of-place LSD between the segment and this CTA's
 // scratch region (Alg. 1 per digit), tile by tile.  Every digit's counts come
 // from one read of the segment; the next tile is copied into the second
 // buffer while the current one is ranked and stored.
@@ -341,6 +343,399 @@ __global__ void __launch_bounds__(SEG_T, 2) k_seg_medium(SegArgs a)
         }
         if (sk != keys + o) { // odd number of passes: the result is in the scratch
             for (uint32_t i = tid; i < len; i += SEG_T) {
+                keys[o + i] = sk[i];
+                if (HASV)
+                    a.vals[o + i] = svp[i];
+            }
+        }
+    }
+}
+
+// medium segments, 8-bit digits: out-of-place LSD between the segment and
+// this CTA's scratch region (Alg. 1 per digit) on one CTA of 16 warps per SM,
+// tile by tile.  What bounds it is shared memory, as in the 8-bit round
+// kernel, whose half-warp ranking and tile reorder it shares; the scratch
+// budget allows fewer CTAs than SMs when the longest segment is long, so each
+// CTA takes a whole SM and the largest tiles that two stages and the rank
+// words leave room for (two CTAs an SM on tiles of half the size sorted 10,000
+// arrays of 4,000 no faster).  The TMA engine copies a tile into one stage
+// while the other is worked on.  Tile starts are multiples of four elements of
+// the arrays (the first tile is up to three shorter), so that only a segment's
+// ends need plain loads.  A segment that fits the two stages stays there for
+// all rounds.  A digit that is the same in the whole segment costs no round.
+// Measured (u32 keys + index, ms, before: 8 warps a CTA, two CTAs an SM, tiles
+// of 4096): 306M elements in segments of 4097 to 2^18, 70 CTAs, 23.9 -> 14.8;
+// 4,000 segments of 10,000 1.34 -> 0.76; 2,000 of 40,000 3.53 -> 2.29; u64 keys
+// + index, 4,000 of 5,000, 2.57 -> 0.77.
+template <typename KT, bool HASV> struct MedCfg {
+    static constexpr int T = 512, NW = T / 32, NTD = int(sizeof(KT));
+    static constexpr int TILE = sizeof(KT) == 4 ? (HASV ? 8192 : 16384) : (HASV ? 6144 : 8192);
+    static constexpr int R = TILE / (2 * NW);  // elements per half-warp
+    static constexpr int ITEMS = R / 16;
+    static_assert(R % 16 == 0 && ITEMS % 2 == 0, "whole rows, an even number");
+    static constexpr bool PAIR = HASV && sizeof(KT) == 4;
+    static constexpr size_t al(size_t x) { return (x + 127) & ~size_t(127); }
+    static constexpr size_t KBYTES = al(size_t(TILE) * sizeof(KT) + 64) - 64; // values 64 past a multiple of 128
+    static constexpr size_t STAGE = al(KBYTES + (HASV ? size_t(TILE) * 4 : 0));
+    // both stages as one tile of 2 TILE elements
+    static constexpr size_t KBYTES2 = al(2 * size_t(TILE) * sizeof(KT) + 64) - 64;
+    static_assert(KBYTES2 + (HASV ? 2 * size_t(TILE) * 4 + 16 : 0) <= 2 * STAGE, "one tile in both stages");
+    static constexpr size_t o_tab = 2 * STAGE;                    // 2 NW x 256 words
+    static constexpr size_t o_gh = o_tab + size_t(2 * NW) * 256 * 4; // NTD x 256 counts
+    static constexpr size_t o_part = o_gh + size_t(NTD) * 256 * 4;   // 2 x 256
+    static constexpr size_t o_run = o_part + 2 * 256 * 4;         // 256: next output position per bucket
+    static constexpr size_t o_off = o_run + 256 * 4;              // 256: output position - tile position
+    static constexpr size_t o_wsum = o_off + 256 * 4;             // 8 words
+    static constexpr size_t o_bar = o_wsum + 32;                  // 2 mbarriers
+    static constexpr size_t SMEM = al(o_bar + 16);
+    static_assert(SMEM <= 227 * 1024, "shared memory budget");
+};
+
+template <typename KT, bool HASV>
+__global__ void __launch_bounds__(512, 1) k_seg_medium8(SegArgs a)
+{
+    using C = MedCfg<KT, HASV>;
+    constexpr int TILE = C::TILE, ITEMS = C::ITEMS, T = C::T, NTD = C::NTD, SI = TILE / T, U = 4;
+    static_assert(SI % U == 0, "whole batches");
+    extern __shared__ __align__(16) unsigned char sm[];
+    uint32_t *tab = reinterpret_cast<uint32_t *>(sm + C::o_tab);
+    uint32_t *gh = reinterpret_cast<uint32_t *>(sm + C::o_gh);
+    uint32_t *part = reinterpret_cast<uint32_t *>(sm + C::o_part);
+    uint32_t *run = reinterpret_cast<uint32_t *>(sm + C::o_run);
+    uint32_t *off = reinterpret_cast<uint32_t *>(sm + C::o_off);
+    uint32_t *wsum = reinterpret_cast<uint32_t *>(sm + C::o_wsum);
+    uint64_t *full = reinterpret_cast<uint64_t *>(sm + C::o_bar);
+    __shared__ uint32_t s_t;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, h = lane >> 4, l16 = lane & 15;
+    uint32_t *row = tab + (2 * warp + h) * 256;                  // this half-warp's words
+    const int c = tid & 255, p = tid >> 8;                       // the column passes' bucket and half of the rows
+    KT *keys = static_cast<KT *>(a.keys);
+    KT *sck = static_cast<KT *>(a.scr_k) + size_t(blockIdx.x) * a.med_stride;
+    uint32_t *scv = HASV ? a.scr_v + size_t(blockIdx.x) * a.med_stride : nullptr;
+    const uint32_t count = a.ctr[1];
+    if (tid == 0) {
+        mbar_init(&full[0], 1);
+        mbar_init(&full[1], 1);
+        fence_mbar_init();
+    }
+    for (int i = tid; i < 2 * C::NW * 256; i += T)
+        tab[i] = 0u;
+
+    // A tile in registers: ITEMS elements a thread, or (a segment that fits
+    // both stages) twice as many.
+    KT key[2 * ITEMS];
+    uint32_t val[HASV ? 2 * ITEMS : 1], rk[ITEMS];
+    // this thread's first element with N elements a thread
+    auto first = [&](int N) { return uint32_t((2 * warp + h) * N * 16 + l16); };
+    // keys at tk and values at tv, lead elements in, or (pairs) as reordered
+    // by an earlier round
+    auto load = [&]<int N>(std::integral_constant<int, N>, const KT *tk, const uint32_t *tv, uint32_t lead, bool pairs) {
+        const uint32_t eh = first(N);
+        if constexpr (C::PAIR) {
+            if (pairs) {
+                const uint2 *tp = reinterpret_cast<const uint2 *>(tk) + eh;
+#pragma unroll
+                for (int it = 0; it < N; ++it) {
+                    const uint2 x = tp[it * 16];
+                    key[it] = x.x;
+                    val[it] = x.y;
+                }
+                return;
+            }
+            // one half-warp reads keys while the other reads values
+            const uint32_t *p0 = (h ? tv : tk) + lead + eh, *p1 = (h ? tk : tv) + lead + eh;
+#pragma unroll
+            for (int it = 0; it < N; ++it) {
+                const uint32_t x = p0[it * 16], y = p1[it * 16];
+                key[it] = h ? y : x;
+                val[it] = h ? x : y;
+            }
+        } else {
+            const KT *pk = tk + lead + eh;
+            const uint32_t *pv = tv + lead + eh;
+#pragma unroll
+            for (int it = 0; it < N; it += 2) {
+                const KT x = pk[it * 16 + h * 16], y = pk[it * 16 + 16 - h * 16];
+                key[it] = h ? y : x;
+                key[it + 1] = h ? x : y;
+                if constexpr (HASV) {
+                    const uint32_t vx = pv[it * 16 + h * 16], vy = pv[it * 16 + 16 - h * 16];
+                    val[it] = h ? vy : vx;
+                    val[it + 1] = h ? vx : vy;
+                }
+            }
+        }
+    };
+    auto rank = [&]<int N>(std::integral_constant<int, N>, uint32_t cnt, uint32_t shift) {
+        const uint32_t eh = first(N);
+        auto digit = [&](int it) { return digit_of(key[it], shift, 255u); };
+        uint32_t(&r)[N / 2] = reinterpret_cast<uint32_t(&)[N / 2]>(rk);
+        if (cnt == uint32_t(N * T))
+            rank_half_warp<N>(row, digit, [](int) { return true; }, r);
+        else if (uint32_t(2 * warp) * N * 16 < cnt) // (else the warp has no element)
+            rank_half_warp<N>(row, digit, [&](int it) { return eh + it * 16 < cnt; }, r);
+    };
+    // Each half-warp's start per bucket in the reordered tile (the ranks'
+    // barrier before it and one after it included); f(start, count): bucket
+    // c's, once per bucket, before that last barrier.
+    auto columns = [&](auto &&after_ranks, auto &&f) {
+        __syncthreads();
+        after_ranks();
+        uint32_t *col = tab + p * C::NW * 256 + c;
+        uint32_t hc[C::NW / 2], sum = 0;
+#pragma unroll
+        for (int r = 0; r < C::NW; r += 2) {
+            const uint32_t x = col[r * 256] >> 16, y = col[(r + 1) * 256] & 0xFFFF0000u;
+            hc[r >> 1] = x | y;
+            sum += x + (y >> 16);
+        }
+        part[p * 256 + c] = sum;
+        __syncthreads();
+        const uint32_t other = part[(p ^ 1) * 256 + c], tot = sum + other;
+        const uint32_t inc = warp_incl_scan(tot);
+        if (lane == 31 && p == 0)
+            wsum[warp] = inc;
+        __syncthreads();
+        uint32_t base = inc - tot;
+#pragma unroll
+        for (int w = 0; w < 7; ++w)
+            base += w < (warp & 7) ? wsum[w] : 0u;
+        if (p == 0)
+            f(base, tot);
+        uint32_t pos = base + (p ? other : 0u);
+#pragma unroll
+        for (int r = 0; r < C::NW; ++r) {
+            col[r * 256] = pos;
+            pos += (r & 1) ? hc[r >> 1] >> 16 : hc[r >> 1] & 0xFFFFu;
+        }
+        __syncthreads();
+    };
+    // reorder in place (every element is in registers), and this warp's words
+    // cleared for the next tile
+    auto reorder = [&]<int N>(std::integral_constant<int, N>, KT *tk, uint32_t *tv, uint32_t cnt, uint32_t shift) {
+        const uint32_t eh = first(N);
+#pragma unroll
+        for (int it = 0; it < N; ++it) {
+            if (eh + it * 16 >= cnt)
+                continue;
+            const uint32_t pos =
+                row[digit_of(key[it], shift, 255u)] + ((it & 1) ? rk[it >> 1] >> 16 : rk[it >> 1] & 0xFFFFu);
+            if (pos >= cnt) { // only a broken scan gets here
+                set_status(ST_INTERNAL);
+                continue;
+            }
+            if constexpr (C::PAIR) {
+                reinterpret_cast<uint2 *>(tk)[pos] = make_uint2(static_cast<uint32_t>(key[it]), val[it]);
+            } else {
+                tk[pos] = key[it];
+                if (HASV)
+                    tv[pos] = val[it];
+            }
+        }
+        __syncwarp();
+        uint4 *z = reinterpret_cast<uint4 *>(tab + 2 * warp * 256);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            z[i * 32 + lane] = make_uint4(0u, 0u, 0u, 0u);
+        __syncthreads();
+    };
+    constexpr std::integral_constant<int, ITEMS> ONE{};
+    constexpr std::integral_constant<int, 2 * ITEMS> BOTH{};
+
+    uint32_t fill = 0; // tiles copied so far: fill f is in stage f % 2
+    for (;;) {
+        __syncthreads(); // every thread has read s_t and finished the last segment
+        if (tid == 0)
+            s_t = atomicAdd(&a.ctr[3], 1u);
+        __syncthreads();
+        const uint32_t t = s_t;
+        if (t >= count)
+            break;
+        const uint32_t sgi = a.med_list[t];
+        const unsigned long long o = a.off[sgi];
+        const unsigned long long len64 = a.off[sgi + 1] - o;
+        if (len64 > a.med_stride) { // the host sized the scratch from its offsets
+            if (tid == 0)
+                set_status(ST_INTERNAL);
+            continue;
+        }
+        const uint32_t len = static_cast<uint32_t>(len64);
+        KT *sk = keys + o, *dk = sck;
+        uint32_t *svp = HASV ? a.vals + o : nullptr, *dvp = scv;
+        // how far the segment and the scratch start past a multiple of four
+        // elements; m: the round's source
+        const uint32_t m_seg = static_cast<uint32_t>(o & 3u), m_scr = (blockIdx.x * a.med_stride) & 3u;
+        uint32_t m = m_seg;
+        // tile ti, elements [start, start of the next), into stage f % 2; one
+        // warp: the 16-byte-aligned middle by bulk copies, the segment's
+        // ragged ends by plain loads
+        auto start_of = [&](uint32_t ti) { return ti ? min(ti * TILE - m, len) : 0u; };
+        auto copy_in = [&](KT *tk, uint32_t *tv, uint32_t t0, uint32_t cnt, uint32_t lead, uint32_t f) {
+            auto side = [&](auto *dst, const auto *src, bool mine) {
+                using E = std::remove_reference_t<decltype(*dst)>;
+                const uintptr_t b0 = reinterpret_cast<uintptr_t>(src + t0), b1 = b0 + uintptr_t(cnt) * sizeof(E);
+                const uintptr_t m0 = (b0 + 15) & ~uintptr_t(15), m1 = b1 & ~uintptr_t(15);
+                const uint32_t head = m0 < m1 ? uint32_t((m0 - b0) / sizeof(E)) : cnt;
+                const uint32_t tail = m0 < m1 ? uint32_t((m1 - b0) / sizeof(E)) : cnt;
+                if (mine && tail > head) {
+                    asm volatile("mbarrier.expect_tx.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&full[f & 1u])),
+                                 "r"((tail - head) * uint32_t(sizeof(E)))
+                                 : "memory");
+                    bulk_g2s(dst + lead + head, reinterpret_cast<const void *>(m0),
+                             (tail - head) * uint32_t(sizeof(E)), &full[f & 1u]);
+                }
+                for (uint32_t e = lane; e < head; e += 32)
+                    dst[lead + e] = src[t0 + e];
+                for (uint32_t e = tail + lane; e < cnt; e += 32)
+                    dst[lead + e] = src[t0 + e];
+            };
+            side(tk, sk, lane == 0);
+            if (HASV)
+                side(tv, svp, lane == 1);
+            __syncwarp();
+            if (lane == 0)
+                mbar_arrive(&full[f & 1u]); // release: the plain stores above are visible
+        };
+        auto stage_k = [&](uint32_t f) { return reinterpret_cast<KT *>(sm + (f & 1u) * C::STAGE); };
+        auto stage_v = [&](uint32_t f) { return reinterpret_cast<uint32_t *>(sm + (f & 1u) * C::STAGE + C::KBYTES); };
+        auto issue = [&](uint32_t ti, uint32_t f) {
+            copy_in(stage_k(f), stage_v(f), start_of(ti), start_of(ti + 1) - start_of(ti), ti ? 0u : m, f);
+        };
+        if (len + m <= uint32_t(2 * TILE)) {
+            // ---- one tile, or both stages as one: every round in place
+            KT *tk = reinterpret_cast<KT *>(sm);
+            uint32_t *tv = reinterpret_cast<uint32_t *>(sm + C::KBYTES2);
+            auto rounds = [&](auto n) {
+                if (warp == 0)
+                    copy_in(tk, tv, 0u, len, m, fill);
+                (void)mbar_wait(&full[fill & 1u], (fill >> 1) & 1u);
+                __syncwarp();
+                for (uint32_t shift = 0; shift < 8u * NTD; shift += 8) {
+                    load(n, tk, tv, shift ? 0u : m, shift != 0);
+                    rank(n, len, shift);
+                    columns([] {}, [](uint32_t, uint32_t) {});
+                    reorder(n, tk, tv, len, shift);
+                }
+            };
+            if (len + m <= uint32_t(TILE))
+                rounds(ONE);
+            else
+                rounds(BOTH);
+            for (uint32_t i = tid; i < len; i += T) {
+                if constexpr (C::PAIR) {
+                    const uint2 x = reinterpret_cast<const uint2 *>(tk)[i];
+                    sk[i] = x.x;
+                    svp[i] = x.y;
+                } else {
+                    sk[i] = tk[i];
+                    if (HASV)
+                        svp[i] = tv[i];
+                }
+            }
+            fence_proxy_async_smem();
+            ++fill;
+            continue;
+        }
+        // every digit's counts in one pass: the multiset is the same in every round
+        for (int i = tid; i < NTD * 256; i += T)
+            gh[i] = 0;
+        __syncthreads();
+#pragma unroll 4
+        for (uint32_t i = tid; i < len; i += T) {
+            const KT k = sk[i];
+#pragma unroll
+            for (int r = 0; r < NTD; ++r)
+                atomicAdd(&gh[r * 256 + digit_of(k, uint32_t(r * 8), 255u)], 1u);
+        }
+        __syncthreads();
+        for (uint32_t shift = 0; shift < 8u * NTD; shift += 8) {
+            // bucket starts in the segment
+            const uint32_t cnt_c = p == 0 ? gh[shift * 32 + c] : 0u;
+            const uint32_t inc0 = warp_incl_scan(cnt_c);
+            if (p == 0 && lane == 31)
+                wsum[warp] = inc0;
+            if (__syncthreads_or(p == 0 && cnt_c == len))
+                continue; // one digit: the round is the identity
+            if (p == 0) {
+                uint32_t s0 = inc0 - cnt_c;
+#pragma unroll
+                for (int w = 0; w < 7; ++w)
+                    s0 += w < warp ? wsum[w] : 0u;
+                run[c] = s0;
+            }
+            const uint32_t ntile = (len + m + TILE - 1) / TILE;
+            if (warp == 0)
+                issue(0, fill);
+            for (uint32_t ti = 0; ti < ntile; ++ti, ++fill) {
+                const uint32_t cnt = start_of(ti + 1) - start_of(ti);
+                KT *tk = stage_k(fill);
+                uint32_t *tv = stage_v(fill);
+                // (a wait that runs out is reported; the tile is then worked
+                // through with what is there)
+                (void)mbar_wait(&full[fill & 1u], (fill >> 1) & 1u);
+                __syncwarp();
+                load(ONE, tk, tv, ti ? 0u : m, false);
+                rank(ONE, cnt, shift);
+                columns(
+                    [&] { // the tile before is stored: its stage is free
+                        if (warp == T / 32 - 1 && ti + 1 < ntile)
+                            issue(ti + 1, fill + 1);
+                    },
+                    [&](uint32_t base, uint32_t tot) {
+                        const uint32_t g = run[c];
+                        off[c] = g - base;
+                        run[c] = g + tot;
+                    });
+                reorder(ONE, tk, tv, cnt, shift);
+                // ---- store every bucket run
+#pragma unroll 1
+                for (int k0 = 0; k0 < SI; k0 += U) {
+                    KT kv[U];
+                    uint32_t vv[U], dst[U];
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const uint32_t i = tid + (k0 + u) * T;
+                        if constexpr (C::PAIR) {
+                            const uint2 pr = reinterpret_cast<const uint2 *>(tk)[i];
+                            kv[u] = pr.x;
+                            vv[u] = pr.y;
+                        } else {
+                            kv[u] = tk[i];
+                            vv[u] = HASV ? tv[i] : 0u;
+                        }
+                    }
+#pragma unroll
+                    for (int u = 0; u < U; ++u)
+                        dst[u] = tid + (k0 + u) * T + off[digit_of(kv[u], shift, 255u)];
+#pragma unroll
+                    for (int u = 0; u < U; ++u)
+                        if (tid + (k0 + u) * T < cnt) {
+                            if (dst[u] >= len) { // only inconsistent counts get here
+                                set_status(ST_INTERNAL);
+                                continue;
+                            }
+                            dk[dst[u]] = kv[u];
+                            if (HASV)
+                                dvp[dst[u]] = vv[u];
+                        }
+                }
+                // the stage was read and written with generic accesses; it is
+                // refilled with bulk copies (async proxy)
+                fence_proxy_async_smem();
+            }
+            // the round's stores precede the next round's bulk copies
+            fence_proxy_async_all();
+            __syncthreads();
+            KT *tkp = sk;
+            sk = dk;
+            dk = tkp;
+            uint32_t *tvp = svp;
+            svp = dvp;
+            dvp = tvp;
+            m = m_seg + m_scr - m;
+        }
+        if (sk != keys + o) { // odd number of passes: the result is in the scratch
+            for (uint32_t i = tid; i < len; i += T) {
                 keys[o + i] = sk[i];
                 if (HASV)
                     a.vals[o + i] = svp[i];
@@ -1072,13 +1467,17 @@ template <typename KT, bool HASV, int DB> struct SegImpl {
         const cudaError_t ea = attr.run([] {
             cudaError_t e = cudaFuncSetAttribute(k_seg_small<KT, HASV, DB, SMALL>,
                                                  cudaFuncAttributeMaxDynamicSharedMemorySize, int(small_smem()));
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(k_seg_medium<KT, HASV, DB, TILE>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, int(med_smem()));
-            if constexpr (DB == 8)
+            if constexpr (DB == 8) {
+                if (e == cudaSuccess)
+                    e = cudaFuncSetAttribute(k_seg_medium8<KT, HASV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             int(MedCfg<KT, HASV>::SMEM));
                 if (e == cudaSuccess)
                     e = cudaFuncSetAttribute(k_seg_medium_ip<KT, HASV, IP_TILE>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, int(IC::SMEM));
+            } else if (e == cudaSuccess) {
+                e = cudaFuncSetAttribute(k_seg_medium<KT, HASV, DB, TILE>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, int(med_smem()));
+            }
             return e;
         });
         if (ea != cudaSuccess)
@@ -1094,7 +1493,10 @@ template <typename KT, bool HASV, int DB> struct SegImpl {
             else
                 return cudaErrorInvalidValue; // the planner picks it for 8-bit digits only
         } else if (a.med_stride) {
-            k_seg_medium<KT, HASV, DB, TILE><<<med_ctas, SEG_T, med_smem(), st>>>(a);
+            if constexpr (DB == 8)
+                k_seg_medium8<KT, HASV><<<med_ctas, MedCfg<KT, HASV>::T, MedCfg<KT, HASV>::SMEM, st>>>(a);
+            else
+                k_seg_medium<KT, HASV, DB, TILE><<<med_ctas, SEG_T, med_smem(), st>>>(a);
         }
         g_launches += 2;
         return cudaGetLastError();
@@ -1103,11 +1505,11 @@ template <typename KT, bool HASV, int DB> struct SegImpl {
 
 uint32_t seg_small_max(int db) { return db <= 8 ? 4096u : 2048u; }
 
-// CTAs of the medium pass: two per SM, fewer when their scratch (med_max
-// elements each) would pass `budget` bytes, at least 16
-uint32_t seg_med_ctas(uint32_t med_max, int kb, bool hasv, size_t budget)
+// CTAs of the medium pass: one per SM (8-bit digits) or two, fewer when their
+// scratch (med_max elements each) would pass `budget` bytes, at least 16
+uint32_t seg_med_ctas(uint32_t med_max, int kb, bool hasv, int db, size_t budget)
 {
-    const uint32_t most = static_cast<uint32_t>(num_sms()) * 2;
+    const uint32_t most = static_cast<uint32_t>(num_sms()) * (db == 8 ? 1 : 2);
     if (!med_max)
         return 0;
     const size_t per = size_t(med_max) * (kb + (hasv ? 4 : 0));

@@ -131,7 +131,6 @@ __global__ void __launch_bounds__(SM_T) k_small_sort(KT *keys, uint32_t *vals, u
         tab[i] = 0u;
     __syncthreads();
 
-    const uint32_t ltm = (1u << l16) - 1u, gtm = 0xFFFFu & ~((2u << l16) - 1u);
     uint32_t *row = tab + (2 * warp + h) * 256;
     const uint32_t eh = uint32_t((2 * warp + h) * C::R + l16);
     const int c = tid & 255, p = tid >> 8; // the column passes' bucket and half of the rows
@@ -155,24 +154,8 @@ __global__ void __launch_bounds__(SM_T) k_small_sort(KT *keys, uint32_t *vals, u
                     val[it] = reinterpret_cast<const uint32_t *>(src + C::KB)[e];
             }
         }
-#pragma unroll
-        for (int it = 0; it < ITEMS; ++it) {
-            const bool real = eh + it * 16 < cnt;
-            uint32_t *w = row + digit_of(key[it], shift, 255u);
-            if (real)
-                atomicOr(w, 1u << l16);
-            __syncwarp();
-            const uint32_t v = *reinterpret_cast<volatile uint32_t *>(w);
-            const uint32_t r = (v >> 16) + __popc(v & ltm);
-            __syncwarp();
-            if (real && !(v & gtm))
-                *reinterpret_cast<volatile uint32_t *>(w) = (r + 1u) << 16;
-            __syncwarp();
-            if (it & 1)
-                rk[it >> 1] |= r << 16;
-            else
-                rk[it >> 1] = r;
-        }
+        rank_half_warp<ITEMS>(row, [&](int it) { return digit_of(key[it], shift, 255u); },
+                              [&](int it) { return eh + it * 16 < cnt; }, rk);
         __syncthreads();
         // ---- 2. the CTA's counts per digit, and their exchange
         uint32_t *col = tab + p * (SM_ROWS / 2) * 256 + c;
