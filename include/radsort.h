@@ -280,16 +280,20 @@ radsort_status radsort_lsd_oop_scratch_size(size_t n, int key_bytes, int value_b
  * kernels); offsets_host the same values on the host (used to plan the long
  * segments).  Segments up to 4096 elements (2048 for 11-bit digits) are sorted
  * in shared memory.  Segments up to 2^18 elements are sorted out of place in
- * per-CTA scratch as long as the longest of them (at most 2 CTAs per SM, held
- * to 6% of the arrays' bytes), the paper's suggestion of reusing T as the A'
- * of Alg. 1 for short arrays (Sec. 5).
+ * per-CTA scratch as long as the longest of them (at most one CTA per SM, 2
+ * with 11-bit digits, held to 6% of the arrays' bytes), the paper's suggestion
+ * of reusing T as the A' of Alg. 1 for short arrays (Sec. 5); with 8-bit
+ * digits, those that fit two tiles (16384 u32 pairs) never leave shared memory.
  * Both classes are handled by one persistent launch each.  Longer segments
  * run the full Radsort (Alg. 2), or Alg. 1 with alternate buffers in the
- * workspace when their start is not 16-byte aligned; they are spread, longest
- * first, over up to 4 library-owned streams (created on the first call that
- * has long segments on a device) that start after the work already on
- * `stream` and that `stream` waits for, each with its own part of the
- * workspace.  workspace: at least radsort_segmented_workspace_size() bytes,
+ * workspace when their start is not 16-byte aligned.  With 8-bit digits those
+ * that fit the workspace's alternate buffers together go out of place in
+ * groups of up to 64, one launch per digit for a group; so do a few medium
+ * segments (longer than 16384) where that takes no more workspace.  The others
+ * are spread, longest first, over up to 4 library-owned streams (created on
+ * the first call that has long segments on a device) that start after the
+ * work already on `stream` and that `stream` waits for, each with its own part
+ * of the workspace.  workspace: at least radsort_segmented_workspace_size() bytes,
  * or NULL to allocate stream-ordered.  With 8-bit digits a smaller caller
  * workspace, down to radsort_segmented_workspace_size_min() bytes, selects
  * the fastest of two low-memory plans that fits: (1) the medium segments
@@ -301,8 +305,8 @@ radsort_status radsort_lsd_oop_scratch_size(size_t n, int key_bytes, int value_b
  * aligned has its first (at most 3) elements set aside, the rest sorted by
  * Radsort and those elements merged back, instead of the alternate buffers.
  * On 20,000 lognormal arrays (2^29 keys + values) the plans hold 9%, 3.4%
- * and 0.95% of the arrays' bytes; (1) and (2) run about 30% slower than the
- * fastest plan.  With a caller workspace the call
+ * and 0.95% of the arrays' bytes; (1) and (2) run at about half the fastest
+ * plan's speed.  With a caller workspace the call
  * issues only kernel launches, memsets and event records / waits, so it can
  * be captured in a CUDA graph (make a first call with long segments before
  * capturing, so that the streams exist).  Calls from several host threads

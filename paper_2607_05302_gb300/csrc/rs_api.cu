@@ -953,15 +953,20 @@ constexpr int SEG_STREAMS_ALT = 4;
 // 14%) -> 20.7.  The low-memory plan (8-bit digits) sorts the medium
 // segments in place instead, in a fixed 514 blocks of 32 elements per CTA.
 constexpr double SEG_MED_SHARE = 0.06;
+// few medium segments: those longer than SEG_LOW join the long ones when the
+// longest has at least SEG_FEW elements
+constexpr uint32_t SEG_LOW = 16384, SEG_FEW = 65536;
 
 struct SegPlan {
     size_t base = 0;    // classify lists + medium scratch
     size_t large = 0;   // workspace of one long-segment stream
     size_t total = 0;   // base + nstr * large
     uint32_t med_max = 0, med_ctas = 0;
+    uint32_t med_lim = SEG_MED; // segments longer than this are long ones
     bool ip = false;    // medium segments in place (level >= 1)
     int level = 0;      // see seg_plan
-    int nstr = 0;       // internal streams used (0: no long segment)
+    int nstr = 0;       // slices for long segments, and internal streams used (0: no long segment)
+    bool fork = false;  // the internal streams are used
 };
 
 // oop: long segments sorted out of place (Alg. 1) into the caller's
@@ -974,7 +979,9 @@ radsort_status seg_plan(const uint64_t *offh, size_t nseg, int kb, bool hasv, in
                         SegPlan *sp)
 {
     size_t large = 0, nlong = 0, nmed = 0;
-    uint32_t med_max = 0;
+    uint32_t med_max = 0, low_max = 0; // longest medium segment, and of those up to SEG_LOW
+    SegGroup few{};                    // the medium segments longer than SEG_LOW
+    bool is_few = level == 0 && !oop && db == 8;
     const uint32_t small_max = seg_small_max(db);
     const size_t n = nseg ? offh[nseg] - offh[0] : 0;
     for (size_t s = 0; s < nseg; ++s) {
@@ -986,6 +993,15 @@ radsort_status seg_plan(const uint64_t *offh, size_t nseg, int kb, bool hasv, in
                 ++nmed;
                 if (len > med_max)
                     med_max = static_cast<uint32_t>(len);
+                if (len <= SEG_LOW) {
+                    if (len > low_max)
+                        low_max = static_cast<uint32_t>(len);
+                } else if (few.narr < SEG_GROUP) {
+                    few.off[few.narr] = offh[s];
+                    few.len[few.narr++] = static_cast<uint32_t>(len);
+                } else {
+                    is_few = false;
+                }
             }
             continue;
         }
@@ -1031,7 +1047,31 @@ radsort_status seg_plan(const uint64_t *offh, size_t nseg, int kb, bool hasv, in
     sp->large = large;
     const size_t smax = sp->level >= 2 ? size_t(SEG_STREAMS) : size_t(SEG_STREAMS_ALT);
     sp->nstr = static_cast<int>(nlong < smax ? nlong : smax);
-    sp->total = sp->base + size_t(sp->nstr) * large;
+    sp->fork = nlong != 0;
+    // A few medium segments would each hold one CTA while most SMs idle: where
+    // alternate arrays for all of them take no more than the scratch of those
+    // CTAs (and 1 MiB), they are sorted together with the long ones, by every SM.  Below
+    // SEG_FEW elements a CTA is done as soon (a group waits for 3 + n_t
+    // launches, 80-100 us with 4-byte keys; a CTA takes 3 ns an element).
+    // Measured: 24 segments of 2^10 to 2^20 u64 keys + index, 2.3M elements,
+    // 1.21 -> 0.24 ms; one of 200,000 u32 keys + index 0.55 -> 0.10.
+    if (is_few && few.narr && med_max >= SEG_FEW) {
+        const uint32_t lctas = seg_med_ctas(low_max, kb, hasv, db,
+                                            static_cast<size_t>(SEG_MED_SHARE * double(n) * (kb + (hasv ? 4 : 0))));
+        const size_t lbase = (seg_scratch_bytes(kb, hasv, nseg, low_max, lctas, false) + 255) / 256 * 256;
+        const int str = sp->nstr ? sp->nstr : 1;
+        const size_t each = (lsd_group_bytes(few, kb, hasv) / str + 256) / 256 * 256;
+        const size_t lg = each > large ? each : large;
+        if (lbase + str * lg <= sp->base + sp->nstr * large + (size_t(1) << 20)) {
+            sp->base = lbase;
+            sp->large = lg;
+            sp->nstr = str;
+            sp->med_max = low_max;
+            sp->med_ctas = lctas;
+            sp->med_lim = SEG_LOW;
+        }
+    }
+    sp->total = sp->base + size_t(sp->nstr) * sp->large;
     return RADSORT_OK;
 }
 
@@ -1068,24 +1108,36 @@ radsort_status seg_streams(SegStreams **out)
 
 // Enqueues main() on st (the short and medium segments) and sorts the long
 // segments beside it: each goes, longest first, to the internal stream with
-// the fewest elements so far; sort_one(offset, length, slice, stream).  The
+// the fewest elements so far; sort_one(offset, length, slice, stream).
+// together(segments, stream): sorts some of them in groups through the whole
+// long-segment workspace on that stream, takes those off the list and returns
+// whether there were any; the others then follow on the same stream.  The
 // internal streams start after the work already on st (so the workspace is
 // free), and st waits for them at the end.
-template <typename M, typename F>
+template <typename M, typename G, typename F>
 radsort_status seg_run(const uint64_t *offh, size_t nseg, const SegPlan &sp, char *lw, cudaStream_t st,
-                       M &&main, F &&sort_one)
+                       M &&main, G &&together, F &&sort_one)
 {
     if (sp.nstr == 0)
         return main();
     std::vector<uint32_t> idx;
     for (size_t s = 0; s < nseg; ++s)
-        if (offh[s + 1] - offh[s] > SEG_MED)
+        if (offh[s + 1] - offh[s] > sp.med_lim)
             idx.push_back(static_cast<uint32_t>(s));
     std::stable_sort(idx.begin(), idx.end(), [&](uint32_t x, uint32_t y) {
         return offh[x + 1] - offh[x] > offh[y + 1] - offh[y];
     });
+    radsort_status rs = RADSORT_OK;
+    if (!sp.fork) { // a few medium segments in a group: on st itself
+        rs = main();
+        if (rs == RADSORT_OK)
+            (void)together(idx, st, &rs);
+        for (size_t i = 0; i < idx.size() && rs == RADSORT_OK; ++i)
+            rs = sort_one(offh[idx[i]], offh[idx[i] + 1] - offh[idx[i]], lw, st);
+        return rs;
+    }
     SegStreams *ss = nullptr;
-    radsort_status rs = seg_streams(&ss);
+    rs = seg_streams(&ss);
     if (rs != RADSORT_OK)
         return rs;
     std::lock_guard<std::mutex> lk(g_seg_mu);
@@ -1095,12 +1147,15 @@ radsort_status seg_run(const uint64_t *offh, size_t nseg, const SegPlan &sp, cha
     if (e != cudaSuccess)
         return cuda_status(e);
     rs = main();
+    int nstr = sp.nstr;
+    if (rs == RADSORT_OK && together(idx, ss->s[0], &rs))
+        nstr = 1;
     unsigned long long load[SEG_STREAMS] = {};
     for (uint32_t sg : idx) {
         if (rs != RADSORT_OK)
             break;
         int best = 0;
-        for (int i = 1; i < sp.nstr; ++i)
+        for (int i = 1; i < nstr; ++i)
             if (load[i] < load[best])
                 best = i;
         const size_t off = offh[sg], len = offh[sg + 1] - off;
@@ -1116,6 +1171,51 @@ radsort_status seg_run(const uint64_t *offh, size_t nseg, const SegPlan &sp, cha
             rs = cuda_status(ej);
     }
     return rs;
+}
+
+// Sorts the long segments of idx (longest first) that fit the pool in groups,
+// out of place through alternate arrays there, one launch per round for a
+// group: a segment of 2^18 to 2^22 elements alone leaves most SMs idle and
+// waits for every launch (measured, u32 keys + index, 372 of them, 239M
+// elements: 12.0 ms one by one on four streams, 6.0 in 15 groups).  Takes
+// them off the list; false if none fits.
+bool seg_groups(void *keys, uint32_t *values, const uint64_t *offh, std::vector<uint32_t> &idx, int kb, char *pool,
+                size_t pool_bytes, cudaStream_t st, radsort_status *rs)
+{
+    std::vector<uint32_t> rest;
+    SegGroup g{};
+    bool any = false;
+    auto flush = [&]() {
+        if (g.narr && *rs == RADSORT_OK)
+            *rs = cuda_status(launch_lsd_group(keys, values, g, kb, pool, st));
+        any |= g.narr != 0;
+        g.narr = 0;
+    };
+    auto add = [&](uint32_t sg) { // into the present group, if it fits
+        if (g.narr == SEG_GROUP)
+            return false;
+        g.off[g.narr] = offh[sg];
+        g.len[g.narr] = static_cast<uint32_t>(offh[sg + 1] - offh[sg]);
+        ++g.narr;
+        if (lsd_group_bytes(g, kb, values != nullptr) <= pool_bytes)
+            return true;
+        --g.narr;
+        return false;
+    };
+    for (uint32_t sg : idx) {
+        if (offh[sg + 1] - offh[sg] >= (uint64_t(1) << 31)) {
+            rest.push_back(sg);
+            continue;
+        }
+        if (add(sg))
+            continue;
+        flush();
+        if (!add(sg))
+            rest.push_back(sg);
+    }
+    flush();
+    idx.swap(rest);
+    return any;
 }
 
 // the caller's workspace, or one allocated stream-ordered
@@ -1205,10 +1305,15 @@ radsort_status radsort_sort_segmented(void *keys, uint32_t *values, const uint64
         return s;
     auto main = [&]() -> radsort_status {
         return cuda_status(launch_segmented(keys, values, reinterpret_cast<const unsigned long long *>(offsets_dev),
-                                            num_segments, key_bytes, digit_bits, sp.med_max, sp.med_ctas, sp.ip, ws,
+                                            num_segments, key_bytes, digit_bits, sp.med_max, sp.med_ctas, sp.med_lim, sp.ip, ws,
                                             st));
     };
     radsort_status rs = seg_run(offsets_host, num_segments, sp, static_cast<char *>(ws) + sp.base, st, main,
+                      [&](std::vector<uint32_t> &idx, cudaStream_t ls, radsort_status *r) {
+                          return sp.level == 0 && digit_bits == 8 &&
+                                 seg_groups(keys, values, offsets_host, idx, key_bytes,
+                                            static_cast<char *>(ws) + sp.base, size_t(sp.nstr) * sp.large, ls, r);
+                      },
                       [&](size_t off, size_t len, char *lw, cudaStream_t ls) -> radsort_status {
                           char *sk = static_cast<char *>(keys) + off * key_bytes;
                           uint32_t *sv = hasv ? values + off : nullptr;
@@ -1361,10 +1466,11 @@ radsort_status radsort_lsd_oop_sort_segmented(void *keys, uint32_t *values, void
         return s;
     auto main = [&]() -> radsort_status {
         return cuda_status(launch_segmented(keys, values, reinterpret_cast<const unsigned long long *>(offsets_dev),
-                                            num_segments, key_bytes, digit_bits, sp.med_max, sp.med_ctas, sp.ip, ws,
+                                            num_segments, key_bytes, digit_bits, sp.med_max, sp.med_ctas, sp.med_lim, sp.ip, ws,
                                             st));
     };
     radsort_status rs = seg_run(offsets_host, num_segments, sp, static_cast<char *>(ws) + sp.base, st, main,
+                      [](std::vector<uint32_t> &, cudaStream_t, radsort_status *) { return false; },
                       [&](size_t off, size_t len, char *lw, cudaStream_t ls) -> radsort_status {
                           char *sk = static_cast<char *>(keys) + off * key_bytes;
                           char *ak = static_cast<char *>(keys_alt) + off * key_bytes;

@@ -1286,10 +1286,22 @@ template <int N> __device__ __forceinline__ void reg_inc()
 // named barriers of k_lb_round8
 enum { LB8_MAIN = 1, LB8_AUX = 2, LB8_CNT = 3, LB8_SCAN = 4, LB8_LIST = 5, LB8_FREE = 6 };
 
-template <typename KT, bool HASV, int TILE, int NW, bool OOP>
+// Several arrays sorted out of place in one launch per round (GRP): their
+// tiles follow one another, array by array, and the first tile of each has the
+// prefix 0, where its other tiles' look-back ends.
+struct LbGroup {
+    uint32_t narr;
+    uint32_t tile0[SEG_GROUP];                 // first tile
+    uint32_t len[SEG_GROUP];
+    unsigned long long in[SEG_GROUP], out[SEG_GROUP]; // first element in ik / iv and in ok / ov
+};
+struct LbNoGroup {};
+
+template <typename KT, bool HASV, int TILE, int NW, bool OOP, bool GRP = false>
 __global__ void __launch_bounds__(Lb8Cfg<KT, HASV, TILE, NW, OOP>::THREADS, Lb8Cfg<KT, HASV, TILE, NW, OOP>::MINB)
-    k_lb_round8(LbArgs<KT> a)
+    k_lb_round8(LbArgs<KT> a, const __grid_constant__ std::conditional_t<GRP, LbGroup, LbNoGroup> grp)
 {
+    static_assert(OOP || !GRP, "groups go out of place");
     using C = Lb8Cfg<KT, HASV, TILE, NW, OOP>;
     constexpr int SIGMA = C::SIGMA, NT = C::NT, ITEMS = C::ITEMS;
     extern __shared__ __align__(128) unsigned char sm[];
@@ -1315,8 +1327,9 @@ __global__ void __launch_bounds__(Lb8Cfg<KT, HASV, TILE, NW, OOP>::THREADS, Lb8C
         misc[0] = misc[1] = 0;
         fence_mbar_init();
     }
-    for (int c = tid; c < (OOP ? SIGMA + 1 : 3 * SIGMA + 1); c += C::THREADS)
-        sO[c] = a.tab[c];
+    if constexpr (!GRP)
+        for (int c = tid; c < (OOP ? SIGMA + 1 : 3 * SIGMA + 1); c += C::THREADS)
+            sO[c] = a.tab[c];
     for (int i = tid; i < C::SROWS * SIGMA; i += C::THREADS)
         tab[i] = 0u;
     __syncthreads();
@@ -1382,13 +1395,26 @@ __global__ void __launch_bounds__(Lb8Cfg<KT, HASV, TILE, NW, OOP>::THREADS, Lb8C
             unsigned char *st = sm + size_t(s) * C::STAGE;
             KT *stk = reinterpret_cast<KT *>(st);
             uint32_t *stv = reinterpret_cast<uint32_t *>(st + C::KBYTES);
-            const uint32_t e0 = ft * uint32_t(TILE);
-            const uint32_t cnt = min(uint32_t(TILE), a.n - e0);
+            uint32_t e0 = ft * uint32_t(TILE), n = a.n, arr = 0; // of a group: in array arr
+            const KT *ik = a.ik;
+            const uint32_t *iv = a.iv;
+            if constexpr (GRP) {
+                unsigned before = 0; // arrays that begin at or before tile ft
+#pragma unroll
+                for (uint32_t j = 0; j < SEG_GROUP; j += 32)
+                    before += __popc(__ballot_sync(0xffffffffu, j + lane < grp.narr && grp.tile0[j + lane] <= ft));
+                arr = before - 1;
+                e0 = (ft - grp.tile0[arr]) * uint32_t(TILE);
+                n = grp.len[arr];
+                ik += grp.in[arr];
+                iv += HASV ? grp.in[arr] : 0;
+            }
+            const uint32_t cnt = min(uint32_t(TILE), n - e0);
             uint32_t leadk = 0, leadv = 0;
             if constexpr (OOP) {
                 // the 16-byte-aligned middle by bulk copies, the ragged ends
                 // (under 16 bytes each) by plain loads
-                const uintptr_t ka = reinterpret_cast<uintptr_t>(a.ik + e0);
+                const uintptr_t ka = reinterpret_cast<uintptr_t>(ik + e0);
                 const uintptr_t kz = ka + uintptr_t(cnt) * sizeof(KT);
                 const uintptr_t ka16 = (ka + 15) & ~uintptr_t(15), kz16 = kz & ~uintptr_t(15);
                 leadk = static_cast<uint32_t>((ka & 15) / sizeof(KT));
@@ -1400,7 +1426,7 @@ __global__ void __launch_bounds__(Lb8Cfg<KT, HASV, TILE, NW, OOP>::THREADS, Lb8C
                 uint32_t vhead = 0, vtail = 0;
                 bool vmid = false;
                 if (HASV) {
-                    const uintptr_t va = reinterpret_cast<uintptr_t>(a.iv + e0);
+                    const uintptr_t va = reinterpret_cast<uintptr_t>(iv + e0);
                     const uintptr_t vz = va + uintptr_t(cnt) * 4;
                     va16 = (va + 15) & ~uintptr_t(15);
                     vz16 = vz & ~uintptr_t(15);
@@ -1422,14 +1448,14 @@ __global__ void __launch_bounds__(Lb8Cfg<KT, HASV, TILE, NW, OOP>::THREADS, Lb8C
                     bulk_g2s(stv + leadv + vhead, reinterpret_cast<const void *>(va16),
                              static_cast<uint32_t>(vz16 - va16), &full[s]);
                 for (uint32_t e = lane; e < khead; e += 32)
-                    stk[leadk + e] = a.ik[e0 + e];
+                    stk[leadk + e] = ik[e0 + e];
                 for (uint32_t e = ktail + lane; e < cnt; e += 32)
-                    stk[leadk + e] = a.ik[e0 + e];
+                    stk[leadk + e] = ik[e0 + e];
                 if (HASV) {
                     for (uint32_t e = lane; e < vhead; e += 32)
-                        stv[leadv + e] = a.iv[e0 + e];
+                        stv[leadv + e] = iv[e0 + e];
                     for (uint32_t e = vtail + lane; e < cnt; e += 32)
-                        stv[leadv + e] = a.iv[e0 + e];
+                        stv[leadv + e] = iv[e0 + e];
                 }
             } else {
                 // blocks ft*M .. of the logical data: block i at stage offset
@@ -1468,8 +1494,8 @@ __global__ void __launch_bounds__(Lb8Cfg<KT, HASV, TILE, NW, OOP>::THREADS, Lb8C
             if (lane == 0) {
                 mt[0] = ft;
                 mt[1] = cnt;
-                mt[2] = leadk;
-                mt[3] = leadv;
+                mt[2] = leadk | (leadv << 8);
+                mt[3] = arr;
             }
             __syncwarp();
             if (lane == 0)
@@ -1504,7 +1530,8 @@ __global__ void __launch_bounds__(Lb8Cfg<KT, HASV, TILE, NW, OOP>::THREADS, Lb8C
         reg_dec<C::AUX_REGS>();
         const int c = tid - NT, aw = warp - NW; // this thread's bucket, its warp among the 8
         const uint32_t *ns0 = sO + SIGMA + 1, *ns1 = ns0 + SIGMA;
-        const uint32_t Oc = sO[c], Oe = sO[c + 1];
+        uint32_t Oc = GRP ? 0u : sO[c];
+        const uint32_t Oe = GRP ? 0u : sO[c + 1];
         const uint32_t n0 = OOP ? 0u : ns0[c], n1 = OOP ? 0u : ns1[c];
         const uint32_t nP = OOP ? 0u : a.hdr[TAB_TAKEN]; // free-list entries taken before the round
         auto kaddr = [&](uint32_t blk) -> KT * {
@@ -1522,15 +1549,21 @@ __global__ void __launch_bounds__(Lb8Cfg<KT, HASV, TILE, NW, OOP>::THREADS, Lb8C
             if (t == TILE_END)
                 break;
             const uint32_t cnt = meta[(k % C::STAGES) * 4 + 1];
+            uint32_t t_first = 0, arr = 0; // the array's first tile
+            if constexpr (GRP) {
+                arr = meta[(k % C::STAGES) * 4 + 3];
+                t_first = grp.tile0[arr];
+                Oc = __ldg(a.tab + size_t(arr) * (SIGMA + 1) + c);
+            }
             // elements past the tile's end were ranked as digit 255
             uint32_t cn = part[c] + (C::PARTS == 2 ? part[SIGMA + c] : 0u);
             if (c == SIGMA - 1)
                 cn -= uint32_t(TILE) - cnt;
             // ---- the count published, the bucket's prefix over the tiles before
             unsigned long long *slot = a.ring + size_t(t & a.rmask) * SIGMA + c;
-            st_volatile64(slot, lbw(a.tagbase + t, t == 0 ? (LB_INCL | cn) : cn));
+            st_volatile64(slot, lbw(a.tagbase + t, t == t_first ? (LB_INCL | cn) : cn));
             uint32_t excl = 0;
-            if (t > 0) {
+            if (t > t_first) {
                 excl = look_back<SIGMA>(a.ring, a.rmask, a.tagbase, t, c);
                 st_volatile64(slot, lbw(a.tagbase + t, LB_INCL | (excl + cn)));
             }
@@ -1543,6 +1576,8 @@ __global__ void __launch_bounds__(Lb8Cfg<KT, HASV, TILE, NW, OOP>::THREADS, Lb8C
                     st_volatile(a.done + (t & a.rmask), a.tagbase + t);
                 named_bar(LB8_SCAN, C::NT + C::NA); // bucket starts in the tile
                 qoff[c] = g - bst[c];
+                if (GRP && c == 0)
+                    misc[k & 1] = arr;
             } else {
                 // the run lies inside the bucket's output range unless the
                 // look-back words were corrupted: then it is reported and its
@@ -1672,7 +1707,7 @@ __global__ void __launch_bounds__(Lb8Cfg<KT, HASV, TILE, NW, OOP>::THREADS, Lb8C
         __syncwarp();
         const uint32_t *mt = meta + s * 4;
         const bool end = mt[0] == TILE_END;
-        const uint32_t cnt = mt[1], leadk = mt[2], leadv = mt[3];
+        const uint32_t cnt = mt[1], leadk = mt[2] & 0xFFu, leadv = mt[2] >> 8;
         unsigned char *st = sm + size_t(s) * C::STAGE;
         KT *tk = reinterpret_cast<KT *>(st);
         uint32_t *tv = reinterpret_cast<uint32_t *>(st + C::KBYTES);
@@ -1790,6 +1825,14 @@ __global__ void __launch_bounds__(Lb8Cfg<KT, HASV, TILE, NW, OOP>::THREADS, Lb8C
             constexpr int SI = TILE / NT, U = SI % 5 == 0 ? 5 : 4;
             static_assert(SI % U == 0, "whole batches");
             const uint32_t TT = OOP ? 0u : misc[(k - 1) & 1];
+            KT *ok = a.ok;
+            uint32_t *ov = a.ov, n = a.n;
+            if constexpr (GRP) {
+                const uint32_t arr = misc[(k - 1) & 1];
+                ok += grp.out[arr];
+                ov += HASV ? grp.out[arr] : 0;
+                n = grp.len[arr];
+            }
             // byte distance from a key block to its value block, in T and in A
             const long long dvT = reinterpret_cast<const char *>(a.Tv) - reinterpret_cast<const char *>(a.Tk);
             const long long dvA = reinterpret_cast<const char *>(a.Av) - reinterpret_cast<const char *>(a.Ak);
@@ -1815,10 +1858,10 @@ __global__ void __launch_bounds__(Lb8Cfg<KT, HASV, TILE, NW, OOP>::THREADS, Lb8C
                         idx[u] = tid + (k0 + u) * NT + qoff[dig(kv[u])];
 #pragma unroll
                     for (int u = 0; u < U; ++u)
-                        if (tid + (k0 + u) * NT < pcnt && idx[u] < a.n) {
-                            a.ok[idx[u]] = kv[u];
+                        if (tid + (k0 + u) * NT < pcnt && idx[u] < n) {
+                            ok[idx[u]] = kv[u];
                             if (HASV)
-                                a.ov[idx[u]] = vv[u];
+                                ov[idx[u]] = vv[u];
                         }
                 } else {
                     // most runs lie in one block, whose base address the run
@@ -1900,6 +1943,80 @@ __global__ void __launch_bounds__(Lb8Cfg<KT, HASV, TILE, NW, OOP>::THREADS, Lb8C
     }
 }
 
+// ---------------------------------------------------------------- groups of arrays
+// Digit counts (8-bit) of every array of a group: a CTA counts one chunk of
+// one array, four digit positions (blockIdx.y: the first four or the last), in
+// counter columns per lane as k_digit_hist_lanes does.  hist[array][position].
+constexpr uint32_t GRP_CHUNK = 1u << 16;
+
+template <typename KT>
+__global__ void __launch_bounds__(1024)
+    k_group_hist(const KT *keys, const __grid_constant__ LbGroup grp, uint32_t *hist)
+{
+    constexpr int NTD = int(sizeof(KT)), G = 4;
+    extern __shared__ uint32_t sh[]; // G * 256 * 32
+    // the chunk's array: chunks per array follow from its length
+    __shared__ uint32_t s_arr, s_chunk;
+    if (threadIdx.x == 0) {
+        uint32_t b = blockIdx.x, i = 0;
+        for (; i < grp.narr; ++i) {
+            const uint32_t nch = (grp.len[i] + GRP_CHUNK - 1) / GRP_CHUNK;
+            if (b < nch)
+                break;
+            b -= nch;
+        }
+        s_arr = i;
+        s_chunk = b;
+    }
+    const int lane = threadIdx.x & 31, r0 = int(blockIdx.y) * G;
+    for (int i = threadIdx.x; i < G * 256 * 32; i += blockDim.x)
+        sh[i] = 0;
+    __syncthreads();
+    if (s_arr >= grp.narr)
+        return;
+    const uint32_t len = grp.len[s_arr], e0 = s_chunk * GRP_CHUNK, e1 = min(e0 + GRP_CHUNK, len);
+    const KT *src = keys + grp.in[s_arr];
+    constexpr uint32_t U = 8;
+    for (uint32_t e = e0 + threadIdx.x; e < e1; e += U * blockDim.x) {
+        KT k[U];
+#pragma unroll
+        for (uint32_t u = 0; u < U; ++u)
+            if (e + u * blockDim.x < e1)
+                k[u] = src[e + u * blockDim.x];
+#pragma unroll
+        for (uint32_t u = 0; u < U; ++u)
+            if (e + u * blockDim.x < e1)
+#pragma unroll
+                for (int r = 0; r < G; ++r)
+                    atomicAdd(&sh[(r * 256 + digit_of(k[u], uint32_t((r0 + r) * 8), 255u)) * 32 + lane], 1u);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < G * 256; i += blockDim.x) {
+        const uint32_t *rw = sh + size_t(i) * 32;
+        uint32_t sum = 0;
+#pragma unroll
+        for (int l = 0; l < 32; ++l)
+            sum += rw[(l + i) & 31]; // rotated start: consecutive threads, different banks
+        if (sum)
+            atomicAdd(&hist[(size_t(s_arr) * NTD + r0) * 256 + i], sum);
+    }
+}
+
+// Bucket starts of every array and round: tab[round][array][257].
+__global__ void __launch_bounds__(256)
+    k_group_offsets(const uint32_t *hist, uint32_t nt, uint32_t narr, const __grid_constant__ LbGroup grp, uint32_t *tab)
+{
+    __shared__ uint32_t s_a[256], s_tmp[16];
+    const uint32_t arr = blockIdx.x % narr, r = blockIdx.x / narr;
+    s_a[threadIdx.x] = hist[(size_t(arr) * nt + r) * 256 + threadIdx.x];
+    __syncthreads();
+    block_scan<256, 256>(s_a, s_tmp, [] { __syncthreads(); }, threadIdx.x);
+    uint32_t *t = tab + (size_t(r) * narr + arr) * 257;
+    t[threadIdx.x] = s_a[threadIdx.x];
+    if (threadIdx.x == 0)
+        t[256] = grp.len[arr];
+}
+
 // ---------------------------------------------------------------- launch helpers
 // The round kernel of a configuration: 8-bit digits with NW ranking warps, or
 // 11-bit digits (NW ignored).
@@ -1912,6 +2029,13 @@ template <typename KT, bool HASV, int DB, int TILE, int NW, bool OOP> struct LbK
             return k_lb_round8<KT, HASV, TILE, NW, OOP>;
         else
             return k_lb_round11<KT, HASV, TILE, OOP>;
+    }
+    static void launch(int grid, const LbArgs<KT> &a, cudaStream_t st)
+    {
+        if constexpr (DB == 8)
+            k_lb_round8<KT, HASV, TILE, NW, OOP><<<grid, C::THREADS, C::SMEM, st>>>(a, LbNoGroup{});
+        else
+            k_lb_round11<KT, HASV, TILE, OOP><<<grid, C::THREADS, C::SMEM, st>>>(a);
     }
     // CTAs of a launch over ntiles tiles (-1: the kernel cannot be set up)
     static int ctas(size_t ntiles)
@@ -2002,6 +2126,15 @@ static size_t ring_bytes(size_t ntiles, uint32_t sigma)
     return r * sigma * 8 + r * 4;
 }
 
+template <typename KT> static void set_ring(LbArgs<KT> &a, void *mem, size_t ntiles, uint32_t sigma, int round)
+{
+    const uint32_t R = ring_rows(ntiles, sigma);
+    a.ring = static_cast<unsigned long long *>(mem);
+    a.done = reinterpret_cast<uint32_t *>(a.ring + size_t(R) * sigma);
+    a.rmask = R - 1;
+    a.tagbase = uint32_t(round + 1) << 24;
+}
+
 size_t grid_ring_bytes(const Geom &g)
 {
     const uint32_t tile = lb_tile(g.kb, g.db, g.hasv, g.shape);
@@ -2087,11 +2220,7 @@ cudaError_t launch_grid_round(const Geom &g, const Bufs &w, const uint32_t *pi, 
         a.pin = pin;
         a.tab = w.tab + size_t(round) * GridTab<(1 << DB)>::WORDS;
         a.hdr = a.tab + GridTab<(1 << DB)>::HDR;
-        const uint32_t R = ring_rows(ntiles, g.sigma);
-        a.ring = reinterpret_cast<unsigned long long *>(w.status);
-        a.done = reinterpret_cast<uint32_t *>(a.ring + size_t(R) * g.sigma);
-        a.rmask = R - 1;
-        a.tagbase = uint32_t(round + 1) << 24;
+        set_ring(a, w.status, ntiles, g.sigma, round);
         a.ticket = w.ctr + round;
         a.n = n;
         a.ntiles = static_cast<uint32_t>(ntiles);
@@ -2100,7 +2229,7 @@ cudaError_t launch_grid_round(const Geom &g, const Bufs &w, const uint32_t *pi, 
         a.npi = g.npi;
         a.lb = g.lb;
         a.shift = static_cast<uint32_t>(round * g.db);
-        K::kernel()<<<grid, K::C::THREADS, K::C::SMEM, st>>>(a);
+        K::launch(grid, a, st);
         g_launches += 1;
         return cudaGetLastError();
     });
@@ -2139,7 +2268,6 @@ cudaError_t launch_lsd_oop_ws(void *keys, uint32_t *vals, void *keys_alt, uint32
     uint32_t *off = reinterpret_cast<uint32_t *>(scr + al(nt * sigma * 4));
     char *ringp = scr + al(nt * sigma * 4) + al(nt * (sigma + 1) * 4);
     uint32_t *ctr = reinterpret_cast<uint32_t *>(ringp + al(ring_bytes(ntiles, sigma)));
-    const uint32_t R = ring_rows(ntiles, sigma);
     e = cudaMemsetAsync(hist, 0, size_t(nt) * sigma * 4, st);
     if (e == cudaSuccess)
         e = cudaMemsetAsync(ctr, 0, 64 * 4, st);
@@ -2170,15 +2298,12 @@ cudaError_t launch_lsd_oop_ws(void *keys, uint32_t *vals, void *keys_alt, uint32
             a.ok = dst;
             a.ov = vd;
             a.tab = off + size_t(r) * (sigma + 1);
-            a.ring = reinterpret_cast<unsigned long long *>(ringp);
-            a.done = reinterpret_cast<uint32_t *>(a.ring + size_t(R) * sigma);
-            a.rmask = R - 1;
-            a.tagbase = uint32_t(r + 1) << 24;
+            set_ring(a, ringp, ntiles, sigma, r);
             a.ticket = ctr + r;
             a.n = nn;
             a.ntiles = static_cast<uint32_t>(ntiles);
             a.shift = static_cast<uint32_t>(r * DB);
-            K::kernel()<<<grid, K::C::THREADS, K::C::SMEM, st>>>(a);
+            K::launch(grid, a, st);
             g_launches += 1;
             std::swap(src, dst);
             std::swap(vs, vd);
@@ -2193,6 +2318,105 @@ cudaError_t launch_lsd_oop_ws(void *keys, uint32_t *vals, void *keys_alt, uint32
     });
     cudaError_t e2 = own ? cudaFreeAsync(scr, st) : cudaSuccess;
     return e != cudaSuccess ? e : e2;
+}
+
+// ---------------------------------------------------------------- groups of arrays, 8-bit digits
+// [alternate keys | alternate values | cleared: counts, tickets, look-back ring | bucket starts]
+struct GroupLayout {
+    size_t altv, hist, ctr, ring, tab, total;
+    uint32_t ntiles;
+};
+
+static GroupLayout group_layout(const SegGroup &g, int kb, bool hasv)
+{
+    auto al = [](size_t x) { return (x + 255) & ~size_t(255); };
+    GroupLayout L{};
+    const uint32_t tile = lb_tile(kb, 8, hasv, 0);
+    size_t el = 0;
+    for (uint32_t i = 0; i < g.narr; ++i) {
+        el += (size_t(g.len[i]) + 3) & ~size_t(3);
+        L.ntiles += (g.len[i] + tile - 1) / tile;
+    }
+    size_t off = al(el * kb);
+    L.altv = off;
+    off += hasv ? al(el * 4) : 0;
+    L.hist = off;
+    off += al(size_t(g.narr) * kb * 256 * 4);
+    L.ctr = off;
+    off += al(64 * 4);
+    L.ring = off;
+    off += al(ring_bytes(L.ntiles, 256));
+    L.tab = off;
+    off += al(size_t(g.narr) * kb * 257 * 4);
+    L.total = off;
+    return L;
+}
+
+size_t lsd_group_bytes(const SegGroup &g, int kb, bool hasv) { return group_layout(g, kb, hasv).total; }
+
+cudaError_t launch_lsd_group(void *keys, uint32_t *vals, const SegGroup &g, int kb, void *pool, cudaStream_t st)
+{
+    const GroupLayout L = group_layout(g, kb, vals != nullptr);
+    char *base = static_cast<char *>(pool);
+    uint32_t *hist = reinterpret_cast<uint32_t *>(base + L.hist), *ctr = reinterpret_cast<uint32_t *>(base + L.ctr);
+    uint32_t *tab = reinterpret_cast<uint32_t *>(base + L.tab);
+    cudaError_t e = cudaMemsetAsync(hist, 0, L.tab - L.hist, st);
+    if (e != cudaSuccess)
+        return e;
+    return lb_dispatch(kb, 8, vals != nullptr, [&]<typename KT, bool HASV, int DB, int TILE, int NW>() {
+        if constexpr (DB != 8) {
+            return cudaErrorInvalidValue;
+        } else {
+            using C = Lb8Cfg<KT, HASV, TILE, NW, true>;
+            const auto kern = k_lb_round8<KT, HASV, TILE, NW, true, true>;
+            static DeviceOnce attr;
+            const cudaError_t ea = attr.run([&] {
+                cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(C::SMEM));
+                if (r == cudaSuccess)
+                    r = cudaFuncSetAttribute(k_group_hist<KT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             4 * 256 * 32 * 4);
+                return r;
+            });
+            if (ea != cudaSuccess)
+                return ea;
+            LbGroup in{}, out{}; // even rounds: from the arrays; odd rounds: back to them
+            in.narr = g.narr;
+            uint32_t tiles = 0, chunks = 0;
+            size_t alt = 0;
+            for (uint32_t i = 0; i < g.narr; ++i) {
+                in.tile0[i] = tiles;
+                in.len[i] = g.len[i];
+                in.in[i] = g.off[i];
+                in.out[i] = alt;
+                tiles += (g.len[i] + TILE - 1) / TILE;
+                chunks += (g.len[i] + GRP_CHUNK - 1) / GRP_CHUNK;
+                alt += (size_t(g.len[i]) + 3) & ~size_t(3);
+            }
+            out = in;
+            std::swap(out.in, out.out);
+            constexpr int nt = int(sizeof(KT));
+            k_group_hist<KT><<<dim3(chunks, nt / 4), 1024, 4 * 256 * 32 * 4, st>>>(static_cast<const KT *>(keys), in, hist);
+            k_group_offsets<<<g.narr * nt, 256, 0, st>>>(hist, nt, g.narr, in, tab);
+            const int sms = num_sms(), grid = tiles < uint32_t(sms) ? static_cast<int>(tiles) : sms;
+            KT *alt_k = reinterpret_cast<KT *>(base);
+            uint32_t *alt_v = HASV ? reinterpret_cast<uint32_t *>(base + L.altv) : nullptr;
+            for (int r = 0; r < nt; ++r) {
+                LbArgs<KT> a{};
+                a.ik = r & 1 ? alt_k : static_cast<KT *>(keys);
+                a.iv = r & 1 ? alt_v : vals;
+                a.ok = r & 1 ? static_cast<KT *>(keys) : alt_k;
+                a.ov = r & 1 ? vals : alt_v;
+                a.tab = tab + size_t(r) * g.narr * 257;
+                set_ring(a, base + L.ring, tiles, 256, r);
+                a.ticket = ctr + r;
+                a.ntiles = tiles;
+                a.shift = static_cast<uint32_t>(r * 8);
+                kern<<<grid, C::THREADS, C::SMEM, st>>>(a, r & 1 ? out : in);
+            }
+            g_launches += 2 + nt;
+            return cudaGetLastError();
+        }
+    });
 }
 
 cudaError_t launch_lsd_oop(void *keys, uint32_t *vals, void *keys_alt, uint32_t *vals_alt,

@@ -111,6 +111,16 @@ cudaError_t launch_lsd_oop(void *keys, uint32_t *vals, void *keys_alt, uint32_t 
 cudaError_t launch_lsd_oop_ws(void *keys, uint32_t *vals, void *keys_alt, uint32_t *vals_alt,
                               size_t n, int kb, int db, void *scratch, cudaStream_t st);
 size_t lsd_oop_scratch_bytes(size_t n, int kb, int db, bool hasv);
+// several arrays sorted out of place together (8-bit digits), one launch per
+// round for all, through alternate arrays in a pool of lsd_group_bytes
+constexpr uint32_t SEG_GROUP = 64; // arrays of a group at most
+struct SegGroup {
+    uint32_t narr;
+    unsigned long long off[SEG_GROUP]; // first element in keys / vals
+    uint32_t len[SEG_GROUP];
+};
+size_t lsd_group_bytes(const SegGroup &g, int kb, bool hasv);
+cudaError_t launch_lsd_group(void *keys, uint32_t *vals, const SegGroup &g, int kb, void *pool, cudaStream_t st);
 // a short array (n <= small_sort_max) sorted in one launch in a cluster's
 // shared memory; flt: keys are float32 bits, transformed on the way
 uint32_t small_sort_max(int kb, bool hasv);
@@ -127,7 +137,7 @@ cudaError_t launch_head_save(const void *keys, const uint32_t *vals, uint32_t h,
 cudaError_t launch_head_merge(void *keys, uint32_t *vals, uint32_t h, size_t nbody, int kb, void *buf, cudaStream_t st);
 size_t seg_scratch_bytes(int kb, bool hasv, size_t nseg, uint32_t med_max, uint32_t med_ctas, bool ip);
 cudaError_t launch_segmented(void *keys, uint32_t *vals, const unsigned long long *off_dev,
-                             size_t nseg, int kb, int db, uint32_t med_max, uint32_t med_ctas, bool ip,
+                             size_t nseg, int kb, int db, uint32_t med_max, uint32_t med_ctas, uint32_t med_lim, bool ip,
                              void *scratch, cudaStream_t st);
 unsigned take_status_seg();
 

@@ -1537,7 +1537,7 @@ size_t seg_scratch_bytes(int kb, bool hasv, size_t nseg, uint32_t med_max, uint3
 }
 
 cudaError_t launch_segmented(void *keys, uint32_t *vals, const unsigned long long *off_dev,
-                             size_t nseg, int kb, int db, uint32_t med_max, uint32_t med_ctas, bool ip,
+                             size_t nseg, int kb, int db, uint32_t med_max, uint32_t med_ctas, uint32_t med_lim, bool ip,
                              void *scratch, cudaStream_t st)
 {
     if (ip && db != 8)
@@ -1568,7 +1568,7 @@ cudaError_t launch_segmented(void *keys, uint32_t *vals, const unsigned long lon
     if (e != cudaSuccess)
         return e;
     k_seg_classify<<<(nseg + 255) / 256 > 0 ? (nseg + 255) / 256 : 1, 256, 0, st>>>(
-        a, seg_small_max(db), SEG_MED);
+        a, seg_small_max(db), med_lim);
     g_launches += 1;
     const int mc = static_cast<int>(med_ctas);
     using u64 = unsigned long long;
