@@ -144,7 +144,7 @@ radsort_status radsort_autotune_digits(const void *keys, const uint32_t *values,
 
 /*
  * Bytes of device workspace radsort_sort_ex needs: the scratch array T
- * (2*sigma*p blocks in the chunk layout, Sec. 2.1 and 4.3; 4*sigma + 1 in the
+ * (2*sigma*p blocks in the chunk layout, Sec. 2.1 and 4.3; 4*256 + 1 in the
  * grid layout), the block permutation pi and its successor, the usage array
  * U (Alg. 5-6, chunk layout), the partial-block list P, the per-chunk
  * counters or (grid layout) the digit histograms and the look-back words of
@@ -158,7 +158,9 @@ radsort_status radsort_workspace_size(size_t n, int key_bytes, int value_bytes, 
  * Alg. 2 (radSort): setup (Alg. 4), n_t rounds of sortPhase (Alg. 5) and
  * fixupPhase (Alg. 6), then Finalize (Alg. 7), in place on keys[0..n) and
  * values[0..n).  key_bytes: 4 or 8.  digit_bits: 8 (sigma = 256) or 11
- * (sigma = 2048).  Allocates its workspace with cudaMallocAsync on `stream`
+ * (sigma = 2048; in the grid layout a pass has at most 256 buckets all the
+ * same: a whole sort runs by bytes, a part of the rounds or a round of the
+ * permuted representation in two stable passes per digit).  Allocates its workspace with cudaMallocAsync on `stream`
  * and frees it the same way.
  */
 radsort_status radsort_sort(void *keys, uint32_t *values, size_t n, int key_bytes, int digit_bits,
@@ -255,8 +257,8 @@ radsort_status radsort_perm_close(radsort_perm *h);
 
 /*
  * Comparison baseline: a conventional out-of-place LSD radix sort, Alg. 1
- * applied for t = n_t-1 .. 0, with one upfront pass that histograms all
- * digits and a decoupled look-back scan per round.  keys_alt / values_alt are
+ * applied for t = n_t-1 .. 0 (11-bit digits: by bytes too), with one upfront
+ * pass that histograms all digits and a decoupled look-back scan per round.  keys_alt / values_alt are
  * caller-provided n-element scratch arrays (the n*(key+value) bytes of extra
  * memory that Radsort avoids); the result ends in keys / values.
  */

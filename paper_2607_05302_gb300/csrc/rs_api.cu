@@ -155,6 +155,9 @@ static radsort_status fill_geom_grid(size_t n, int kb, bool hasv, int db, uint32
 {
     if (shape < 0 || shape > 2)
         return RADSORT_EINVAL;
+    // 11-bit digits take blocks of 4096 elements with every key and value width
+    if (db == 11 && b == 4096 && lb_tile(kb, db, hasv, shape) % b != 0)
+        shape = LB_SHAPE_4096;
     if (!pow2(b) || b < 64 || b > 4096 || lb_tile(kb, db, hasv, shape) % b != 0)
         return RADSORT_EINVAL; // a tile holds whole blocks
     if (n >= (size_t(1) << 31))
@@ -163,8 +166,9 @@ static radsort_status fill_geom_grid(size_t n, int kb, bool hasv, int db, uint32
     g->kb = kb;
     g->hasv = hasv;
     g->db = db;
-    g->sigma = 1u << db;
+    g->sigma = 256; // buckets of a pass
     g->nt = (8 * kb + db - 1) / db;
+    g->whole = false;
     g->b = b;
     g->lb = ilog2(b);
     g->p = 1;
@@ -211,8 +215,8 @@ static void auto_plan(size_t n, int kb, int vb, int db, radsort_plan *pl)
         size_t least = 0;
         for (int i = 0; i < 5; ++i) {
             Geom g;
-            if (fill_geom_grid(n, kb, vb != 0, db, cands[i], 0, &g) != RADSORT_OK)
-                continue;
+            if (fill_geom_grid(n, kb, vb != 0, db, cands[i], 0, &g) != RADSORT_OK || g.shape != 0)
+                continue; // (not for smaller tiles)
             ws[i] = layout(g, nullptr, nullptr);
             if (!least || ws[i] < least)
                 least = ws[i];
@@ -363,7 +367,7 @@ static size_t layout(const Geom &g, void *base, Bufs *w)
         // (one memset clears from here to the end of the look-back words)
         b.state = static_cast<uint32_t *>(take(ST_WORDS * 4));
         b.ctr = static_cast<uint32_t *>(take(64 * 4));
-        b.hist = static_cast<uint32_t *>(take(size_t(g.nt) * g.sigma * 4));
+        b.hist = static_cast<uint32_t *>(take(size_t(digit_passes(g.kb, g.db, false)) * 256 * 4));
         const size_t jump = align_up(npi2 * 8, 256), fin = finalize_extra_bytes(g);
         const size_t lbw = grid_ring_bytes(g);
         char *z = static_cast<char *>(take(lbw > jump + fin ? lbw : jump + fin));
@@ -439,15 +443,18 @@ static cudaError_t run_rounds(const Geom &g, Bufs &w, int rounds, cudaStream_t s
             Scope sc(0, -1, st);
             e = launch_grid_setup(g, w, pc, st);
         }
-        for (int r = 0; r < rounds && e == cudaSuccess; ++r) {
-            {   // the parts of the next map known before the round (head
+        const bool bytes = by_bytes(g.db, g.whole);
+        const int ppd = bytes ? 1 : 2, np = g.whole ? digit_passes(g.kb, g.db, true) : rounds * ppd;
+        for (int q = 0; q < np && e == cudaSuccess; ++q) {
+            const int r = bytes ? 8 * q / g.db : q / ppd; // the digit it belongs to
+            {   // the parts of the next map known before the pass (head
                 // start, shared blocks, each bucket's first blocks)
                 Scope sc(2, r, st);
-                e = launch_grid_prep(g, w, pc, pn, r, st);
+                e = launch_grid_prep(g, w, pc, pn, q, st);
             }
             if (e == cudaSuccess) {
                 Scope sc(1, r, st);
-                e = launch_grid_round(g, w, pc, pn, r, st);
+                e = launch_grid_round(g, w, pc, pn, q, st);
             }
             uint32_t *t = pc;
             pc = pn;
@@ -702,6 +709,7 @@ static radsort_status sort_common(void *keys, uint32_t *values, size_t n, int ke
     g.npi = g.nA + g.nT;
     if (rounds > g.nt)
         return RADSORT_EINVAL;
+    g.whole = rounds < 0 || rounds == g.nt;
     cudaStream_t st = as_stream(stream);
     const size_t need = layout(g, nullptr, nullptr);
     void *ws = workspace;
@@ -1692,14 +1700,15 @@ radsort_status radsort_perm_rounds(radsort_perm *h, int first, int count, void *
         if (e == cudaSuccess)
             h->hist_ok = true;
     }
-    for (int r = first; r < first + count && e == cudaSuccess; ++r) {
+    const int ppd = g.db == 8 ? 1 : 2;
+    for (int q = first * ppd; q < (first + count) * ppd && e == cudaSuccess; ++q) {
         {
-            Scope sc(2, r, st);
-            e = launch_grid_prep(g, h->w, h->pc, h->pn, r, st);
+            Scope sc(2, q / ppd, st);
+            e = launch_grid_prep(g, h->w, h->pc, h->pn, q, st);
         }
         if (e == cudaSuccess) {
-            Scope sc(1, r, st);
-            e = launch_grid_round(g, h->w, h->pc, h->pn, r, st);
+            Scope sc(1, q / ppd, st);
+            e = launch_grid_round(g, h->w, h->pc, h->pn, q, st);
         }
         std::swap(h->pc, h->pn);
     }

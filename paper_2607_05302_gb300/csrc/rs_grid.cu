@@ -39,8 +39,7 @@
 // number of CTAs, and after the last round every block but the array's tail
 // is full: Finalize is a block permutation plus one tail copy.
 //
-// Round kernels (k_lb_round8, k_lb_round11; both layouts): a producer warp
-// takes tiles in ticket order and streams them into a ring of shared-memory
+// Round kernel (k_lb_round8; both layouts): a producer warp takes tiles in ticket order and streams them into a ring of shared-memory
 // stages with bulk copies (TMA) that complete on mbarriers; other warps rank
 // each tile's digits stably, publish the tile's per-digit counts, reorder the
 // tile by digit in shared memory, resolve the global per-digit offsets by
@@ -89,74 +88,6 @@ __device__ __forceinline__ unsigned long long lbw(uint32_t tag, uint32_t v)
 }
 
 // ---------------------------------------------------------------- digit histograms
-// Counts of every digit position in one read of the keys.  Each thread
-// keeps, per digit position, the digit of its last key and the run length,
-// and adds a run to the shared histogram when the digit changes (one atomic
-// per key on random keys, one per run on sorted or constant ones).  Four
-// 16-byte loads per thread are in flight per step.
-template <typename KT, int DB>
-__global__ void __launch_bounds__(512) k_digit_hist(const KT *keys, uint32_t n, uint32_t *hist)
-{
-    constexpr int SIGMA = 1 << DB;
-    constexpr int NTD = (8 * int(sizeof(KT)) + DB - 1) / DB;
-    constexpr int V = 16 / sizeof(KT), U = 4;
-    extern __shared__ uint32_t sh[];
-    for (int i = threadIdx.x; i < NTD * SIGMA; i += blockDim.x)
-        sh[i] = 0;
-    __syncthreads();
-    uint32_t last[NTD], run[NTD];
-#pragma unroll
-    for (int r = 0; r < NTD; ++r) {
-        last[r] = 0;
-        run[r] = 0;
-    }
-    auto put = [&](KT k) {
-#pragma unroll
-        for (int r = 0; r < NTD; ++r) {
-            const uint32_t d = digit_of(k, uint32_t(r * DB), SIGMA - 1);
-            if (d == last[r]) {
-                ++run[r];
-            } else {
-                if (run[r])
-                    atomicAdd(&sh[r * SIGMA + last[r]], run[r]);
-                last[r] = d;
-                run[r] = 1;
-            }
-        }
-    };
-    const size_t stride = size_t(gridDim.x) * blockDim.x;
-    const size_t first = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    const bool vec = (reinterpret_cast<uintptr_t>(keys) & 15u) == 0;
-    const size_t nv = vec ? n / V : 0;
-    const uint4 *kv = reinterpret_cast<const uint4 *>(keys);
-    for (size_t i = first; i < nv; i += U * stride) {
-        uint4 v[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (i + u * stride < nv)
-                v[u] = kv[i + u * stride];
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (i + u * stride < nv) {
-                KT k[V];
-                memcpy(k, &v[u], 16);
-#pragma unroll
-                for (int q = 0; q < V; ++q)
-                    put(k[q]);
-            }
-    }
-    for (size_t i = nv * V + first; i < n; i += stride)
-        put(keys[i]);
-#pragma unroll
-    for (int r = 0; r < NTD; ++r)
-        if (run[r])
-            atomicAdd(&sh[r * SIGMA + last[r]], run[r]);
-    __syncthreads();
-    for (int i = threadIdx.x; i < NTD * SIGMA; i += blockDim.x)
-        if (sh[i])
-            atomicAdd(&hist[i], sh[i]);
-}
-
 // 8-bit digits: counts of four digit positions r0 .. r0+3 with one counter
 // column per lane (counter (r, d) of lane l at word (r*256 + d)*32 + l), so
 // the 32 atomics of a warp instruction fall in 32 different banks whatever
@@ -216,40 +147,82 @@ __global__ void __launch_bounds__(1024) k_digit_hist_lanes(const KT *keys, uint3
     }
 }
 
-// Launches the digit histograms for the key and digit widths.
-static cudaError_t launch_digit_hist(const void *keys, uint32_t n, int kb, int db, uint32_t *hist,
+// 11-bit digits one by one: counts of all passes (at most 64 buckets each) in one read,
+// in counter columns per lane too: 48 or 96 KB of counters.
+template <typename KT>
+__global__ void __launch_bounds__(1024) k_pass_hist_lanes(const KT *keys, uint32_t n, uint32_t *hist)
+{
+    constexpr int NP = digit_passes(int(sizeof(KT)), 11, false), B = 64, U = 4;
+    extern __shared__ uint32_t sh[]; // NP * B * 32
+    const int lane = threadIdx.x & 31;
+    for (int i = threadIdx.x; i < NP * B * 32; i += blockDim.x)
+        sh[i] = 0;
+    __syncthreads();
+    const size_t stride = size_t(gridDim.x) * blockDim.x;
+    for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += U * stride) {
+        KT k[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (i + u * stride < n)
+                k[u] = keys[i + u * stride];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (i + u * stride < n)
+#pragma unroll
+                for (int q = 0; q < NP; ++q) {
+                    const DigitPass dp = digit_pass(int(sizeof(KT)), 11, false, q);
+                    atomicAdd(&sh[(q * B + digit_of(k[u], dp.shift, dp.mask())) * 32 + lane], 1u);
+                }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < NP * B; i += blockDim.x) {
+        const uint32_t *row = sh + size_t(i) * 32;
+        uint32_t sum = 0;
+#pragma unroll
+        for (int l = 0; l < 32; ++l)
+            sum += row[(l + i) & 31]; // rotated start: consecutive threads, different banks
+        if (sum)
+            atomicAdd(&hist[(i / B) * 256 + i % B], sum);
+    }
+}
+
+// Launches the bucket counts of every pass, by bytes or (11-bit digits one by
+// one) by half digits.
+static cudaError_t launch_digit_hist(const void *keys, uint32_t n, int kb, bool bytes, uint32_t *hist,
                                      cudaStream_t st)
 {
     using u64 = unsigned long long;
-    if (db == 8) {
-        constexpr int LSM = 4 * 256 * 32 * 4;
-        static DeviceOnce attr;
-        const cudaError_t ea = attr.run([] {
-            cudaError_t e = cudaFuncSetAttribute(k_digit_hist_lanes<uint32_t>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, LSM);
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(k_digit_hist_lanes<u64>, cudaFuncAttributeMaxDynamicSharedMemorySize, LSM);
-            return e;
-        });
-        if (ea != cudaSuccess)
-            return ea;
-        const int grid = num_sms();
+    constexpr int LSM = 4 * 256 * 32 * 4;
+    constexpr int P4 = digit_passes(4, 11, false) * 64 * 32 * 4, P8 = digit_passes(8, 11, false) * 64 * 32 * 4;
+    static DeviceOnce attr;
+    const cudaError_t ea = attr.run([] {
+        cudaError_t e = cudaFuncSetAttribute(k_digit_hist_lanes<uint32_t>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, LSM);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_digit_hist_lanes<u64>, cudaFuncAttributeMaxDynamicSharedMemorySize, LSM);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_pass_hist_lanes<uint32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, P4);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_pass_hist_lanes<u64>, cudaFuncAttributeMaxDynamicSharedMemorySize, P8);
+        return e;
+    });
+    if (ea != cudaSuccess)
+        return ea;
+    const int grid = num_sms();
+    g_launches += 1;
+    if (bytes) {
         if (kb == 4) {
             k_digit_hist_lanes<uint32_t><<<grid, 1024, LSM, st>>>(static_cast<const uint32_t *>(keys), n, 0, hist);
-            g_launches += 1;
         } else {
             for (int r0 = 0; r0 < 8; r0 += 4)
                 k_digit_hist_lanes<u64><<<grid, 1024, LSM, st>>>(static_cast<const u64 *>(keys), n, r0, hist);
-            g_launches += 2;
+            g_launches += 1;
         }
-        return cudaGetLastError();
+    } else if (kb == 4) {
+        k_pass_hist_lanes<uint32_t><<<2 * grid, 1024, P4, st>>>(static_cast<const uint32_t *>(keys), n, hist);
+    } else {
+        k_pass_hist_lanes<u64><<<grid, 1024, P8, st>>>(static_cast<const u64 *>(keys), n, hist);
     }
-    const int grid = num_sms() * 2;
-    if (kb == 4)
-        k_digit_hist<uint32_t, 11><<<grid, 512, 3 * 2048 * 4, st>>>(static_cast<const uint32_t *>(keys), n, hist);
-    else
-        k_digit_hist<u64, 11><<<grid, 512, 6 * 2048 * 4, st>>>(static_cast<const u64 *>(keys), n, hist);
-    g_launches += 1;
     return cudaGetLastError();
 }
 
@@ -297,17 +270,17 @@ __device__ __forceinline__ uint32_t block_scan(uint32_t *a, uint32_t *tmp, F &&b
     return tot;
 }
 
-// Per-round bucket offsets of the out-of-place sort: O[r][c] exclusive over
-// digits, O[r][sigma] = n (one block per digit position).
-template <int DB> __global__ void __launch_bounds__(1024) k_offsets(const uint32_t *hist, uint32_t *off, uint32_t n)
+// Bucket offsets of every pass of the out-of-place sort: O[r][c] exclusive over
+// buckets, O[r][256] = n (one block per pass).
+__global__ void __launch_bounds__(256) k_offsets(const uint32_t *hist, uint32_t *off, uint32_t n)
 {
-    constexpr int SIGMA = 1 << DB;
-    __shared__ uint32_t s_a[SIGMA], s_tmp[40];
+    constexpr int SIGMA = 256;
+    __shared__ uint32_t s_a[SIGMA], s_tmp[16];
     const int r = blockIdx.x;
     for (int c = threadIdx.x; c < SIGMA; c += blockDim.x)
         s_a[c] = hist[r * SIGMA + c];
     __syncthreads();
-    block_scan<SIGMA, 1024>(s_a, s_tmp, [] { __syncthreads(); }, threadIdx.x);
+    block_scan<SIGMA, SIGMA>(s_a, s_tmp, [] { __syncthreads(); }, threadIdx.x);
     for (int c = threadIdx.x; c < SIGMA; c += blockDim.x)
         off[r * (SIGMA + 1) + c] = s_a[c];
     if (threadIdx.x == 0)
@@ -320,8 +293,8 @@ template <int DB> __global__ void __launch_bounds__(1024) k_offsets(const uint32
 // the free-list index of its first one, the shared blocks (those with a bucket
 // start strictly inside) in order, and a header.
 enum { TAB_SKIP = 0, TAB_TAKEN = 1, TAB_NS = 2 }; // identity round; free-list entries taken before it; shared blocks
-template <int SIGMA> struct GridTab {
-    static constexpr int O = 0, NS0 = SIGMA + 1, NS1 = NS0 + SIGMA, FREE = NS1 + SIGMA, SHARED = FREE + SIGMA,
+struct GridTab {
+    static constexpr int SIGMA = 256, O = 0, NS0 = SIGMA + 1, NS1 = NS0 + SIGMA, FREE = NS1 + SIGMA, SHARED = FREE + SIGMA,
                          HDR = SHARED + SIGMA, WORDS = HDR + 3;
 };
 
@@ -330,14 +303,14 @@ template <int SIGMA> struct GridTab {
 // pi = [scratch 0 .. H) ++ [A's blocks] ++ [scratch block H: the input tail],
 // and copy that tail.  A digit with one non-empty bucket leaves the sequence
 // unchanged: its round is skipped.
-template <typename KT, int DB>
+template <typename KT>
 __global__ void __launch_bounds__(1024)
     k_grid_tables(const uint32_t *hist, uint32_t *tab, uint32_t r0, uint32_t nr, uint32_t n, uint32_t lb, uint32_t H,
                   uint32_t nA, uint32_t npi, const KT *Ak, const uint32_t *Av, KT *Tk, uint32_t *Tv, uint32_t *pi,
                   uint2 *P, uint32_t *state)
 {
-    constexpr int SIGMA = 1 << DB;
-    using T = GridTab<SIGMA>;
+    using T = GridTab;
+    constexpr int SIGMA = T::SIGMA;
     const uint32_t b = 1u << lb;
     if (blockIdx.x >= nr) { // setup (Alg. 4)
         const uint32_t id = (blockIdx.x - nr) * blockDim.x + threadIdx.x, step = (gridDim.x - nr) * blockDim.x;
@@ -469,13 +442,12 @@ __global__ void __launch_bounds__(1024)
 // took 10-12 us a round (and a memset before it past 65536 blocks); the tables
 // of all rounds in one launch at setup and this kernel take 8 + 4 x 6 us of a
 // sort of 2^20 where that took 45.
-template <int DB>
 __global__ void __launch_bounds__(256)
     k_grid_fill(const uint32_t *tab, uint32_t n, uint32_t lb, uint32_t H, uint32_t nA, uint32_t npi,
                 const uint32_t *pi, uint32_t *pin)
 {
-    constexpr int SIGMA = 1 << DB;
-    using T = GridTab<SIGMA>;
+    using T = GridTab;
+    constexpr int SIGMA = T::SIGMA;
     __shared__ uint32_t s_O[SIGMA + 1], s_list[SIGMA];
     const uint32_t skip = tab[T::HDR + TAB_SKIP], nS = skip ? 0u : tab[T::HDR + TAB_NS];
     if (!skip) {
@@ -528,58 +500,7 @@ __global__ void __launch_bounds__(256)
     }
 }
 
-// ---------------------------------------------------------------- round kernel, 11-bit digits
-template <typename KT, bool HASV, int TILE, bool OOP> struct LbCfg {
-    static constexpr int DB = 11, SIGMA = 1 << DB, STAGES = 2, NW = 16;
-    static constexpr int NT = NW * 32;            // consumer threads
-    static constexpr int THREADS = NT + 32;       // + one producer warp
-    static constexpr int MINB = 1;                // CTAs per SM
-    static constexpr int MAXM = TILE / 64;   // blocks per tile (b >= 64)
-    static constexpr int R = TILE / NW;      // tile elements ranked per warp
-    static constexpr int ITEMS = R / 32;     // elements per consumer thread
-    static_assert(R % 32 == 0, "warp range must be a multiple of 32");
-    // threads per bucket in the column passes (each sums NW / TPB warp rows):
-    // two were 5% faster at 2^26 but at 2^30 u64 left some rounds 3x slower,
-    // four do not
-    static constexpr int TPB = 4;
-    static_assert(NW % TPB == 0, "rows split evenly");
-    // more than 16 elements per thread: digits are recomputed from the keys
-    // and warp ranks kept as 16-bit halves, to stay within the registers
-    static constexpr bool LEAN = ITEMS > 16;
-    // one ballot per digit bit finds the lanes with the same digit; a
-    // per-warp 16-bit row keeps the running count of each digit, later the
-    // warp's start per digit in the reordered tile
-    static constexpr bool PAIR = HASV && sizeof(KT) == 4;
-    static constexpr int HROW = SIGMA + 2;
-    static constexpr size_t al(size_t x) { return (x + 127) & ~size_t(127); }
-    // 16 bytes of slack per array: the lead of a misaligned source (out of place)
-    static constexpr size_t KBYTES = al(size_t(TILE) * sizeof(KT) + 16);
-    static constexpr size_t STAGE = al(KBYTES + (HASV ? size_t(TILE) * 4 + 16 : 0));
-    // warp rows, per-bucket words (tcnt, bstart, gpos), run offsets, block
-    // list, counters and scan scratch
-    static constexpr size_t HIST_BYTES = al(size_t(NW) * HROW * 2);
-    static constexpr size_t BK_BYTES = al(size_t(3) * SIGMA * 4);
-    // touched blocks per tile: at most TILE/b + 2 per bucket with elements
-    static constexpr int LIST = MAXM + 2 * (SIGMA < TILE ? SIGMA : TILE) + 2;
-    // per bucket (offset, list slot of its first block)
-    static constexpr size_t QB_BYTES = al(size_t(SIGMA) * 8);
-    static constexpr size_t LK_BYTES = OOP ? 0 : al(size_t(LIST) * 4);
-    // the per-bucket run offsets and the block list live in the warp-row
-    // region, which the tile no longer needs once reordered
-    static_assert(QB_BYTES + LK_BYTES <= HIST_BYTES, "run offsets and block list fit the warp rows");
-    static constexpr size_t o_stage = 0;
-    static constexpr size_t o_hist = STAGES * STAGE;
-    static constexpr size_t o_bk = o_hist + HIST_BYTES;
-    static constexpr size_t o_qb = o_hist;
-    static constexpr size_t o_lk = o_qb + QB_BYTES;
-    static constexpr size_t o_misc = o_bk + BK_BYTES;
-    static constexpr size_t o_tabs = o_misc + 512; // O (sigma + 1)
-    static constexpr size_t o_meta = o_tabs + al((size_t(SIGMA) + 4) * 4);
-    static constexpr size_t o_bar = o_meta + al(STAGES * 16);
-    static constexpr size_t SMEM = o_bar + al(2 * STAGES * 8);
-    static_assert(SMEM <= 227 * 1024, "shared memory budget");
-};
-
+// ---------------------------------------------------------------- round kernel
 template <typename KT> struct LbArgs {
     const KT *ik;           // out of place: source
     const uint32_t *iv;
@@ -598,7 +519,8 @@ template <typename KT> struct LbArgs {
     uint32_t rmask;         // R - 1 (R a power of two)
     uint32_t tagbase;       // tag of tile t: tagbase + t (grows with the round)
     const uint32_t *hdr;    // Radsort: the tables' header
-    uint32_t n, ntiles, H, nT, npi, lb, shift;
+    uint32_t n, ntiles, H, nT, npi, lb;
+    uint32_t shift, mask;   // the pass's digit: key >> shift & mask, at most 255
 };
 
 // Exclusive prefix of bucket c before tile t: sum of the counts of the tiles
@@ -671,535 +593,6 @@ __device__ __forceinline__ uint32_t wait_pi(const uint32_t *p)
     return PI_NONE;
 }
 
-template <typename KT, bool HASV, int TILE, bool OOP>
-__global__ void __launch_bounds__(LbCfg<KT, HASV, TILE, OOP>::THREADS, 1) k_lb_round11(LbArgs<KT> a)
-{
-    using C = LbCfg<KT, HASV, TILE, OOP>;
-    constexpr int SIGMA = C::SIGMA, NT = C::NT, NW = C::NW, STAGES = C::STAGES, DB = C::DB;
-    extern __shared__ __align__(128) unsigned char sm[];
-    if (!OOP && a.hdr[TAB_SKIP])
-        return; // the digit is constant: the round is the identity
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    uint16_t *hist = reinterpret_cast<uint16_t *>(sm + C::o_hist);
-    uint32_t *bk = reinterpret_cast<uint32_t *>(sm + C::o_bk);
-    uint32_t *tcnt = bk, *bstart = bk + SIGMA, *gpos = bk + 2 * SIGMA;
-    uint32_t *sO = reinterpret_cast<uint32_t *>(sm + C::o_tabs); // sigma + 1 entries
-    const uint32_t *ns0 = a.tab + SIGMA + 1, *ns1 = ns0 + SIGMA;
-    uint2 *qb = reinterpret_cast<uint2 *>(sm + C::o_qb);
-    uint32_t *listb = reinterpret_cast<uint32_t *>(sm + C::o_lk); // block indices
-    uint32_t *meta = reinterpret_cast<uint32_t *>(sm + C::o_meta);
-    uint64_t *full = reinterpret_cast<uint64_t *>(sm + C::o_bar);
-    uint64_t *empty = full + STAGES;
-    // [1..3] a tile's list slots, blocks taken and blocks taken by earlier
-    // tiles, [8..] scan scratch
-    uint32_t *misc = reinterpret_cast<uint32_t *>(sm + C::o_misc);
-
-    const uint32_t b = 1u << a.lb;
-    const uint32_t mask = SIGMA - 1;
-
-    if (tid == 0) {
-        for (int s = 0; s < STAGES; ++s) {
-            mbar_init(&full[s], 1);
-            mbar_init(&empty[s], 1);
-        }
-        fence_mbar_init();
-    }
-    for (int c = tid; c <= SIGMA; c += C::THREADS)
-        sO[c] = a.tab[c];
-    __syncthreads();
-
-    auto kaddr = [&](uint32_t blk) -> KT * {
-        return blk < a.nT ? a.Tk + (size_t(blk) << a.lb) : a.Ak + (size_t(blk - a.nT) << a.lb);
-    };
-    auto vaddr = [&](uint32_t blk) -> uint32_t * {
-        return blk < a.nT ? a.Tv + (size_t(blk) << a.lb) : a.Av + (size_t(blk - a.nT) << a.lb);
-    };
-
-    if (warp == NW) {
-        // ================================================================ producer
-        uint32_t k = 0;
-        uint32_t wm = 0; // tiles below wm have finished their look-back
-        for (;; ++k) {
-            const int s = k % STAGES;
-            const uint32_t par = ((k / STAGES) & 1u) ^ 1u;
-            if (!mbar_wait(&empty[s], par))
-                break;
-            uint32_t t = 0;
-            if (lane == 0)
-                t = atomicAdd(a.ticket, 1u);
-            t = __shfl_sync(0xffffffffu, t, 0);
-            uint32_t *mt = meta + s * 4;
-            // the ring slot of tile t held tile t - R: wait until every tile
-            // up to t - R + 1 has finished its look-back
-            if (t < a.ntiles && t > a.rmask) {
-                const uint32_t need = t - a.rmask + 1; // tiles below `need` must be done
-                unsigned spins = 0;
-                while (wm < need) {
-                    const uint32_t z = wm + lane;
-                    const bool ok = z >= need || ld_volatile(a.done + (z & a.rmask)) >= a.tagbase + z;
-                    const unsigned bal = __ballot_sync(0xffffffffu, ok);
-                    const uint32_t adv = bal == 0xffffffffu ? 32u : uint32_t(__ffs(~bal) - 1);
-                    wm = min(need, wm + adv);
-                    if (wm < need) {
-                        if (++spins > SPIN_LIMIT || ((spins & 1023u) == 0 && wait_failed())) {
-                            set_status(ST_TIMEOUT);
-                            break;
-                        }
-                        __nanosleep(64);
-                    }
-                }
-            }
-            if (t >= a.ntiles) {
-                if (lane == 0) {
-                    mt[0] = TILE_END;
-                    mbar_arrive(&full[s]);
-                }
-                ++k;
-                break;
-            }
-            unsigned char *st = sm + C::o_stage + size_t(s) * C::STAGE;
-            KT *stk = reinterpret_cast<KT *>(st);
-            uint32_t *stv = reinterpret_cast<uint32_t *>(st + C::KBYTES);
-            const uint32_t e0 = t * uint32_t(TILE);
-            const uint32_t cnt = min(uint32_t(TILE), a.n - e0);
-            uint32_t leadk = 0, leadv = 0;
-            if constexpr (OOP) {
-                // the 16-byte-aligned middle by bulk copies, the ragged ends
-                // (under 16 bytes each) by plain loads
-                const uintptr_t ka = reinterpret_cast<uintptr_t>(a.ik + e0);
-                const uintptr_t kz = ka + uintptr_t(cnt) * sizeof(KT);
-                const uintptr_t ka16 = (ka + 15) & ~uintptr_t(15), kz16 = kz & ~uintptr_t(15);
-                leadk = static_cast<uint32_t>((ka & 15) / sizeof(KT));
-                const bool kmid = ka16 < kz16;
-                const uint32_t khead = kmid ? static_cast<uint32_t>((ka16 - ka) / sizeof(KT)) : cnt;
-                const uint32_t ktail = kmid ? static_cast<uint32_t>((kz16 - ka) / sizeof(KT)) : cnt;
-                uint32_t bytes = kmid ? static_cast<uint32_t>(kz16 - ka16) : 0u;
-                uintptr_t va = 0, va16 = 0, vz16 = 0;
-                uint32_t vhead = 0, vtail = 0;
-                bool vmid = false;
-                if (HASV) {
-                    va = reinterpret_cast<uintptr_t>(a.iv + e0);
-                    const uintptr_t vz = va + uintptr_t(cnt) * 4;
-                    va16 = (va + 15) & ~uintptr_t(15);
-                    vz16 = vz & ~uintptr_t(15);
-                    leadv = static_cast<uint32_t>((va & 15) / 4);
-                    vmid = va16 < vz16;
-                    vhead = vmid ? static_cast<uint32_t>((va16 - va) / 4) : cnt;
-                    vtail = vmid ? static_cast<uint32_t>((vz16 - va) / 4) : cnt;
-                    bytes += vmid ? static_cast<uint32_t>(vz16 - va16) : 0u;
-                }
-                if (lane == 0 && bytes)
-                    asm volatile("mbarrier.expect_tx.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&full[s])),
-                                 "r"(bytes)
-                                 : "memory");
-                __syncwarp();
-                if (lane == 0 && kmid)
-                    bulk_g2s(stk + leadk + khead, reinterpret_cast<const void *>(ka16),
-                             static_cast<uint32_t>(kz16 - ka16), &full[s]);
-                if (HASV && lane == 1 && vmid)
-                    bulk_g2s(stv + leadv + vhead, reinterpret_cast<const void *>(va16),
-                             static_cast<uint32_t>(vz16 - va16), &full[s]);
-                for (uint32_t e = lane; e < khead; e += 32)
-                    stk[leadk + e] = a.ik[e0 + e];
-                for (uint32_t e = ktail + lane; e < cnt; e += 32)
-                    stk[leadk + e] = a.ik[e0 + e];
-                if (HASV) {
-                    for (uint32_t e = lane; e < vhead; e += 32)
-                        stv[leadv + e] = a.iv[e0 + e];
-                    for (uint32_t e = vtail + lane; e < cnt; e += 32)
-                        stv[leadv + e] = a.iv[e0 + e];
-                }
-            } else {
-                // blocks t*M .. of the logical data: block i at stage offset i*b
-                const uint32_t nb = (cnt + b - 1) >> a.lb;
-                const uint32_t i0 = a.H + t * (uint32_t(TILE) >> a.lb);
-                uint32_t tot = 0;
-                // (a block index outside the block store is reported and skipped)
-                for (uint32_t base = 0; base < nb; base += 32) {
-                    const uint32_t i = base + lane;
-                    uint32_t bytes = 0;
-                    if (i < nb && a.pi[i0 + i] < a.npi) {
-                        const uint32_t len = min(b, cnt - i * b);
-                        bytes = ((len * uint32_t(sizeof(KT)) + 15u) & ~15u) + (HASV ? ((len * 4u + 15u) & ~15u) : 0u);
-                    }
-                    tot += warp_sum(bytes);
-                }
-                if (lane == 0 && tot)
-                    asm volatile("mbarrier.expect_tx.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&full[s])),
-                                 "r"(tot)
-                                 : "memory");
-                __syncwarp();
-                for (uint32_t i = lane; i < nb; i += 32) {
-                    const uint32_t len = min(b, cnt - i * b);
-                    const uint32_t phys = a.pi[i0 + i];
-                    if (phys >= a.npi) {
-                        set_status(ST_INTERNAL);
-                        continue;
-                    }
-                    bulk_g2s(stk + size_t(i) * b, kaddr(phys), (len * uint32_t(sizeof(KT)) + 15u) & ~15u, &full[s]);
-                    if (HASV)
-                        bulk_g2s(stv + size_t(i) * b, vaddr(phys), (len * 4u + 15u) & ~15u, &full[s]);
-                }
-            }
-            __syncwarp();
-            if (lane == 0) {
-                mt[0] = t;
-                mt[1] = cnt;
-                mt[2] = leadk;
-                mt[3] = leadv;
-            }
-            __syncwarp();
-            if (lane == 0)
-                mbar_arrive(&full[s]); // release: the plain stores above are visible
-        }
-        // drain: every issued copy lands before this CTA exits (only the last
-        // STAGES fills can still be in flight, and no fill follows them, so
-        // the phase each of them completes stays readable)
-        if (lane == 0) {
-            const uint32_t t0 = k > STAGES ? k - STAGES : 0;
-            for (uint32_t t = t0; t < k; ++t)
-                mbar_wait(&full[t % STAGES], (t / STAGES) & 1u);
-        }
-        return;
-    }
-
-    // ==================================================================== consumers
-    const int ctid = tid, cw = warp;
-    uint32_t *tmp = misc + 8;
-    auto bar = [] { named_bar(1, NT); };
-    const uint32_t nP = OOP ? 0u : a.hdr[TAB_TAKEN]; // free-list entries taken before the round
-    const uint32_t M = uint32_t(TILE) >> a.lb;
-
-    for (uint32_t k = 0;; ++k) { // fill k
-        const int s = k % STAGES;
-        if (!mbar_wait(&full[s], (k / STAGES) & 1u))
-            break;
-        const uint32_t *mt = meta + s * 4;
-        const uint32_t t = mt[0];
-        if (t == TILE_END)
-            break;
-        const uint32_t cnt = mt[1], leadk = mt[2], leadv = mt[3];
-        unsigned char *st = sm + C::o_stage + size_t(s) * C::STAGE;
-        KT *tk = reinterpret_cast<KT *>(st);
-        uint32_t *tv = reinterpret_cast<uint32_t *>(st + C::KBYTES);
-        uint2 *tp = reinterpret_cast<uint2 *>(st); // (key, value) pairs after the reorder
-
-        // ---- 1. this thread's elements into registers; stable rank within the warp
-        KT key[C::ITEMS];
-        uint32_t val[C::ITEMS];
-        uint32_t digs[C::LEAN ? 1 : C::ITEMS];
-        uint32_t rks[C::LEAN ? (C::ITEMS + 1) / 2 : C::ITEMS];
-        // digit of item it (SIGMA past the tile's end) and its rank in the warp
-        auto dig = [&](int it) -> uint32_t {
-            if constexpr (C::LEAN)
-                return cw * C::R + it * 32 + lane < cnt ? digit_of(key[it], a.shift, mask)
-                                                          : uint32_t(SIGMA);
-            else
-                return digs[it];
-        };
-        auto set_rk = [&](int it, uint32_t v) {
-            if constexpr (C::LEAN)
-                rks[it >> 1] = (it & 1) ? ((rks[it >> 1] & 0xFFFFu) | (v << 16)) : ((rks[it >> 1] & 0xFFFF0000u) | v);
-            else
-                rks[it] = v;
-        };
-        auto get_rk = [&](int it) -> uint32_t {
-            if constexpr (C::LEAN)
-                return (it & 1) ? (rks[it >> 1] >> 16) : (rks[it >> 1] & 0xFFFFu);
-            else
-                return rks[it];
-        };
-#pragma unroll
-        for (int it = 0; it < C::ITEMS; ++it) {
-            const uint32_t e = cw * C::R + it * 32 + lane;
-            key[it] = tk[leadk + e];
-            if (HASV)
-                val[it] = tv[leadv + e];
-            if constexpr (!C::LEAN)
-                digs[it] = e < cnt ? digit_of(key[it], a.shift, mask) : uint32_t(SIGMA);
-        }
-        const unsigned lt = lanemask_lt();
-        uint16_t *hw = hist + cw * C::HROW;
-        for (int c = lane; c < SIGMA; c += 32)
-            hw[c] = 0;
-        {
-            // a few rows at a time: their peer masks (independent ballots),
-            // then row by row the lowest lane of each digit group reads and
-            // advances the running count and passes the old count to its
-            // group with a shuffle
-            constexpr int CH = C::ITEMS % 4 == 0 ? 4 : (C::ITEMS % 2 == 0 ? 2 : 1);
-            __syncwarp();
-#pragma unroll
-            for (int i0 = 0; i0 < C::ITEMS; i0 += CH) {
-                unsigned peers[CH];
-#pragma unroll
-                for (int q = 0; q < CH; ++q)
-                    peers[q] = peer_mask<DB>(dig(i0 + q), dig(i0 + q) < SIGMA);
-#pragma unroll
-                for (int q = 0; q < CH; ++q) {
-                    const uint32_t d = dig(i0 + q);
-                    const unsigned pm = peers[q];
-                    const int ld = pm ? __ffs(pm) - 1 : lane;
-                    uint32_t base = 0;
-                    if (d < SIGMA && ld == lane) {
-                        base = hw[d];
-                        hw[d] = static_cast<uint16_t>(base + __popc(pm));
-                    }
-                    base = __shfl_sync(0xffffffffu, base, ld);
-                    set_rk(i0 + q, base + __popc(pm & lt));
-                    __syncwarp();
-                }
-            }
-        }
-        bar();
-
-        if (ctid == 0) // this tile's slot counters (step 4)
-            misc[1] = misc[2] = misc[3] = 0u;
-
-        // ---- 2. tile counts per bucket, published for the look-back, and
-        // their exclusive scan (bucket starts in the reordered tile)
-        auto cnt_at = [&](int w, int c) -> uint32_t { return hist[w * C::HROW + c]; };
-        constexpr int RPT = NW / C::TPB;
-        for (int i = ctid; i < SIGMA * C::TPB; i += NT) {
-            const int c = i / C::TPB, part = i % C::TPB;
-            uint32_t sum = 0;
-#pragma unroll
-            for (int r = 0; r < RPT; ++r)
-                sum += cnt_at(part * RPT + r, c);
-#pragma unroll
-            for (int o = C::TPB / 2; o > 0; o >>= 1)
-                sum += __shfl_xor_sync(0xffffffffu, sum, o, C::TPB);
-            if (part == C::TPB - 1) {
-                tcnt[c] = sum;
-                bstart[c] = sum;
-                st_volatile64(a.ring + size_t(t & a.rmask) * SIGMA + c,
-                              lbw(a.tagbase + t, t == 0 ? (LB_INCL | sum) : sum));
-            }
-        }
-        bar();
-        block_scan<SIGMA, NT>(bstart, tmp, bar, ctid);
-        // each warp's start per bucket in the reordered tile: bucket start +
-        // the counts of the warps before it (the ranks are warp-relative)
-        for (int i = ctid; i < SIGMA * C::TPB; i += NT) {
-            const int c = i / C::TPB, part = i % C::TPB;
-            uint32_t h[RPT], sum = 0;
-#pragma unroll
-            for (int r = 0; r < RPT; ++r) {
-                h[r] = cnt_at(part * RPT + r, c);
-                sum += h[r];
-            }
-            uint32_t incl = sum;
-#pragma unroll
-            for (int o = 1; o < C::TPB; o <<= 1) {
-                const uint32_t x = __shfl_up_sync(0xffffffffu, incl, o, C::TPB);
-                if (part >= o)
-                    incl += x;
-            }
-            uint32_t run = bstart[c] + incl - sum;
-#pragma unroll
-            for (int r = 0; r < RPT; ++r) {
-                hist[(part * RPT + r) * C::HROW + c] = static_cast<uint16_t>(run);
-                run += h[r];
-            }
-        }
-        bar();
-
-        // ---- 3. reorder the tile by digit, in place in its stage buffer
-        // (every element is in registers since the barriers above)
-#pragma unroll
-        for (int it = 0; it < C::ITEMS; ++it) {
-            const uint32_t d = dig(it);
-            if (d < SIGMA) {
-                const uint32_t pos = cnt_at(cw, d) + get_rk(it);
-                if (pos >= uint32_t(TILE)) { // only a broken scan gets here
-                    set_status(ST_INTERNAL);
-                    continue;
-                }
-                if constexpr (C::PAIR) {
-                    tp[pos] = make_uint2(static_cast<uint32_t>(key[it]), val[it]);
-                } else {
-                    tk[pos] = key[it];
-                    if (HASV)
-                        tv[pos] = val[it];
-                }
-            }
-        }
-
-        bar(); // every warp has read its row before qb and the list overwrite it
-
-        // ---- 4. global offset of each bucket's run (look-back); Radsort:
-        // blocks touched, blocks taken here and by earlier tiles, list slots
-        // and free-list offsets (shared counters: the order of the blocks a
-        // tile takes does not matter, only that each index is used once), and
-        // a prefetch of the map entry of the first block touched
-        constexpr int PFN = (SIGMA + NT - 1) / NT;
-        uint32_t pf[PFN], l0s[PFN], kos[PFN];
-#pragma unroll
-        for (int q = 0; q < PFN; ++q) {
-            const int c = ctid + q * NT;
-            pf[q] = PI_NONE;
-            l0s[q] = kos[q] = 0;
-            if (c >= SIGMA) // whole warps: SIGMA and NT are multiples of 32
-                continue;
-            const uint32_t cn = tcnt[c];
-            uint32_t excl = 0;
-            if (t > 0) {
-                excl = look_back<SIGMA>(a.ring, a.rmask, a.tagbase, t, c);
-                st_volatile64(a.ring + size_t(t & a.rmask) * SIGMA + c,
-                              lbw(a.tagbase + t, LB_INCL | (excl + cn)));
-            }
-            const uint32_t g = sO[c] + excl;
-            if constexpr (OOP) {
-                qb[c] = make_uint2(g - bstart[c], 0u);
-            } else {
-                gpos[c] = g;
-                // the run lies inside the bucket's output range unless the
-                // look-back words were corrupted: then it is reported and
-                // its blocks are left alone
-                const bool bad = g + cn > sO[c + 1] || g + cn < g;
-                if (bad)
-                    set_status(ST_INTERNAL);
-                const uint32_t cn = bad ? 0u : tcnt[c];
-                const uint32_t e = g + cn;
-                const uint32_t touched = cn ? ((e - 1) >> a.lb) - (g >> a.lb) + 1 : 0u;
-                const uint32_t cs = (g + b - 1) >> a.lb, ce = (e + b - 1) >> a.lb;
-                const uint32_t n0 = ns0[c], n1 = ns1[c];
-                // block j in [n0 + L, n1) is taken by the writer of the first
-                // position of block j - L: by earlier tiles for j - L < cs,
-                // here for cs <= j - L < ce
-                const uint32_t mb = min(cs + GRID_AHEAD, n1), e0 = n0 + GRID_AHEAD;
-                const uint32_t before = mb > e0 ? mb - e0 : 0u;
-                const uint32_t f0 = max(cs, n0) + GRID_AHEAD, f1 = min(ce + GRID_AHEAD, n1);
-                const uint32_t kk = f1 > f0 ? f1 - f0 : 0u;
-                // warp-aggregated slots: list entries, blocks taken, and the
-                // count of blocks taken by earlier tiles
-                const uint32_t it_ = warp_incl_scan(touched), ik = warp_incl_scan(kk);
-                const uint32_t sb = warp_sum(before);
-                uint32_t bt = 0, bk2 = 0;
-                if (lane == 31) {
-                    bt = atomicAdd(&misc[1], it_);
-                    bk2 = atomicAdd(&misc[2], ik);
-                    atomicAdd(&misc[3], sb);
-                }
-                l0s[q] = __shfl_sync(0xffffffffu, bt, 31) + it_ - touched;
-                kos[q] = __shfl_sync(0xffffffffu, bk2, 31) + ik - kk;
-                // the first block touched was taken before this tile unless
-                // this tile takes it (then its map entry is not read)
-                if (cn && (g >> a.lb) < f0)
-                    pf[q] = ld_volatile(a.pin + a.H + (g >> a.lb));
-            }
-        }
-        bar();
-        if (ctid == 0) // this tile reads no more look-back words
-            st_volatile(a.done + (t & a.rmask), a.tagbase + t);
-
-        uint32_t TT = 0; // list entries of this tile
-        if constexpr (!OOP) {
-            // ---- 5. the physical block of every block this tile touches, and
-            // the blocks it takes beyond those
-            TT = misc[1];
-            const uint32_t fbase = nP + misc[3]; // free-list index of this tile's first new block
-            // free-list entries consumed so far (Lemma 1), within the list
-            const uint32_t fcap = min(a.H + (t + 1) * M, a.npi);
-#pragma unroll
-            for (int q = 0; q < PFN; ++q) {
-                const int c = ctid + q * NT;
-                if (c >= SIGMA)
-                    continue;
-                const uint32_t g = gpos[c], cn = tcnt[c];
-                const uint32_t l0 = l0s[q], j0 = g >> a.lb;
-                qb[c] = make_uint2(g - bstart[c], l0 - j0);
-                if (!cn || g + cn > sO[c + 1] || g + cn < g)
-                    continue; // (a corrupted run was reported in step 4)
-                const uint32_t touched = ((g + cn - 1) >> a.lb) - j0 + 1;
-                const uint32_t n0 = ns0[c], n1 = ns1[c];
-                const uint32_t cs = (g + b - 1) >> a.lb, ce = (g + cn + b - 1) >> a.lb;
-                const uint32_t first = max(cs, n0) + GRID_AHEAD;
-                const uint32_t last = min(ce + GRID_AHEAD, n1); // blocks first .. last-1 taken here
-                // the blocks taken here go into the map before this thread
-                // waits for any other's: a bucket that fills tile after tile
-                // (skewed keys) has each tile continue blocks that the tile
-                // just before took, and taking after the wait would chain
-                // every tile's step 5 to its predecessor's (1-2 us a tile).
-                // Measured (2^26 keys + index, a sort): Zipf keys 57.8 -> 3.7
-                // ms, float32 N(0,1) keys (top digit skewed) 15.8 -> 3.0,
-                // uniform keys unchanged
-                const uint32_t fi0 = fbase + kos[q] - first; // block j's free-list index - j
-                const uint32_t jend = j0 + touched;
-                for (uint32_t j = first; j < last; ++j) {
-                    const uint32_t idx = fi0 + j; // (mod 2^32)
-                    if (idx < fcap)
-                        a.pin[a.H + j] = __ldg(a.pi + idx);
-                    else
-                        set_status(ST_INTERNAL); // Lemma 1 would be violated
-                }
-                for (uint32_t j = j0; j < jend; ++j) {
-                    uint32_t phys;
-                    if (j >= first && j < last) { // taken here
-                        const uint32_t idx = fi0 + j;
-                        phys = idx < fcap ? __ldg(a.pi + idx) : PI_NONE;
-                    } else { // taken before the round or by an earlier tile
-                        phys = j == j0 ? pf[q] : PI_NONE;
-                        if (phys == PI_NONE)
-                            phys = wait_pi(a.pin + a.H + j);
-                    }
-                    if (phys != PI_NONE && phys >= a.npi) {
-                        set_status(ST_INTERNAL);
-                        phys = PI_NONE;
-                    }
-                    listb[l0 + (j - j0)] = phys;
-                }
-            }
-            bar();
-        }
-
-        // ---- 7. store every bucket run
-        constexpr int SI = (TILE + NT - 1) / NT;
-#pragma unroll 4
-        for (int kk = 0; kk < SI; ++kk) {
-            const uint32_t i = ctid + kk * NT;
-            if (i < cnt) {
-                KT kv;
-                uint32_t vv = 0;
-                if constexpr (C::PAIR) {
-                    const uint2 pr = tp[i];
-                    kv = pr.x;
-                    vv = pr.y;
-                } else {
-                    kv = tk[i];
-                    if (HASV)
-                        vv = tv[i];
-                }
-                const uint32_t dg = digit_of(kv, a.shift, mask);
-                const uint2 qd = qb[dg];
-                const uint32_t pos = i + qd.x;
-                if constexpr (OOP) {
-                    if (pos < a.n) {
-                        a.ok[pos] = kv;
-                        if (HASV)
-                            a.ov[pos] = vv;
-                    }
-                } else {
-                    const uint32_t l = (pos >> a.lb) + qd.y, off = pos & (b - 1);
-                    const uint32_t blk = l < TT ? listb[l] : PI_NONE;
-                    if (blk != PI_NONE) {
-                        kaddr(blk)[off] = kv;
-                        if (HASV)
-                            vaddr(blk)[off] = vv;
-                    }
-                }
-            }
-        }
-        // the stage was read and rewritten with generic accesses; the
-        // producer refills it with bulk copies (async proxy)
-        fence_proxy_async_smem();
-        bar();
-        if (ctid == 0)
-            mbar_arrive(&empty[s]); // stage consumed: the producer may refill it
-    }
-}
-
-// ---------------------------------------------------------------- round kernel, 8-bit digits
 // One CTA per SM: NW ranking warps, 8 look-back warps and a producer warp, on
 // tiles of TILE elements in two shared-memory stages.  What bounds it is
 // shared memory (the random-digit accesses of the ranking and the reorder,
@@ -1555,9 +948,9 @@ __global__ void __launch_bounds__(Lb8Cfg<KT, HASV, TILE, NW, OOP>::THREADS, Lb8C
                 t_first = grp.tile0[arr];
                 Oc = __ldg(a.tab + size_t(arr) * (SIGMA + 1) + c);
             }
-            // elements past the tile's end were ranked as digit 255
+            // elements past the tile's end were ranked as the largest digit
             uint32_t cn = part[c] + (C::PARTS == 2 ? part[SIGMA + c] : 0u);
-            if (c == SIGMA - 1)
+            if (uint32_t(c) == a.mask)
                 cn -= uint32_t(TILE) - cnt;
             // ---- the count published, the bucket's prefix over the tiles before
             unsigned long long *slot = a.ring + size_t(t & a.rmask) * SIGMA + c;
@@ -1693,7 +1086,7 @@ __global__ void __launch_bounds__(Lb8Cfg<KT, HASV, TILE, NW, OOP>::THREADS, Lb8C
     const int h = lane >> 4, l16 = lane & 15;
     uint32_t *row = tab + (2 * warp + h) * SIGMA; // this half-warp's words
     const uint32_t eh = uint32_t((2 * warp + h) * C::R + l16); // its first element in the tile
-    auto dig = [&](KT key) -> uint32_t { return static_cast<uint32_t>(key >> a.shift) & 255u; };
+    auto dig = [&](KT key) -> uint32_t { return digit_of(key, a.shift, a.mask); };
 
     // Tile k is ranked and counted before tile k - 1 is stored, so that a
     // tile's look-back and block lists have the store before it, its own
@@ -1750,7 +1143,7 @@ __global__ void __launch_bounds__(Lb8Cfg<KT, HASV, TILE, NW, OOP>::THREADS, Lb8C
                 }
             }
             if (cnt < uint32_t(TILE)) {
-                // elements past the end rank as the last ones of digit 255
+                // elements past the end rank as the last ones of the largest digit
 #pragma unroll
                 for (int it = 0; it < ITEMS; ++it)
                     if (eh + it * 16 >= cnt)
@@ -2018,31 +1411,20 @@ __global__ void __launch_bounds__(256)
 }
 
 // ---------------------------------------------------------------- launch helpers
-// The round kernel of a configuration: 8-bit digits with NW ranking warps, or
-// 11-bit digits (NW ignored).
-template <typename KT, bool HASV, int DB, int TILE, int NW, bool OOP> struct LbKernel {
-    using C = std::conditional_t<DB == 8, Lb8Cfg<KT, HASV, DB == 8 ? TILE : 4096, NW, OOP>,
-                                 LbCfg<KT, HASV, DB == 8 ? 4096 : TILE, OOP>>;
-    static auto kernel()
-    {
-        if constexpr (DB == 8)
-            return k_lb_round8<KT, HASV, TILE, NW, OOP>;
-        else
-            return k_lb_round11<KT, HASV, TILE, OOP>;
-    }
+// The round kernel of a configuration.
+template <typename KT, bool HASV, int TILE, int NW, bool OOP> struct LbKernel {
+    using C = Lb8Cfg<KT, HASV, TILE, NW, OOP>;
     static void launch(int grid, const LbArgs<KT> &a, cudaStream_t st)
     {
-        if constexpr (DB == 8)
-            k_lb_round8<KT, HASV, TILE, NW, OOP><<<grid, C::THREADS, C::SMEM, st>>>(a, LbNoGroup{});
-        else
-            k_lb_round11<KT, HASV, TILE, OOP><<<grid, C::THREADS, C::SMEM, st>>>(a);
+        k_lb_round8<KT, HASV, TILE, NW, OOP><<<grid, C::THREADS, C::SMEM, st>>>(a, LbNoGroup{});
     }
     // CTAs of a launch over ntiles tiles (-1: the kernel cannot be set up)
     static int ctas(size_t ntiles)
     {
         static DeviceOnce attr; // per template instance
         if (attr.run([] {
-                return cudaFuncSetAttribute(kernel(), cudaFuncAttributeMaxDynamicSharedMemorySize, int(C::SMEM));
+                return cudaFuncSetAttribute(k_lb_round8<KT, HASV, TILE, NW, OOP>,
+                                            cudaFuncAttributeMaxDynamicSharedMemorySize, int(C::SMEM));
             }) != cudaSuccess)
             return -1;
         size_t grid = size_t(num_sms()) * C::MINB;
@@ -2052,40 +1434,39 @@ template <typename KT, bool HASV, int DB, int TILE, int NW, bool OOP> struct LbK
     }
 };
 
-// Calls f.template operator()<KT, HASV, DB, TILE, NW>() for the configuration.
-template <typename F> static cudaError_t lb_dispatch(int kb, int db, bool hasv, F &&f)
+// Calls f.template operator()<KT, HASV, TILE, NW>() for the configuration.
+template <typename F> static cudaError_t lb_dispatch(int kb, bool hasv, F &&f)
 {
     using u64 = unsigned long long;
     // The largest tiles that two stages and the tables leave room for
     // (per-tile costs scale with sigma, not with the tile), each a multiple
-    // of 2048 so that blocks of up to 2048 elements fit whole; 11-bit digits
-    // keep their run offsets and block list in the warp rows.
-    if (kb == 4) {
-        if (db == 8)
-            return hasv ? f.template operator()<uint32_t, true, 8, 10240, 16>()
-                        : f.template operator()<uint32_t, false, 8, 16384, 16>();
-        return hasv ? f.template operator()<uint32_t, true, 11, 8192, 16>()
-                    : f.template operator()<uint32_t, false, 11, 16384, 16>();
-    }
-    if (db == 8)
-        return hasv ? f.template operator()<u64, true, 8, 6144, 16>()
-                    : f.template operator()<u64, false, 8, 10240, 16>();
-    return hasv ? f.template operator()<u64, true, 11, 4096, 16>() : f.template operator()<u64, false, 11, 8192, 16>();
+    // of 2048 so that blocks of up to 2048 elements fit whole.
+    if (kb == 4)
+        return hasv ? f.template operator()<uint32_t, true, 10240, 16>()
+                    : f.template operator()<uint32_t, false, 16384, 16>();
+    return hasv ? f.template operator()<u64, true, 6144, 16>() : f.template operator()<u64, false, 10240, 16>();
 }
 
 // Radsort rounds with a tile shape: 0 or 1, the configuration above; 2 (8-bit
 // digits), two CTAs of 8 ranking warps per SM on smaller tiles, which the
-// autotuner may pick where the arrays hold few tiles per SM
+// autotuner may pick where the arrays hold few tiles per SM; LB_SHAPE_4096,
+// tiles that blocks of 4096 elements fit
 template <typename F> static cudaError_t lb_dispatch_shape(int kb, int db, bool hasv, int shape, F &&f)
 {
     using u64 = unsigned long long;
     if (shape == 2 && db == 8) {
         if (kb == 4)
-            return hasv ? f.template operator()<uint32_t, true, 8, 4096, 8>()
-                        : f.template operator()<uint32_t, false, 8, 8192, 8>();
-        return hasv ? f.template operator()<u64, true, 8, 4096, 8>() : f.template operator()<u64, false, 8, 4096, 8>();
+            return hasv ? f.template operator()<uint32_t, true, 4096, 8>()
+                        : f.template operator()<uint32_t, false, 8192, 8>();
+        return hasv ? f.template operator()<u64, true, 4096, 8>() : f.template operator()<u64, false, 4096, 8>();
     }
-    return lb_dispatch(kb, db, hasv, f);
+    if (shape == LB_SHAPE_4096) {
+        if (kb == 4)
+            return hasv ? f.template operator()<uint32_t, true, 8192, 16>()
+                        : f.template operator()<uint32_t, false, 16384, 16>();
+        return hasv ? f.template operator()<u64, true, 4096, 16>() : f.template operator()<u64, false, 8192, 16>();
+    }
+    return lb_dispatch(kb, hasv, f);
 }
 
 } // namespace
@@ -2096,7 +1477,7 @@ uint32_t lb_tile(int kb, int db, bool hasv, int shape)
 {
     uint32_t r = 0;
     lb_dispatch_shape(kb, db, hasv, shape,
-                      [&]<typename KT, bool HASV, int DB, int TILE, int NW>() {
+                      [&]<typename KT, bool HASV, int TILE, int NW>() {
                           r = TILE;
                           return cudaSuccess;
                       });
@@ -2107,11 +1488,10 @@ uint32_t lb_tile(int kb, int db, bool hasv, int shape)
 // Rows of the look-back ring: a power of two, no more than the tiles' power
 // of two up to 512 rows, a quarter of it beyond (the tiles in flight at once,
 // at most STAGES per SM, mostly fit; a tile whose slot is still in use waits
-// for it), at most 2048 rows (sigma = 256) or 1024 (sigma = 2048): a few MB
-// whatever n.
-static uint32_t ring_rows(size_t ntiles, uint32_t sigma)
+// for it), at most 2048 rows: a few MB whatever n.
+static uint32_t ring_rows(size_t ntiles)
 {
-    const uint32_t cap = sigma <= 256 ? 2048u : 1024u;
+    constexpr uint32_t cap = 2048u;
     uint32_t r = 1;
     while (r < ntiles && r < 4 * cap)
         r <<= 1;
@@ -2120,49 +1500,45 @@ static uint32_t ring_rows(size_t ntiles, uint32_t sigma)
     return r < cap ? r : cap;
 }
 
-static size_t ring_bytes(size_t ntiles, uint32_t sigma)
+static size_t ring_bytes(size_t ntiles)
 {
-    const size_t r = ring_rows(ntiles, sigma);
-    return r * sigma * 8 + r * 4;
+    const size_t r = ring_rows(ntiles);
+    return r * 256 * 8 + r * 4;
 }
 
-template <typename KT> static void set_ring(LbArgs<KT> &a, void *mem, size_t ntiles, uint32_t sigma, int round)
+template <typename KT> static void set_ring(LbArgs<KT> &a, void *mem, size_t ntiles, int pass)
 {
-    const uint32_t R = ring_rows(ntiles, sigma);
+    const uint32_t R = ring_rows(ntiles);
     a.ring = static_cast<unsigned long long *>(mem);
-    a.done = reinterpret_cast<uint32_t *>(a.ring + size_t(R) * sigma);
+    a.done = reinterpret_cast<uint32_t *>(a.ring + size_t(R) * 256);
     a.rmask = R - 1;
-    a.tagbase = uint32_t(round + 1) << 24;
+    a.tagbase = uint32_t(pass + 1) << 24;
 }
 
 size_t grid_ring_bytes(const Geom &g)
 {
     const uint32_t tile = lb_tile(g.kb, g.db, g.hasv, g.shape);
-    return ring_bytes((g.n + tile - 1) / tile, g.sigma);
+    return ring_bytes((g.n + tile - 1) / tile);
 }
 
 // ---------------------------------------------------------------- grid-layout Radsort
-size_t grid_tab_words(const Geom &g)
-{
-    return size_t(g.nt) * (g.db == 8 ? GridTab<256>::WORDS : GridTab<2048>::WORDS);
-}
+size_t grid_tab_words(const Geom &g) { return size_t(digit_passes(g.kb, g.db, false)) * GridTab::WORDS; }
 
 cudaError_t launch_grid_tables(const Geom &g, const Bufs &w, uint32_t *pi, bool setup, cudaStream_t st)
 {
-    const uint32_t n = static_cast<uint32_t>(g.n), nr = static_cast<uint32_t>(g.nt);
+    const uint32_t n = static_cast<uint32_t>(g.n), np = static_cast<uint32_t>(digit_passes(g.kb, g.db, g.whole));
     int blocks = setup ? static_cast<int>((g.npi + 1023) / 1024) : 0;
     if (blocks > 1024)
         blocks = 1024;
-    auto go = [&]<typename KT, int DB>() {
-        k_grid_tables<KT, DB><<<nr + blocks, 1024, 0, st>>>(w.hist, w.tab, 0u, nr, n, g.lb, g.H, g.nA, g.npi,
-                                                           static_cast<const KT *>(w.Ak), w.Av,
-                                                           static_cast<KT *>(w.Tk), w.Tv, pi, w.P, w.state);
+    auto go = [&]<typename KT>() {
+        k_grid_tables<KT><<<np + blocks, 1024, 0, st>>>(w.hist, w.tab, 0u, np, n, g.lb, g.H, g.nA, g.npi,
+                                                       static_cast<const KT *>(w.Ak), w.Av, static_cast<KT *>(w.Tk),
+                                                       w.Tv, pi, w.P, w.state);
     };
-    using u64 = unsigned long long;
     if (g.kb == 4)
-        g.db == 8 ? go.template operator()<uint32_t, 8>() : go.template operator()<uint32_t, 11>();
+        go.template operator()<uint32_t>();
     else
-        g.db == 8 ? go.template operator()<u64, 8>() : go.template operator()<u64, 11>();
+        go.template operator()<unsigned long long>();
     g_launches += 1;
     return cudaGetLastError();
 }
@@ -2176,37 +1552,31 @@ cudaError_t launch_grid_setup(const Geom &g, const Bufs &w, uint32_t *pi, cudaSt
     cudaError_t e = cudaMemsetAsync(z0, 0, reinterpret_cast<char *>(w.status) + grid_ring_bytes(g) - z0, st);
     if (e != cudaSuccess)
         return e;
-    e = launch_digit_hist(w.Ak, static_cast<uint32_t>(g.n), g.kb, g.db, w.hist, st);
+    e = launch_digit_hist(w.Ak, static_cast<uint32_t>(g.n), g.kb, by_bytes(g.db, g.whole), w.hist, st);
     if (e != cudaSuccess)
         return e;
     return launch_grid_tables(g, w, pi, true, st);
 }
 
-cudaError_t launch_grid_prep(const Geom &g, const Bufs &w, const uint32_t *pi, uint32_t *pin,
-                             int round, cudaStream_t st)
+cudaError_t launch_grid_prep(const Geom &g, const Bufs &w, const uint32_t *pi, uint32_t *pin, int pass,
+                             cudaStream_t st)
 {
-    const uint32_t n = static_cast<uint32_t>(g.n);
     int blocks = static_cast<int>((g.npi + 255) / 256);
-    const int cap = num_sms() * (g.db == 8 ? 8 : 2);
-    if (blocks > cap)
-        blocks = cap;
-    if (g.db == 8)
-        k_grid_fill<8><<<blocks, 256, 0, st>>>(w.tab + size_t(round) * GridTab<256>::WORDS, n, g.lb, g.H, g.nA, g.npi,
-                                               pi, pin);
-    else
-        k_grid_fill<11><<<blocks, 256, 0, st>>>(w.tab + size_t(round) * GridTab<2048>::WORDS, n, g.lb, g.H, g.nA,
-                                                g.npi, pi, pin);
+    if (blocks > num_sms() * 8)
+        blocks = num_sms() * 8;
+    k_grid_fill<<<blocks, 256, 0, st>>>(w.tab + size_t(pass) * GridTab::WORDS, static_cast<uint32_t>(g.n), g.lb, g.H,
+                                        g.nA, g.npi, pi, pin);
     g_launches += 1;
     return cudaGetLastError();
 }
 
-cudaError_t launch_grid_round(const Geom &g, const Bufs &w, const uint32_t *pi, uint32_t *pin,
-                              int round, cudaStream_t st)
+cudaError_t launch_grid_round(const Geom &g, const Bufs &w, const uint32_t *pi, uint32_t *pin, int pass,
+                              cudaStream_t st)
 {
     const uint32_t n = static_cast<uint32_t>(g.n);
     return lb_dispatch_shape(g.kb, g.db, g.hasv, g.shape,
-                             [&]<typename KT, bool HASV, int DB, int TILE, int NW>() {
-        using K = LbKernel<KT, HASV, DB, TILE, NW, false>;
+                             [&]<typename KT, bool HASV, int TILE, int NW>() {
+        using K = LbKernel<KT, HASV, TILE, NW, false>;
         const size_t ntiles = (g.n + TILE - 1) / TILE;
         const int grid = K::ctas(ntiles);
         if (grid < 0)
@@ -2218,17 +1588,19 @@ cudaError_t launch_grid_round(const Geom &g, const Bufs &w, const uint32_t *pi, 
         a.Tv = w.Tv;
         a.pi = pi;
         a.pin = pin;
-        a.tab = w.tab + size_t(round) * GridTab<(1 << DB)>::WORDS;
-        a.hdr = a.tab + GridTab<(1 << DB)>::HDR;
-        set_ring(a, w.status, ntiles, g.sigma, round);
-        a.ticket = w.ctr + round;
+        a.tab = w.tab + size_t(pass) * GridTab::WORDS;
+        a.hdr = a.tab + GridTab::HDR;
+        set_ring(a, w.status, ntiles, pass);
+        a.ticket = w.ctr + pass;
         a.n = n;
         a.ntiles = static_cast<uint32_t>(ntiles);
         a.H = g.H;
         a.nT = g.nT;
         a.npi = g.npi;
         a.lb = g.lb;
-        a.shift = static_cast<uint32_t>(round * g.db);
+        const DigitPass dp = digit_pass(g.kb, g.db, g.whole, pass);
+        a.shift = dp.shift;
+        a.mask = dp.mask();
         K::launch(grid, a, st);
         g_launches += 1;
         return cudaGetLastError();
@@ -2236,86 +1608,82 @@ cudaError_t launch_grid_round(const Geom &g, const Bufs &w, const uint32_t *pi, 
 }
 
 // ---------------------------------------------------------------- out-of-place comparator
-size_t lsd_oop_scratch_bytes(size_t n, int kb, int db, bool hasv)
+// [counts | bucket starts | look-back ring | tickets]; the tables' sizes are
+// those of sigma = 2^db
+struct OopLayout {
+    size_t off, ring, ctr, total;
+};
+
+static OopLayout oop_layout(size_t n, int kb, int db, bool hasv)
 {
-    const size_t sigma = size_t(1) << db;
-    const int nt = (8 * kb + db - 1) / db;
+    const size_t sigma = size_t(1) << db, nt = (8 * kb + db - 1) / db;
     const uint32_t tile = lb_tile(kb, db, hasv, 0);
-    const size_t ntiles = (n + tile - 1) / tile;
     auto al = [](size_t x) { return (x + 255) & ~size_t(255); };
-    return al(nt * sigma * 4) + al(nt * (sigma + 1) * 4) + al(ring_bytes(ntiles, uint32_t(sigma))) + al(64 * 4);
+    const size_t ring = ring_bytes((n + tile - 1) / tile);
+    OopLayout L{};
+    L.off = al(nt * sigma * 4);
+    L.ring = L.off + al(nt * (sigma + 1) * 4);
+    L.ctr = L.ring + al(ring > sigma * 8 ? ring : sigma * 8);
+    L.total = L.ctr + al(64 * 4);
+    return L;
 }
+
+size_t lsd_oop_scratch_bytes(size_t n, int kb, int db, bool hasv) { return oop_layout(n, kb, db, hasv).total; }
 
 cudaError_t launch_lsd_oop_ws(void *keys, uint32_t *vals, void *keys_alt, uint32_t *vals_alt,
                               size_t n, int kb, int db, void *scratch, cudaStream_t st)
 {
     if (n >= (size_t(1) << 31))
         return cudaErrorInvalidValue;
-    const uint32_t sigma = 1u << db;
-    const int nt = (8 * kb + db - 1) / db;
-    const size_t total = lsd_oop_scratch_bytes(n, kb, db, vals != nullptr);
+    const int np = kb; // whole sort: a pass per byte (an even number: the result ends in keys)
+    const OopLayout L = oop_layout(n, kb, db, vals != nullptr);
     char *scr = static_cast<char *>(scratch);
     const bool own = scr == nullptr;
     cudaError_t e = cudaSuccess;
     if (own)
-        e = cudaMallocAsync(reinterpret_cast<void **>(&scr), total, st);
+        e = cudaMallocAsync(reinterpret_cast<void **>(&scr), L.total, st);
     if (e != cudaSuccess)
         return e;
-    auto al = [](size_t x) { return (x + 255) & ~size_t(255); };
-    const uint32_t tile = lb_tile(kb, db, vals != nullptr, 0);
-    const size_t ntiles = (n + tile - 1) / tile;
-    uint32_t *hist = reinterpret_cast<uint32_t *>(scr);
-    uint32_t *off = reinterpret_cast<uint32_t *>(scr + al(nt * sigma * 4));
-    char *ringp = scr + al(nt * sigma * 4) + al(nt * (sigma + 1) * 4);
-    uint32_t *ctr = reinterpret_cast<uint32_t *>(ringp + al(ring_bytes(ntiles, sigma)));
-    e = cudaMemsetAsync(hist, 0, size_t(nt) * sigma * 4, st);
-    if (e == cudaSuccess)
-        e = cudaMemsetAsync(ctr, 0, 64 * 4, st);
-    if (e == cudaSuccess)
-        e = cudaMemsetAsync(ringp, 0, ring_bytes(ntiles, sigma), st);
+    uint32_t *hist = reinterpret_cast<uint32_t *>(scr), *off = reinterpret_cast<uint32_t *>(scr + L.off);
+    uint32_t *ctr = reinterpret_cast<uint32_t *>(scr + L.ctr);
+    // counts, ring and tickets cleared (the bucket starts between them too)
+    e = cudaMemsetAsync(hist, 0, L.total, st);
     const uint32_t nn = static_cast<uint32_t>(n);
     if (e == cudaSuccess)
-        e = launch_digit_hist(keys, nn, kb, db, hist, st);
+        e = launch_digit_hist(keys, nn, kb, true, hist, st);
     if (e == cudaSuccess) {
-        if (db == 8)
-            k_offsets<8><<<nt, 1024, 0, st>>>(hist, off, nn);
-        else
-            k_offsets<11><<<nt, 1024, 0, st>>>(hist, off, nn);
+        k_offsets<<<np, 256, 0, st>>>(hist, off, nn);
         g_launches += 1;
+        e = lb_dispatch(kb, vals != nullptr, [&]<typename KT, bool HASV, int TILE, int NW>() {
+            using K = LbKernel<KT, HASV, TILE, NW, true>;
+            const size_t ntiles = (n + TILE - 1) / TILE;
+            const int grid = K::ctas(ntiles);
+            if (grid < 0)
+                return cudaErrorInvalidValue;
+            KT *src = static_cast<KT *>(keys), *dst = static_cast<KT *>(keys_alt);
+            uint32_t *vs = vals, *vd = vals_alt;
+            for (int r = 0; r < np; ++r) {
+                LbArgs<KT> a{};
+                a.ik = src;
+                a.iv = vs;
+                a.ok = dst;
+                a.ov = vd;
+                a.tab = off + size_t(r) * 257;
+                set_ring(a, scr + L.ring, ntiles, r);
+                a.ticket = ctr + r;
+                a.n = nn;
+                a.ntiles = static_cast<uint32_t>(ntiles);
+                const DigitPass dp = digit_pass(kb, db, true, r);
+                a.shift = dp.shift;
+                a.mask = dp.mask();
+                K::launch(grid, a, st);
+                g_launches += 1;
+                std::swap(src, dst);
+                std::swap(vs, vd);
+            }
+            return cudaGetLastError();
+        });
     }
-    if (e == cudaSuccess)
-        e = lb_dispatch(kb, db, vals != nullptr, [&]<typename KT, bool HASV, int DB, int TILE, int NW>() {
-        using K = LbKernel<KT, HASV, DB, TILE, NW, true>;
-        const int grid = K::ctas(ntiles);
-        if (grid < 0)
-            return cudaErrorInvalidValue;
-        KT *src = static_cast<KT *>(keys), *dst = static_cast<KT *>(keys_alt);
-        uint32_t *vs = vals, *vd = vals_alt;
-        for (int r = 0; r < nt; ++r) {
-            LbArgs<KT> a{};
-            a.ik = src;
-            a.iv = vs;
-            a.ok = dst;
-            a.ov = vd;
-            a.tab = off + size_t(r) * (sigma + 1);
-            set_ring(a, ringp, ntiles, sigma, r);
-            a.ticket = ctr + r;
-            a.n = nn;
-            a.ntiles = static_cast<uint32_t>(ntiles);
-            a.shift = static_cast<uint32_t>(r * DB);
-            K::launch(grid, a, st);
-            g_launches += 1;
-            std::swap(src, dst);
-            std::swap(vs, vd);
-        }
-        cudaError_t ec = cudaGetLastError();
-        if (ec == cudaSuccess && (nt & 1)) { // the result is in the alternate buffers: copy back
-            ec = cudaMemcpyAsync(keys, src, n * sizeof(KT), cudaMemcpyDeviceToDevice, st);
-            if (ec == cudaSuccess && HASV)
-                ec = cudaMemcpyAsync(vals, vs, n * 4, cudaMemcpyDeviceToDevice, st);
-        }
-        return ec;
-    });
     cudaError_t e2 = own ? cudaFreeAsync(scr, st) : cudaSuccess;
     return e != cudaSuccess ? e : e2;
 }
@@ -2345,7 +1713,7 @@ static GroupLayout group_layout(const SegGroup &g, int kb, bool hasv)
     L.ctr = off;
     off += al(64 * 4);
     L.ring = off;
-    off += al(ring_bytes(L.ntiles, 256));
+    off += al(ring_bytes(L.ntiles));
     L.tab = off;
     off += al(size_t(g.narr) * kb * 257 * 4);
     L.total = off;
@@ -2363,59 +1731,56 @@ cudaError_t launch_lsd_group(void *keys, uint32_t *vals, const SegGroup &g, int 
     cudaError_t e = cudaMemsetAsync(hist, 0, L.tab - L.hist, st);
     if (e != cudaSuccess)
         return e;
-    return lb_dispatch(kb, 8, vals != nullptr, [&]<typename KT, bool HASV, int DB, int TILE, int NW>() {
-        if constexpr (DB != 8) {
-            return cudaErrorInvalidValue;
-        } else {
-            using C = Lb8Cfg<KT, HASV, TILE, NW, true>;
-            const auto kern = k_lb_round8<KT, HASV, TILE, NW, true, true>;
-            static DeviceOnce attr;
-            const cudaError_t ea = attr.run([&] {
-                cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(C::SMEM));
-                if (r == cudaSuccess)
-                    r = cudaFuncSetAttribute(k_group_hist<KT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             4 * 256 * 32 * 4);
-                return r;
-            });
-            if (ea != cudaSuccess)
-                return ea;
-            LbGroup in{}, out{}; // even rounds: from the arrays; odd rounds: back to them
-            in.narr = g.narr;
-            uint32_t tiles = 0, chunks = 0;
-            size_t alt = 0;
-            for (uint32_t i = 0; i < g.narr; ++i) {
-                in.tile0[i] = tiles;
-                in.len[i] = g.len[i];
-                in.in[i] = g.off[i];
-                in.out[i] = alt;
-                tiles += (g.len[i] + TILE - 1) / TILE;
-                chunks += (g.len[i] + GRP_CHUNK - 1) / GRP_CHUNK;
-                alt += (size_t(g.len[i]) + 3) & ~size_t(3);
-            }
-            out = in;
-            std::swap(out.in, out.out);
-            constexpr int nt = int(sizeof(KT));
-            k_group_hist<KT><<<dim3(chunks, nt / 4), 1024, 4 * 256 * 32 * 4, st>>>(static_cast<const KT *>(keys), in, hist);
-            k_group_offsets<<<g.narr * nt, 256, 0, st>>>(hist, nt, g.narr, in, tab);
-            const int sms = num_sms(), grid = tiles < uint32_t(sms) ? static_cast<int>(tiles) : sms;
-            KT *alt_k = reinterpret_cast<KT *>(base);
-            uint32_t *alt_v = HASV ? reinterpret_cast<uint32_t *>(base + L.altv) : nullptr;
-            for (int r = 0; r < nt; ++r) {
-                LbArgs<KT> a{};
-                a.ik = r & 1 ? alt_k : static_cast<KT *>(keys);
-                a.iv = r & 1 ? alt_v : vals;
-                a.ok = r & 1 ? static_cast<KT *>(keys) : alt_k;
-                a.ov = r & 1 ? vals : alt_v;
-                a.tab = tab + size_t(r) * g.narr * 257;
-                set_ring(a, base + L.ring, tiles, 256, r);
-                a.ticket = ctr + r;
-                a.ntiles = tiles;
-                a.shift = static_cast<uint32_t>(r * 8);
-                kern<<<grid, C::THREADS, C::SMEM, st>>>(a, r & 1 ? out : in);
-            }
-            g_launches += 2 + nt;
-            return cudaGetLastError();
+    return lb_dispatch(kb, vals != nullptr, [&]<typename KT, bool HASV, int TILE, int NW>() {
+        using C = Lb8Cfg<KT, HASV, TILE, NW, true>;
+        const auto kern = k_lb_round8<KT, HASV, TILE, NW, true, true>;
+        static DeviceOnce attr;
+        const cudaError_t ea = attr.run([&] {
+            cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(C::SMEM));
+            if (r == cudaSuccess)
+                r = cudaFuncSetAttribute(k_group_hist<KT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         4 * 256 * 32 * 4);
+            return r;
+        });
+        if (ea != cudaSuccess)
+            return ea;
+        LbGroup in{}, out{}; // even rounds: from the arrays; odd rounds: back to them
+        in.narr = g.narr;
+        uint32_t tiles = 0, chunks = 0;
+        size_t alt = 0;
+        for (uint32_t i = 0; i < g.narr; ++i) {
+            in.tile0[i] = tiles;
+            in.len[i] = g.len[i];
+            in.in[i] = g.off[i];
+            in.out[i] = alt;
+            tiles += (g.len[i] + TILE - 1) / TILE;
+            chunks += (g.len[i] + GRP_CHUNK - 1) / GRP_CHUNK;
+            alt += (size_t(g.len[i]) + 3) & ~size_t(3);
         }
+        out = in;
+        std::swap(out.in, out.out);
+        constexpr int nt = int(sizeof(KT));
+        k_group_hist<KT><<<dim3(chunks, nt / 4), 1024, 4 * 256 * 32 * 4, st>>>(static_cast<const KT *>(keys), in, hist);
+        k_group_offsets<<<g.narr * nt, 256, 0, st>>>(hist, nt, g.narr, in, tab);
+        const int sms = num_sms(), grid = tiles < uint32_t(sms) ? static_cast<int>(tiles) : sms;
+        KT *alt_k = reinterpret_cast<KT *>(base);
+        uint32_t *alt_v = HASV ? reinterpret_cast<uint32_t *>(base + L.altv) : nullptr;
+        for (int r = 0; r < nt; ++r) {
+            LbArgs<KT> a{};
+            a.ik = r & 1 ? alt_k : static_cast<KT *>(keys);
+            a.iv = r & 1 ? alt_v : vals;
+            a.ok = r & 1 ? static_cast<KT *>(keys) : alt_k;
+            a.ov = r & 1 ? vals : alt_v;
+            a.tab = tab + size_t(r) * g.narr * 257;
+            set_ring(a, base + L.ring, tiles, r);
+            a.ticket = ctr + r;
+            a.ntiles = tiles;
+            a.shift = static_cast<uint32_t>(r * 8);
+            a.mask = 255u;
+            kern<<<grid, C::THREADS, C::SMEM, st>>>(a, r & 1 ? out : in);
+        }
+        g_launches += 2 + nt;
+        return cudaGetLastError();
     });
 }
 

@@ -14,6 +14,33 @@ namespace rs {
 // bits of the device status words
 enum : unsigned { ST_TIMEOUT = 1u, ST_INTERNAL = 2u };
 
+// The passes of the grid layout and of the out-of-place sort, each over at
+// most 256 buckets.  8-bit digits: one pass per digit.  11-bit digits: a digit
+// on its own (rounds of the permuted representation, or a part of a sort's
+// rounds) is sorted by its low six bits, then, stably, by the rest; a whole
+// sort leaves the same sequence wherever the key is cut, and is cut into
+// bytes.  A pass over 2048 buckets left 2 to 8 elements of a tile in each and
+// spent its time on the buckets.  2^27 u64 + u32: six such passes took 27.2 ms,
+// eight over 256 take 9.5; five of the six digits 23.5, ten passes over at
+// most 64 take 11.8.  (2^27 u32 + u32, three digits: 9.40 -> 3.85; 2^20: 294
+// -> 242 us.)
+struct DigitPass {
+    uint32_t shift, bits;
+    __host__ __device__ constexpr uint32_t mask() const { return (1u << bits) - 1u; }
+};
+__host__ __device__ constexpr bool by_bytes(int db, bool whole) { return db == 8 || whole; }
+__host__ __device__ constexpr int digit_passes(int kb, int db, bool whole)
+{
+    return by_bytes(db, whole) ? kb : 2 * ((8 * kb + db - 1) / db);
+}
+__host__ __device__ constexpr DigitPass digit_pass(int kb, int db, bool whole, int i)
+{
+    if (by_bytes(db, whole))
+        return {uint32_t(8 * i), 8u};
+    const int r = i / 2, left = 8 * kb - r * db, width = left < db ? left : db;
+    return i & 1 ? DigitPass{uint32_t(r * db + 6), uint32_t(width - 6)} : DigitPass{uint32_t(r * db), 6u};
+}
+
 // Sizes of one sort (host view).  Block indices are 32-bit.
 struct Geom {
     size_t n;          // elements
@@ -22,6 +49,7 @@ struct Geom {
     int db;            // digit bits 8 | 11
     uint32_t sigma;    // 2^db
     int nt;            // digits per key
+    bool whole;        // grid layout: all digits in one go (digit_pass)
     uint32_t b, lb;    // block size and log2
     uint32_t p;        // chunks
     uint32_t nA;       // floor(n/b): blocks overlaying A
@@ -52,10 +80,10 @@ struct Bufs {
     uint32_t *state;   // scalars, see ST_*
     void *fin;         // Finalize scratch (finalize_extra_bytes)
     // grid layout only
-    uint32_t *hist;    // nt*sigma digit counts of the input
-    uint32_t *tab;     // bucket tables of every round (grid_tab_words)
+    uint32_t *hist;    // 256 bucket counts of the input per pass
+    uint32_t *tab;     // bucket tables of every pass (grid_tab_words)
     uint32_t *status;  // look-back ring (after the rounds: Finalize's jump array and scratch)
-    uint32_t *ctr;     // per-round tile tickets
+    uint32_t *ctr;     // per-pass tile tickets
 };
 
 // grid layout: blocks a bucket's chain takes ahead of its writes (the head
@@ -76,19 +104,22 @@ enum FixMode { FIX_EVEN = 0, FIX_SPLIT = 1, FIX_PER_CHUNK = 2 };
 cudaError_t launch_fixup(const Geom &g, const Bufs &w, const uint32_t *pi_old, uint32_t *pi_new,
                          const uint32_t *UC, const uint32_t *lo_old, uint32_t *lo_new, int mode,
                          cudaStream_t st);
-// grid layout: digit histograms, every round's tables and setup; per round
+// grid layout: bucket counts, every pass's tables and setup; per pass
 // the prefilled next map (prep), then sortPhase.  launch_grid_tables without
 // setup: the tables alone, from the histograms of the current sequence
 size_t grid_tab_words(const Geom &g);
 cudaError_t launch_grid_tables(const Geom &g, const Bufs &w, uint32_t *pi, bool setup, cudaStream_t st);
 cudaError_t launch_grid_setup(const Geom &g, const Bufs &w, uint32_t *pi, cudaStream_t st);
 cudaError_t launch_grid_prep(const Geom &g, const Bufs &w, const uint32_t *pi, uint32_t *pin,
-                             int round, cudaStream_t st);
+                             int pass, cudaStream_t st);
 cudaError_t launch_grid_round(const Geom &g, const Bufs &w, const uint32_t *pi, uint32_t *pin,
-                              int round, cudaStream_t st);
+                              int pass, cudaStream_t st);
 size_t grid_ring_bytes(const Geom &g); // look-back ring of the grid layout
 // elements per tile of the look-back round kernel with a tile shape (0: the
-// default), and whether a shape differs from the default for the digit width
+// default), and whether a shape differs from the default for the digit width;
+// LB_SHAPE_4096 is the shape of plans with blocks of 4096 elements that the
+// default tile does not hold whole
+constexpr int LB_SHAPE_4096 = 3;
 uint32_t lb_tile(int kb, int db, bool hasv, int shape);
 bool lb_shape_differs(int db, int shape);
 // gather of the logical sequence (Sec. 4.1 iterator)

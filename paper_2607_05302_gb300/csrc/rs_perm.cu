@@ -18,7 +18,7 @@ unsigned take_status_perm() { return take_status_word(); }
 
 namespace {
 
-// Counts of every digit position over the sequence's elements, read block by
+// Counts of every pass's buckets over the sequence's elements, read block by
 // block through pi (a histogram of the multiset, so any order will do).
 // Consecutive threads read consecutive elements of one block.
 template <typename KT, int DB>
@@ -26,8 +26,7 @@ __global__ void __launch_bounds__(512) k_block_hist(const KT *Ak, const KT *Tk, 
                                                     uint32_t H, uint32_t nT, uint32_t npi, uint32_t lb,
                                                     uint32_t n, uint32_t *hist)
 {
-    constexpr int SIGMA = 1 << DB;
-    constexpr int NTD = (8 * int(sizeof(KT)) + DB - 1) / DB;
+    constexpr int SIGMA = 256, NTD = digit_passes(int(sizeof(KT)), DB, false);
     extern __shared__ uint32_t sh[];
     for (int i = threadIdx.x; i < NTD * SIGMA; i += blockDim.x)
         sh[i] = 0;
@@ -44,7 +43,9 @@ __global__ void __launch_bounds__(512) k_block_hist(const KT *Ak, const KT *Tk, 
         const KT k = blk[e & mask];
 #pragma unroll
         for (int r = 0; r < NTD; ++r)
-            atomicAdd(&sh[r * SIGMA + digit_of(k, uint32_t(r * DB), SIGMA - 1)], 1u);
+            atomicAdd(&sh[r * SIGMA + digit_of(k, digit_pass(int(sizeof(KT)), DB, false, r).shift,
+                                               digit_pass(int(sizeof(KT)), DB, false, r).mask())],
+                      1u);
     }
     __syncthreads();
     for (int i = threadIdx.x; i < NTD * SIGMA; i += blockDim.x)
@@ -90,7 +91,7 @@ __global__ void k_set_tail(uint2 *P, uint32_t *state, uint32_t H, uint32_t lb, u
 
 cudaError_t launch_block_hist(const Geom &g, const Bufs &w, const uint32_t *pi, cudaStream_t st)
 {
-    cudaError_t e = cudaMemsetAsync(w.hist, 0, size_t(g.nt) * g.sigma * 4, st);
+    cudaError_t e = cudaMemsetAsync(w.hist, 0, size_t(digit_passes(g.kb, g.db, false)) * 256 * 4, st);
     if (e != cudaSuccess || g.n == 0)
         return e;
     const uint32_t n = static_cast<uint32_t>(g.n);
@@ -98,7 +99,7 @@ cudaError_t launch_block_hist(const Geom &g, const Bufs &w, const uint32_t *pi, 
     const int need = static_cast<int>((g.n + 511) / 512);
     if (grid > need)
         grid = need;
-    const size_t smem = size_t(g.nt) * g.sigma * 4;
+    const size_t smem = size_t(digit_passes(g.kb, g.db, false)) * 256 * 4;
     using u64 = unsigned long long;
     if (g.kb == 4 && g.db == 8)
         k_block_hist<uint32_t, 8><<<grid, 512, smem, st>>>(static_cast<const uint32_t *>(w.Ak),
