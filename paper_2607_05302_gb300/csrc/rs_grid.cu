@@ -622,7 +622,8 @@ template <typename KT, bool HASV, int TILE, int NW, bool OOP> struct Lb8Cfg {
     static constexpr int SIGMA = 256, STAGES = 2;
     static constexpr int NT = NW * 32;             // ranking threads
     static constexpr int NA = SIGMA;               // look-back threads, one per bucket
-    static constexpr int THREADS = NT + NA + 128;  // + the producer's warpgroup (one warp works)
+    static constexpr int THREADS = NT + NA + 128;  // + the producer's warpgroup
+    static constexpr int NPW = OOP ? 1 : 4;        // its warps that work
     static constexpr int SROWS = 2 * NW;           // half-warps
     static constexpr int R = TILE / SROWS;         // elements ranked per half-warp
     static constexpr int ITEMS = R / 16;           // elements per ranking thread
@@ -677,7 +678,7 @@ template <int N> __device__ __forceinline__ void reg_inc()
 }
 
 // named barriers of k_lb_round8
-enum { LB8_MAIN = 1, LB8_AUX = 2, LB8_CNT = 3, LB8_SCAN = 4, LB8_LIST = 5, LB8_FREE = 6 };
+enum { LB8_MAIN = 1, LB8_AUX = 2, LB8_CNT = 3, LB8_SCAN = 4, LB8_LIST = 5, LB8_FREE = 6, LB8_PROD = 7 };
 
 // Several arrays sorted out of place in one launch per round (GRP): their
 // tiles follow one another, array by array, and the first tile of each has the
@@ -714,7 +715,7 @@ __global__ void __launch_bounds__(Lb8Cfg<KT, HASV, TILE, NW, OOP>::THREADS, Lb8C
 
     if (tid == 0) {
         for (int s = 0; s < C::STAGES; ++s) {
-            mbar_init(&full[s], 1);
+            mbar_init(&full[s], C::NPW);
             meta[s * 4] = TILE_END;
         }
         misc[0] = misc[1] = 0;
@@ -730,7 +731,8 @@ __global__ void __launch_bounds__(Lb8Cfg<KT, HASV, TILE, NW, OOP>::THREADS, Lb8C
     if (warp >= NW + SIGMA / 32) {
         // ============================================================ producer
         reg_dec<C::PROD_REGS>();
-        if (warp > NW + SIGMA / 32)
+        const int pw = warp - (NW + SIGMA / 32); // the first draws tickets, all copy (Radsort: a block each lane)
+        if (pw >= C::NPW)
             return;
         auto kaddr = [&](uint32_t blk) -> KT * {
             return blk < a.nT ? a.Tk + (size_t(blk) << a.lb) : a.Ak + (size_t(blk - a.nT) << a.lb);
@@ -739,17 +741,22 @@ __global__ void __launch_bounds__(Lb8Cfg<KT, HASV, TILE, NW, OOP>::THREADS, Lb8C
             return blk < a.nT ? a.Tv + (size_t(blk) << a.lb) : a.Av + (size_t(blk - a.nT) << a.lb);
         };
         // fill fk (this CTA's tile fk) goes to stage fk % 2
-        uint32_t ft = 0, fphys = 0, wm = 0; // drawn ticket; its block `lane`; tiles below wm have looked back
-        auto draw = [&]() {
+        uint32_t ft = 0, fphys = 0, wm = 0; // drawn ticket; its block bi; tiles below wm have looked back
+        const uint32_t bi = uint32_t(lane * C::NPW + pw);
+        auto draw = [&](int fk) {
             uint32_t t = 0;
-            if (lane == 0)
+            if (pw == 0 && lane == 0)
                 t = atomicAdd(a.ticket, 1u);
             ft = __shfl_sync(0xffffffffu, t, 0);
             if constexpr (!OOP) {
+                if (pw == 0 && lane == 0)
+                    misc[2 + (fk & 1)] = ft;
+                named_bar(LB8_PROD, C::NPW * 32);
+                ft = misc[2 + (fk & 1)];
                 if (ft < a.ntiles) {
                     const uint32_t cnt = min(uint32_t(TILE), a.n - ft * uint32_t(TILE));
                     const uint32_t nb = (cnt + b - 1) >> a.lb;
-                    fphys = uint32_t(lane) < nb ? a.pi[a.H + ft * (uint32_t(TILE) >> a.lb) + lane] : 0u;
+                    fphys = bi < nb ? a.pi[a.H + ft * (uint32_t(TILE) >> a.lb) + bi] : 0u;
                 }
             }
         };
@@ -780,7 +787,8 @@ __global__ void __launch_bounds__(Lb8Cfg<KT, HASV, TILE, NW, OOP>::THREADS, Lb8C
             uint32_t *mt = meta + s * 4;
             if (ft >= a.ntiles) { // the end mark
                 if (lane == 0) {
-                    mt[0] = TILE_END;
+                    if (pw == 0)
+                        mt[0] = TILE_END;
                     mbar_arrive(&full[s]);
                 }
                 return;
@@ -857,8 +865,8 @@ __global__ void __launch_bounds__(Lb8Cfg<KT, HASV, TILE, NW, OOP>::THREADS, Lb8C
                 const uint32_t nb = (cnt + b - 1) >> a.lb;
                 const uint32_t i0 = a.H + ft * (uint32_t(TILE) >> a.lb);
                 uint32_t tot = 0;
-                for (uint32_t base = 0; base < nb; base += 32) {
-                    const uint32_t i = base + lane;
+                for (uint32_t base = 0; base < nb; base += 32 * C::NPW) {
+                    const uint32_t i = base + bi;
                     uint32_t bytes = 0;
                     if (i < nb && (base ? a.pi[i0 + i] : fphys) < a.npi) {
                         const uint32_t len = min(b, cnt - i * b);
@@ -871,9 +879,9 @@ __global__ void __launch_bounds__(Lb8Cfg<KT, HASV, TILE, NW, OOP>::THREADS, Lb8C
                                  "r"(tot)
                                  : "memory");
                 __syncwarp();
-                for (uint32_t i = lane; i < nb; i += 32) {
+                for (uint32_t i = bi; i < nb; i += 32 * C::NPW) {
                     const uint32_t len = min(b, cnt - i * b);
-                    const uint32_t phys = i < 32 ? fphys : a.pi[i0 + i];
+                    const uint32_t phys = i == bi ? fphys : a.pi[i0 + i];
                     if (phys >= a.npi) {
                         set_status(ST_INTERNAL);
                         continue;
@@ -884,7 +892,7 @@ __global__ void __launch_bounds__(Lb8Cfg<KT, HASV, TILE, NW, OOP>::THREADS, Lb8C
                 }
             }
             __syncwarp();
-            if (lane == 0) {
+            if (pw == 0 && lane == 0) {
                 mt[0] = ft;
                 mt[1] = cnt;
                 mt[2] = leadk | (leadv << 8);
@@ -894,21 +902,32 @@ __global__ void __launch_bounds__(Lb8Cfg<KT, HASV, TILE, NW, OOP>::THREADS, Lb8C
             if (lane == 0)
                 mbar_arrive(&full[s]); // release: the plain stores above are visible
         };
+        // Radsort: the copies of a fill, two a block, are dealt over the four
+        // warps, as a warp issues its lanes' copies one after the other, about
+        // 0.12 us each: 4.8 us of the 8.4 us a tile with blocks of 512.  A round
+        // of 2^20 u32 + u32 23.0 -> 21.3 us, 2^24 110 -> 105 us (blocks of 512),
+        // 2^28 unchanged (blocks of 2048).  (2^26 with Zipf keys, whose tiles
+        // take unequal times: 2.78 -> 2.82 ms a sort.)
         // The ticket of fill k + 1 is drawn when tile k is counted, not before:
         // every look-back waits for the tiles drawn earlier, and a CTA that
         // drew two tiles in a row at its start held up all between them
-        draw();
-        ring_free();
+        draw(0);
+        if (pw == 0)
+            ring_free();
         issue(0);
         int k = 0; // fill k is issued
         while (ft < a.ntiles) {
-            named_bar(LB8_CNT, C::NT + C::NA + 32);
-            draw();
-            ring_free();
+            if (pw == 0)
+                named_bar(LB8_CNT, C::NT + C::NA + 32);
+            draw(k + 1);
+            if (pw == 0)
+                ring_free();
             if (k >= 1)
-                named_bar(LB8_FREE, NT + 32); // tile k - 1 is stored: the stage of fill k + 1 is free
+                named_bar(LB8_FREE, NT + C::NPW * 32); // tile k - 1 is stored: the stage of fill k + 1 is free
             issue(++k);
         }
+        if (pw != 0)
+            return;
         named_bar(LB8_CNT, C::NT + C::NA + 32); // (the end mark's)
         // every issued copy lands before this CTA exits (only after a wait
         // that ran out can one still be in flight)
@@ -1301,7 +1320,7 @@ __global__ void __launch_bounds__(Lb8Cfg<KT, HASV, TILE, NW, OOP>::THREADS, Lb8C
             // the stage was read and rewritten with generic accesses; it is
             // refilled with bulk copies (async proxy)
             fence_proxy_async_smem();
-            bar_arrive(LB8_FREE, NT + 32);
+            bar_arrive(LB8_FREE, NT + C::NPW * 32);
         }
         if (end)
             break;
