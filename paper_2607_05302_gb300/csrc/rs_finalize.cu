@@ -305,140 +305,193 @@ __global__ void k_fz_order(FinArgs a)
     }
 }
 
-// Everything up to the order array for a small permutation (n_pi <=
-// FZ_SMALL_NPI): one CTA with the map and the entries in shared memory, one
-// launch.  The steps are those of the kernels above; each jumping pass stops
-// at the step that changes nothing (windows at least double each step, so 34
-// steps bound it).  What bounds it is latency: with nine launches
-// (the jumping in one CTA already) Finalize took 74 us at 2^20 elements of 8
-// bytes and 101 at 2^22, with this one 45 and 67.
-constexpr uint32_t FZ_SMALL_NPI = 12288;
+// Everything up to the order array for a permutation of at most FZ_PLAN_NPI
+// positions in one launch: one CTA, or a thread-block cluster of FZ_CTAS with
+// the positions dealt over their shared memories.
+//
+// One jumping pass finds the heads and the ranks together.  A position's entry
+// describes a window of the chain from it on, in 16-bit fields: where the
+// window ends (next), its smallest position + 1, the distance to that one and
+// the window's length.  A position that no block leaves (a path's free end)
+// stands for itself with the minimum 0 and the length 0.  Joining x's window
+// with the one at its end at least doubles it, whichever state of that one is
+// read; a path's positions end with the minimum 0, its end and the distance to
+// it, a cycle's with its smallest position and the distance to that: head and
+// rank in the sense of the kernels above.
+//
+// What bounds it is latency (about 16 dependent steps), so launches between
+// the steps cost most of it.  Finalize of 2^20 u32 + u32 (npi 3073) 45 us with
+// two passes in one CTA, 40 with this one; 2^22 (npi 9217) 70 and 60; 2^24 (npi
+// 33,793) 197 with 27 launches, 143 here.  The line at FZ_ONE_NPI: npi 2587
+// takes 33 us in one CTA and 37 in a cluster, 3073 and 5121 the same in both.
+// 16-bit fields set the line at FZ_PLAN_NPI.
+constexpr uint32_t FZ_ONE_NPI = 4096, FZ_PLAN_NPI = 65534, FZ_CTAS = 8;
+constexpr uint32_t FZ_LEN = 0xFFFEu, FZ_HEAD = 0xFFFFu; // length field: longest, and the mark of a head's entry
 
-__global__ void __launch_bounds__(1024) k_fz_plan_small(FinArgs a, uint32_t clear)
+__device__ __forceinline__ unsigned long long fz_entry(uint32_t next, uint32_t mn, uint32_t dist, uint32_t len)
 {
-    extern __shared__ unsigned long long sj[]; // n_pi entries, then the map (n_pi words)
-    uint32_t *sp = reinterpret_cast<uint32_t *>(sj + a.npi);
-    __shared__ uint32_t s_order, s_rec;
-    const uint32_t tid = threadIdx.x, nt = blockDim.x, npi = a.npi;
+    return pk(next | mn << 16, dist | len << 16);
+}
+__device__ __forceinline__ uint32_t fz_next(unsigned long long e) { return lo32(e) & 0xFFFFu; }
+__device__ __forceinline__ uint32_t fz_min(unsigned long long e) { return lo32(e) >> 16; }
+__device__ __forceinline__ uint32_t fz_dist(unsigned long long e) { return hi32(e) & 0xFFFFu; }
+__device__ __forceinline__ uint32_t fz_len(unsigned long long e) { return hi32(e) >> 16; }
+
+// per: positions of a CTA
+template <bool MULTI> __device__ __forceinline__ void fz_plan(const FinArgs &a, uint32_t clear, uint32_t per)
+{
+    extern __shared__ unsigned long long sj[]; // entries of this CTA's positions x0 ..
+    __shared__ uint32_t s_more[3], s_cnt[2];   // (the counts of order places and records: the first CTA's)
+    const uint32_t tid = threadIdx.x, nt = blockDim.x, npi = a.npi, rank = MULTI ? cluster_rank() : 0u;
+    const uint32_t gt = rank * nt + tid, gn = MULTI ? FZ_CTAS * nt : nt;
+    const uint32_t x0 = rank * per, mine = x0 < npi ? min(per, npi - x0) : 0u;
     const uint32_t NL = a.state[ST_F] - a.H, R = NL - a.nA;
-    for (uint32_t i = tid; i < clear; i += nt) // counters and flags of the moves
-        a.ctr[i] = 0u;
-    if (tid == 0)
-        s_order = s_rec = 0;
-    auto reset = [&]() {
-        for (uint32_t x = tid; x < npi; x += nt)
-            sj[x] = pk(x, ABS);
-        __syncthreads();
+    const uint32_t inv = 0xFFFFFFFFu / per + 1u; // x / per == umulhi(x, inv) for x < 2^16
+    const uint32_t sja = smem_u32(sj), cnta = MULTI ? cluster_addr(smem_u32(s_cnt), 0u) : smem_u32(s_cnt);
+    auto at = [&](uint32_t x) {
+        const uint32_t q = __umulhi(x, inv);
+        return cluster_addr(sja + (x - q * per) * 8u, q);
     };
-    auto jump = [&](bool sum) {
-        for (int step = 0; step < 34; ++step) {
-            bool changed = false;
-            for (uint32_t x = tid; x < npi; x += nt) {
-                const unsigned long long e = ld64(&sj[x]);
-                const uint32_t v = hi32(e), nx = lo32(e);
-                if (v == ABS || nx >= npi)
-                    continue; // (only a broken entry points out of the permutation)
-                const unsigned long long f = ld64(&sj[nx]);
-                const uint32_t fv = hi32(f);
-                if (fv == ABS)
-                    continue;
-                const unsigned long long ne = pk(lo32(f), sum ? v + fv : min(v, fv));
-                if (ne != e) {
-                    st64(&sj[x], ne);
-                    changed = true;
-                }
+    auto get = [&](uint32_t x) { return MULTI ? ld_cluster64(at(x)) : ld64(&sj[x]); };
+    auto put = [&](uint32_t x, unsigned long long e) {
+        if (MULTI)
+            st_cluster(at(x), e);
+        else
+            st64(&sj[x], e);
+    };
+    auto sync = [&]() {
+        if (MULTI)
+            cluster_sync();
+        else
+            __syncthreads();
+    };
+    for (uint32_t i = gt; i < clear; i += gn) // counters and flags of the moves
+        a.ctr[i] = 0u;
+    if (tid < 3)
+        s_more[tid] = 0u;
+    if (tid < 2)
+        s_cnt[tid] = 0u;
+    for (uint32_t i = tid; i < mine; i += nt)
+        sj[i] = fz_entry(x0 + i, 0u, 0u, 0u);
+    sync();
+    for (uint32_t q = gt; q < NL; q += gn) { // block at x moves to t
+        const uint32_t x = a.pi[a.H + q], t = target_of(q, a.nA, a.nT);
+        if (x < npi && t < npi && x != t)
+            put(x, fz_entry(t, x + 1u, 0u, 1u));
+    }
+    sync();
+    for (uint32_t step = 0; step < 34; ++step) {
+        bool more = false;
+        constexpr int U = 4; // joins in flight
+        for (uint32_t i = tid; i < mine; i += U * nt) {
+            unsigned long long e[U], f[U];
+            bool on[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                e[u] = i + u * nt < mine ? ld64(&sj[i + u * nt]) : 0ull;
+                on[u] = fz_min(e[u]) != 0u && fz_len(e[u]) < npi; // not to the path's end or round the cycle
             }
-            if (!__syncthreads_or(changed))
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                f[u] = on[u] ? get(fz_next(e[u])) : 0ull;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (!on[u])
+                    continue;
+                const bool less = fz_min(f[u]) < fz_min(e[u]);
+                const uint32_t mn = less ? fz_min(f[u]) : fz_min(e[u]);
+                const uint32_t dist = less ? fz_len(e[u]) + fz_dist(f[u]) : fz_dist(e[u]);
+                const uint32_t len = min(fz_len(e[u]) + fz_len(f[u]), FZ_LEN);
+                st64(&sj[i + u * nt], fz_entry(fz_next(f[u]), mn, dist, len));
+                more |= mn != 0u && len < npi;
+            }
+        }
+        const bool any = __syncthreads_or(more);
+        if (!MULTI) {
+            if (!any)
+                break;
+        } else {
+            if (tid == 0)
+                s_more[(step + 1) % 3] = 0u; // (last read two steps ago)
+            if (any && tid < FZ_CTAS)
+                st_cluster(cluster_addr(smem_u32(&s_more[step % 3]), tid), 1u);
+            sync();
+            if (!*reinterpret_cast<volatile uint32_t *>(&s_more[step % 3]))
                 break;
         }
-    };
-    reset();
-    for (uint32_t q = tid; q < NL; q += nt) { // edges
+    }
+    sync();
+    for (uint32_t q = gt; q < NL; q += gn) { // chains
         const uint32_t x = a.pi[a.H + q], t = target_of(q, a.nA, a.nT);
-        sp[q] = x;
-        if (x < npi && x != t)
-            sj[x] = pk(t, x);
-    }
-    __syncthreads();
-    jump(false);
-    for (uint32_t q = tid; q < NL; q += nt) { // moving, on a cycle, the cycle's minimum
-        const uint32_t x = sp[q];
-        if (x >= npi || x == target_of(q, a.nA, a.nT))
+        if (x >= npi || t >= npi || x == t)
             continue;
-        const unsigned long long e = sj[x];
-        const bool cyc = lo32(e) < npi && hi32(sj[lo32(e)]) != ABS;
-        sp[q] = x | F_MOVE | (cyc ? F_CYC : 0u) | (cyc && hi32(e) == x ? F_MIN : 0u);
-    }
-    __syncthreads();
-    reset();
-    for (uint32_t q = tid; q < NL; q += nt) { // rank edges
-        const uint32_t v = sp[q];
-        if ((v & F_MOVE) && !(v & F_MIN))
-            sj[v & POS_MASK] = pk(target_of(q, a.nA, a.nT), 1u);
-    }
-    __syncthreads();
-    jump(true);
-    for (uint32_t q = tid; q < NL; q += nt) { // chains
-        const uint32_t v = sp[q];
-        if (!(v & F_MOVE))
-            continue;
-        const uint32_t x = v & POS_MASK;
-        const bool cyc = (v & F_CYC) != 0;
+        // (a head's entry is overwritten here: a path's end, from which no
+        // block moves, or a cycle's minimum, which only its own thread reads)
+        const bool start = (x < a.nT && x >= R) || x >= a.nT + a.nA; // no block moves into x
+        const unsigned long long e = get(x);
+        const bool cyc = fz_min(e) != 0u;
         uint32_t h, r;
         if (cyc) {
-            if (!(v & F_MIN))
+            if (fz_min(e) != x + 1u || fz_len(e) == FZ_HEAD)
                 continue;
             h = x;
-            r = hi32(sj[target_of(q, a.nA, a.nT)]);
+            r = fz_dist(get(t)); // the successor is the farthest from it
         } else {
-            if (!((x < a.nT && x >= R) || x >= a.nT + a.nA))
+            if (!start)
                 continue;
-            const unsigned long long e = sj[x];
-            h = lo32(e);
-            r = hi32(e);
+            h = fz_next(e);
+            r = fz_dist(e);
         }
-        const uint32_t len = r + 1;
-        const uint32_t base = atomicAdd(&s_order, len);
+        const uint32_t len = r + 1u;
+        const uint32_t base = add_cluster(cnta, len);
         uint32_t defer = 0;
         if (cyc && base / a.K != (base + len - 1) / a.K) {
-            const uint32_t ri = atomicAdd(&s_rec, 1u);
+            const uint32_t ri = add_cluster(cnta + 4u, 1u);
             if (ri < a.nrec_cap) {
                 const uint32_t slot = ri < a.nslots ? ri : SLOT_NONE;
                 a.rec[ri] = make_uint4(base, len, slot, 0);
-                defer = slot == SLOT_NONE ? H_DEFER : 0u;
+                defer = slot == SLOT_NONE ? 2u : 0u;
             } else {
                 set_status(ST_INTERNAL);
             }
         }
-        if (h < npi)
-            st64(&sj[h], pk(base, len | H_HEAD | (cyc ? H_CYC : 0u) | defer));
+        if (base + len > npi || h >= npi)
+            set_status(ST_INTERNAL); // (only a broken map gets here)
+        else
+            put(h, fz_entry(base, (cyc ? 1u : 0u) | defer, len, FZ_HEAD));
     }
-    __syncthreads();
-    if (tid == 0) {
-        a.ctr[C_ORDER] = s_order;
-        a.ctr[C_REC] = s_rec;
+    sync();
+    if (gt == 0) {
+        a.ctr[C_ORDER] = s_cnt[0];
+        a.ctr[C_REC] = s_cnt[1];
     }
-    for (uint32_t x = tid; x < npi; x += nt) { // order
-        const unsigned long long e = sj[x];
-        const uint32_t v = hi32(e);
-        if (v == ABS)
-            continue;
-        uint32_t base, info, r;
-        if (v & H_HEAD) {
-            base = lo32(e);
-            info = v;
-            r = 0;
-        } else {
-            const unsigned long long hd = lo32(e) < npi ? sj[lo32(e)] : 0ull;
-            base = lo32(hd);
-            info = hi32(hd);
-            r = v;
+    for (uint32_t i = tid; i < mine; i += nt) { // order
+        const unsigned long long e = ld64(&sj[i]);
+        unsigned long long hd = e;
+        uint32_t r = 0;
+        if (fz_len(e) == 0u)
+            continue; // nothing moves here
+        if (fz_len(e) != FZ_HEAD) {
+            const uint32_t h = fz_min(e) ? fz_min(e) - 1u : fz_next(e);
+            hd = get(h);
+            r = fz_dist(e);
+            if (fz_len(hd) != FZ_HEAD)
+                continue; // (a broken map, reported above)
         }
-        const uint32_t len = info & H_LEN;
-        if (base + r < npi)
-            a.pi[base + r] = x | (r == 0 ? O_FIRST : 0u) | (r + 1 == len ? O_LAST : 0u) |
-                             ((info & H_CYC) ? O_CYC : 0u) | ((info & H_DEFER) ? O_DEFER : 0u);
+        const uint32_t pos = fz_next(hd) + r, len = fz_dist(hd), fl = fz_min(hd);
+        if (pos < npi)
+            a.pi[pos] = (x0 + i) | (r == 0 ? O_FIRST : 0u) | (r + 1 == len ? O_LAST : 0u) |
+                        ((fl & 1u) ? O_CYC : 0u) | ((fl & 2u) ? O_DEFER : 0u);
     }
+    if (MULTI)
+        sync(); // no CTA leaves while others read its entries
+}
+
+__global__ void __launch_bounds__(1024) k_fz_plan_one(FinArgs a, uint32_t clear) { fz_plan<false>(a, clear, a.npi); }
+__global__ void __cluster_dims__(FZ_CTAS, 1, 1) __launch_bounds__(1024)
+    k_fz_plan_cluster(FinArgs a, uint32_t clear, uint32_t per)
+{
+    fz_plan<true>(a, clear, per);
 }
 
 // record of the straddling cycle that contains order index g (linear search;
@@ -1037,7 +1090,7 @@ cudaError_t fin_impl(const Geom &g, const Bufs &w, uint32_t *pi, unsigned long l
     a.W = L.W;
 
     cudaError_t e = cudaSuccess;
-    const bool small = g.npi <= FZ_SMALL_NPI;
+    const bool small = g.npi <= FZ_PLAN_NPI;
     if (!small || !g.grid) // (a small permutation's plan clears what the moves need)
         e = cudaMemsetAsync(base, 0, L.rec, st);
     if (e != cudaSuccess)
@@ -1048,15 +1101,20 @@ cudaError_t fin_impl(const Geom &g, const Bufs &w, uint32_t *pi, unsigned long l
             return e;
     }
     const int sms = num_sms();
-    if (small) {
+    const uint32_t clear = static_cast<uint32_t>(L.rec / 4);
+    if (g.npi <= FZ_ONE_NPI) {
+        k_fz_plan_one<<<1, 1024, size_t(g.npi) * 8, st>>>(a, clear);
+        g_launches += 1;
+    } else if (small) {
+        constexpr uint32_t most = (FZ_PLAN_NPI + FZ_CTAS - 1) / FZ_CTAS;
         static DeviceOnce jattr;
         const cudaError_t ej = jattr.run([] {
-            return cudaFuncSetAttribute(k_fz_plan_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        int(FZ_SMALL_NPI * 12));
+            return cudaFuncSetAttribute(k_fz_plan_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, int(most * 8));
         });
         if (ej != cudaSuccess)
             return ej;
-        k_fz_plan_small<<<1, 1024, size_t(g.npi) * 12, st>>>(a, static_cast<uint32_t>(L.rec / 4));
+        const uint32_t per = (g.npi + FZ_CTAS - 1) / FZ_CTAS;
+        k_fz_plan_cluster<<<FZ_CTAS, 1024, size_t(per) * 8, st>>>(a, clear, per);
         g_launches += 1;
     } else {
         int grid = static_cast<int>((g.npi + FIN_T - 1) / FIN_T);

@@ -27,49 +27,6 @@ constexpr int SM_T = 512;            // threads per CTA
 constexpr int SM_ROWS = SM_T / 16;   // half-warps
 constexpr int SM_MAXC = 16;          // CTAs of the largest cluster
 
-__device__ __forceinline__ uint32_t cluster_rank()
-{
-    uint32_t r;
-    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ uint32_t cluster_size()
-{
-    uint32_t r;
-    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
-    return r;
-}
-// every thread of the cluster; orders shared-memory accesses across its CTAs
-__device__ __forceinline__ void cluster_sync()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// this shared-memory address in CTA `rank` of the cluster
-__device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, uint32_t rank)
-{
-    uint32_t r;
-    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-    return r;
-}
-__device__ __forceinline__ uint32_t ld_cluster(uint32_t addr)
-{
-    uint32_t v;
-    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
-    return v;
-}
-__device__ __forceinline__ void st_cluster(uint32_t addr, uint32_t v)
-{
-    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
-}
-__device__ __forceinline__ void st_cluster(uint32_t addr, unsigned long long v)
-{
-    asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(addr), "l"(v) : "memory");
-}
-__device__ __forceinline__ void st_cluster(uint32_t addr, uint2 v)
-{
-    asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(addr), "r"(v.x), "r"(v.y) : "memory");
-}
-
 // IEEE float32 bits <-> unsigned-orderable bits
 __device__ __forceinline__ uint32_t float_to_ordered(uint32_t x) { return x ^ ((x >> 31) ? 0xFFFFFFFFu : 0x80000000u); }
 __device__ __forceinline__ uint32_t ordered_to_float(uint32_t x) { return x ^ ((x >> 31) ? 0x80000000u : 0xFFFFFFFFu); }
