@@ -169,6 +169,7 @@ static radsort_status fill_geom_grid(size_t n, int kb, bool hasv, int db, uint32
     g->sigma = 256; // buckets of a pass
     g->nt = (8 * kb + db - 1) / db;
     g->whole = false;
+    g->flt = false;
     g->b = b;
     g->lb = ilog2(b);
     g->p = 1;
@@ -442,6 +443,11 @@ static cudaError_t run_rounds(const Geom &g, Bufs &w, int rounds, cudaStream_t s
         {
             Scope sc(0, -1, st);
             e = launch_grid_setup(g, w, pc, st);
+        }
+        if (g.flt && e == cudaSuccess) {
+            Scope sc(4, -1, st); // (a first pass that is left out; the tail is in T)
+            e = launch_float_keys(static_cast<uint32_t *>(w.Ak), g.n, 0, st, grid_skip_word(w, 0),
+                                  size_t(g.nA) * g.b, static_cast<uint32_t *>(w.Tk) + size_t(g.H) * g.b);
         }
         const bool bytes = by_bytes(g.db, g.whole);
         const int ppd = bytes ? 1 : 2, np = g.whole ? digit_passes(g.kb, g.db, true) : rounds * ppd;
@@ -728,7 +734,10 @@ static radsort_status sort_common(void *keys, uint32_t *values, size_t n, int ke
     w.Ak = keys;
     w.Av = values;
     cudaError_t e = cudaSuccess;
-    if (flags & RADSORT_KEY_FLOAT32) {
+    // float keys: in the grid layout the histograms and the first pass read
+    // them as ordered integers and the last pass writes them back
+    g.flt = g.grid && (flags & RADSORT_KEY_FLOAT32) && rounds < 0;
+    if ((flags & RADSORT_KEY_FLOAT32) && !g.flt) {
         Scope sc(4, -1, st);
         e = launch_float_keys(static_cast<uint32_t *>(keys), n, 0, st);
     }
@@ -748,8 +757,9 @@ static radsort_status sort_common(void *keys, uint32_t *values, size_t n, int ke
             e = launch_gather(g, w, pc, out_keys, out_values, st);
     }
     if (e == cudaSuccess && (flags & RADSORT_KEY_FLOAT32) && rounds < 0) {
-        Scope sc(4, -1, st);
-        e = launch_float_keys(static_cast<uint32_t *>(keys), n, 1, st);
+        Scope sc(4, -1, st); // (a last pass that the passes left out)
+        e = launch_float_keys(static_cast<uint32_t *>(keys), n, 1, st,
+                              g.flt ? grid_skip_word(w, digit_passes(g.kb, g.db, true) - 1) : nullptr);
     }
     if (own) {
         cudaError_t e2 = cudaFreeAsync(ws, st);

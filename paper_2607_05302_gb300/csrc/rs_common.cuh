@@ -267,4 +267,9 @@ template <typename KT> __device__ __forceinline__ uint32_t digit_of(KT k, uint32
     return static_cast<uint32_t>(k >> shift) & mask;
 }
 
+// IEEE float32 bits <-> unsigned-orderable bits: the sign bit of non-negative
+// values flips, every bit of negative ones
+__device__ __forceinline__ uint32_t float_to_ordered(uint32_t x) { return x ^ ((x >> 31) ? 0xFFFFFFFFu : 0x80000000u); }
+__device__ __forceinline__ uint32_t ordered_to_float(uint32_t x) { return x ^ ((x >> 31) ? 0x80000000u : 0xFFFFFFFFu); }
+
 } // namespace rs

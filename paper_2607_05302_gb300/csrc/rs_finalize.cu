@@ -1190,16 +1190,16 @@ cudaError_t launch_finalize(const Geom &g, const Bufs &w, uint32_t *pi, unsigned
 }
 
 // ---------------------------------------------------------------- float keys
-// IEEE float32 bits -> unsigned-orderable bits: flip the sign bit of
-// non-negative values and every bit of negative ones (and back).
-__global__ void k_float_keys(uint32_t *u, size_t n, int inverse)
+// The whole array's pass (also radsort_float_keys).  Given `only`, the pass is
+// left out unless that word is set, and the elements from `tail` on are at t.
+__global__ void k_float_keys(uint32_t *u, size_t n, int inverse, const uint32_t *only, size_t tail, uint32_t *t)
 {
+    if (only && !*only)
+        return;
     const size_t stride = size_t(gridDim.x) * blockDim.x;
     for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += stride) {
-        const uint32_t x = u[i];
-        const bool top = (x & 0x80000000u) != 0;
-        u[i] = inverse ? (x ^ (top ? 0x80000000u : 0xFFFFFFFFu))
-                       : (x ^ (top ? 0xFFFFFFFFu : 0x80000000u));
+        uint32_t *p = i < tail ? u + i : t + (i - tail);
+        *p = inverse ? ordered_to_float(*p) : float_to_ordered(*p);
     }
 }
 
@@ -1221,7 +1221,8 @@ cudaError_t launch_wait_probe(const uint32_t *flag, unsigned limit, cudaStream_t
     return cudaGetLastError();
 }
 
-cudaError_t launch_float_keys(uint32_t *keys, size_t n, int inverse, cudaStream_t st)
+cudaError_t launch_float_keys(uint32_t *keys, size_t n, int inverse, cudaStream_t st, const uint32_t *only,
+                              size_t tail, uint32_t *tail_keys)
 {
     if (n == 0)
         return cudaSuccess;
@@ -1229,7 +1230,7 @@ cudaError_t launch_float_keys(uint32_t *keys, size_t n, int inverse, cudaStream_
     const int cap = num_sms() * 8;
     if (blocks > cap)
         blocks = cap;
-    k_float_keys<<<blocks, 256, 0, st>>>(keys, n, inverse);
+    k_float_keys<<<blocks, 256, 0, st>>>(keys, n, inverse, only, tail_keys ? tail : n, tail_keys);
     g_launches += 1;
     return cudaGetLastError();
 }

@@ -91,8 +91,10 @@ __device__ __forceinline__ unsigned long long lbw(uint32_t tag, uint32_t v)
 // 8-bit digits: counts of four digit positions r0 .. r0+3 with one counter
 // column per lane (counter (r, d) of lane l at word (r*256 + d)*32 + l), so
 // the 32 atomics of a warp instruction fall in 32 different banks whatever
-// the digits.  One CTA of 1024 threads per SM, 128 KB of counters.
-template <typename KT>
+// the digits.  One CTA of 1024 threads per SM, 128 KB of counters.  FLT: float32
+// keys, counted as ordered integers (a run-time switch made the counts of all
+// keys 0.25 -> 0.33 ms at 2^28).
+template <typename KT, bool FLT = false>
 __global__ void __launch_bounds__(1024) k_digit_hist_lanes(const KT *keys, uint32_t n, int r0, uint32_t *hist)
 {
     constexpr int NTD = 8 * int(sizeof(KT)) / 8;
@@ -105,6 +107,8 @@ __global__ void __launch_bounds__(1024) k_digit_hist_lanes(const KT *keys, uint3
     __syncthreads();
     const int npos = min(G, NTD - r0);
     auto put = [&](KT k) {
+        if constexpr (FLT)
+            k = float_to_ordered(k);
 #pragma unroll
         for (int r = 0; r < G; ++r)
             if (r < npos)
@@ -188,7 +192,7 @@ __global__ void __launch_bounds__(1024) k_pass_hist_lanes(const KT *keys, uint32
 
 // Launches the bucket counts of every pass, by bytes or (11-bit digits one by
 // one) by half digits.
-static cudaError_t launch_digit_hist(const void *keys, uint32_t n, int kb, bool bytes, uint32_t *hist,
+static cudaError_t launch_digit_hist(const void *keys, uint32_t n, int kb, bool bytes, bool flt, uint32_t *hist,
                                      cudaStream_t st)
 {
     using u64 = unsigned long long;
@@ -198,6 +202,9 @@ static cudaError_t launch_digit_hist(const void *keys, uint32_t n, int kb, bool 
     const cudaError_t ea = attr.run([] {
         cudaError_t e = cudaFuncSetAttribute(k_digit_hist_lanes<uint32_t>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, LSM);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_digit_hist_lanes<uint32_t, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     LSM);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_digit_hist_lanes<u64>, cudaFuncAttributeMaxDynamicSharedMemorySize, LSM);
         if (e == cudaSuccess)
@@ -211,7 +218,9 @@ static cudaError_t launch_digit_hist(const void *keys, uint32_t n, int kb, bool 
     const int grid = num_sms();
     g_launches += 1;
     if (bytes) {
-        if (kb == 4) {
+        if (kb == 4 && flt) {
+            k_digit_hist_lanes<uint32_t, true><<<grid, 1024, LSM, st>>>(static_cast<const uint32_t *>(keys), n, 0, hist);
+        } else if (kb == 4) {
             k_digit_hist_lanes<uint32_t><<<grid, 1024, LSM, st>>>(static_cast<const uint32_t *>(keys), n, 0, hist);
         } else {
             for (int r0 = 0; r0 < 8; r0 += 4)
@@ -521,6 +530,10 @@ template <typename KT> struct LbArgs {
     const uint32_t *hdr;    // Radsort: the tables' header
     uint32_t n, ntiles, H, nT, npi, lb;
     uint32_t shift, mask;   // the pass's digit: key >> shift & mask, at most 255
+    // FLT kernels: float32 keys, made ordered (1) or floats again (2) by this
+    // pass.  A transform of its own reads and writes every key: 0.135 ms before
+    // and after a sort of 2^26 (2.56 ms in all; 2.33 without them)
+    uint32_t flt;
 };
 
 // Exclusive prefix of bucket c before tile t: sum of the counts of the tiles
@@ -596,8 +609,8 @@ __device__ __forceinline__ uint32_t wait_pi(const uint32_t *p)
 // One CTA per SM: NW ranking warps, 8 look-back warps and a producer warp, on
 // tiles of TILE elements in two shared-memory stages.  What bounds it is
 // shared memory (the random-digit accesses of the ranking and the reorder,
-// each 3.4 wavefronts a row of 32 elements) and instruction issue, both near
-// 60% busy; DRAM is at 40% of its peak.  Hence
+// each 3.4 wavefronts a row of 32 elements), 75% busy, then instruction issue,
+// 48%; DRAM is at 36% of its peak.  Hence
 //  * the ranking works on half-warps.  Each half-warp ranks its own run of
 //    TILE / (2 NW) elements, 16 a row, with one word per digit: the count so
 //    far in the high half, the lanes of this row in the low half.  A row is
@@ -691,7 +704,7 @@ struct LbGroup {
 };
 struct LbNoGroup {};
 
-template <typename KT, bool HASV, int TILE, int NW, bool OOP, bool GRP = false>
+template <typename KT, bool HASV, int TILE, int NW, bool OOP, bool GRP = false, bool FLT = false>
 __global__ void __launch_bounds__(Lb8Cfg<KT, HASV, TILE, NW, OOP>::THREADS, Lb8Cfg<KT, HASV, TILE, NW, OOP>::MINB)
     k_lb_round8(LbArgs<KT> a, const __grid_constant__ std::conditional_t<GRP, LbGroup, LbNoGroup> grp)
 {
@@ -1161,6 +1174,12 @@ __global__ void __launch_bounds__(Lb8Cfg<KT, HASV, TILE, NW, OOP>::THREADS, Lb8C
                     }
                 }
             }
+            if constexpr (FLT)
+                if (a.flt & 1u) {
+#pragma unroll
+                    for (int it = 0; it < ITEMS; ++it)
+                        key[it] = float_to_ordered(key[it]);
+                }
             if (cnt < uint32_t(TILE)) {
                 // elements past the end rank as the last ones of the largest digit
 #pragma unroll
@@ -1304,7 +1323,10 @@ __global__ void __launch_bounds__(Lb8Cfg<KT, HASV, TILE, NW, OOP>::THREADS, Lb8C
                     for (int u = 0; u < U; ++u)
                         if (w[u]) {
                             KT *dk = reinterpret_cast<KT *>(w[u] & ~3ull) + idx[u];
-                            *dk = kv[u];
+                            if constexpr (FLT)
+                                *dk = a.flt & 2u ? ordered_to_float(kv[u]) : kv[u];
+                            else
+                                *dk = kv[u];
                             if (HASV) {
                                 uint32_t *dv;
                                 if constexpr (sizeof(KT) == 4)
@@ -1433,17 +1455,25 @@ __global__ void __launch_bounds__(256)
 // The round kernel of a configuration.
 template <typename KT, bool HASV, int TILE, int NW, bool OOP> struct LbKernel {
     using C = Lb8Cfg<KT, HASV, TILE, NW, OOP>;
+    static constexpr bool FLT = sizeof(KT) == 4 && !OOP; // there is a kernel for float keys
     static void launch(int grid, const LbArgs<KT> &a, cudaStream_t st)
     {
-        k_lb_round8<KT, HASV, TILE, NW, OOP><<<grid, C::THREADS, C::SMEM, st>>>(a, LbNoGroup{});
+        if (FLT && a.flt)
+            k_lb_round8<KT, HASV, TILE, NW, OOP, false, FLT><<<grid, C::THREADS, C::SMEM, st>>>(a, LbNoGroup{});
+        else
+            k_lb_round8<KT, HASV, TILE, NW, OOP><<<grid, C::THREADS, C::SMEM, st>>>(a, LbNoGroup{});
     }
     // CTAs of a launch over ntiles tiles (-1: the kernel cannot be set up)
     static int ctas(size_t ntiles)
     {
         static DeviceOnce attr; // per template instance
         if (attr.run([] {
-                return cudaFuncSetAttribute(k_lb_round8<KT, HASV, TILE, NW, OOP>,
-                                            cudaFuncAttributeMaxDynamicSharedMemorySize, int(C::SMEM));
+                const cudaError_t e = cudaFuncSetAttribute(k_lb_round8<KT, HASV, TILE, NW, OOP>,
+                                                           cudaFuncAttributeMaxDynamicSharedMemorySize, int(C::SMEM));
+                return e != cudaSuccess || !FLT
+                           ? e
+                           : cudaFuncSetAttribute(k_lb_round8<KT, HASV, TILE, NW, OOP, false, FLT>,
+                                                  cudaFuncAttributeMaxDynamicSharedMemorySize, int(C::SMEM));
             }) != cudaSuccess)
             return -1;
         size_t grid = size_t(num_sms()) * C::MINB;
@@ -1543,6 +1573,11 @@ size_t grid_ring_bytes(const Geom &g)
 // ---------------------------------------------------------------- grid-layout Radsort
 size_t grid_tab_words(const Geom &g) { return size_t(digit_passes(g.kb, g.db, false)) * GridTab::WORDS; }
 
+const uint32_t *grid_skip_word(const Bufs &w, int pass)
+{
+    return w.tab + size_t(pass) * GridTab::WORDS + GridTab::HDR + TAB_SKIP;
+}
+
 cudaError_t launch_grid_tables(const Geom &g, const Bufs &w, uint32_t *pi, bool setup, cudaStream_t st)
 {
     const uint32_t n = static_cast<uint32_t>(g.n), np = static_cast<uint32_t>(digit_passes(g.kb, g.db, g.whole));
@@ -1571,7 +1606,7 @@ cudaError_t launch_grid_setup(const Geom &g, const Bufs &w, uint32_t *pi, cudaSt
     cudaError_t e = cudaMemsetAsync(z0, 0, reinterpret_cast<char *>(w.status) + grid_ring_bytes(g) - z0, st);
     if (e != cudaSuccess)
         return e;
-    e = launch_digit_hist(w.Ak, static_cast<uint32_t>(g.n), g.kb, by_bytes(g.db, g.whole), w.hist, st);
+    e = launch_digit_hist(w.Ak, static_cast<uint32_t>(g.n), g.kb, by_bytes(g.db, g.whole), g.flt, w.hist, st);
     if (e != cudaSuccess)
         return e;
     return launch_grid_tables(g, w, pi, true, st);
@@ -1617,6 +1652,8 @@ cudaError_t launch_grid_round(const Geom &g, const Bufs &w, const uint32_t *pi, 
         a.nT = g.nT;
         a.npi = g.npi;
         a.lb = g.lb;
+        if (g.flt)
+            a.flt = (pass == 0 ? 1u : 0u) | (pass == digit_passes(g.kb, g.db, true) - 1 ? 2u : 0u);
         const DigitPass dp = digit_pass(g.kb, g.db, g.whole, pass);
         a.shift = dp.shift;
         a.mask = dp.mask();
@@ -1669,7 +1706,7 @@ cudaError_t launch_lsd_oop_ws(void *keys, uint32_t *vals, void *keys_alt, uint32
     e = cudaMemsetAsync(hist, 0, L.total, st);
     const uint32_t nn = static_cast<uint32_t>(n);
     if (e == cudaSuccess)
-        e = launch_digit_hist(keys, nn, kb, true, hist, st);
+        e = launch_digit_hist(keys, nn, kb, true, false, hist, st);
     if (e == cudaSuccess) {
         k_offsets<<<np, 256, 0, st>>>(hist, off, nn);
         g_launches += 1;

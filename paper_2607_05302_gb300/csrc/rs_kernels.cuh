@@ -50,6 +50,7 @@ struct Geom {
     uint32_t sigma;    // 2^db
     int nt;            // digits per key
     bool whole;        // grid layout: all digits in one go (digit_pass)
+    bool flt;          // grid layout, whole sort: float32 keys, transformed by the passes
     uint32_t b, lb;    // block size and log2
     uint32_t p;        // chunks
     uint32_t nA;       // floor(n/b): blocks overlaying A
@@ -109,6 +110,8 @@ cudaError_t launch_fixup(const Geom &g, const Bufs &w, const uint32_t *pi_old, u
 // setup: the tables alone, from the histograms of the current sequence
 size_t grid_tab_words(const Geom &g);
 cudaError_t launch_grid_tables(const Geom &g, const Bufs &w, uint32_t *pi, bool setup, cudaStream_t st);
+// the word that says whether a pass is left out (a constant digit)
+const uint32_t *grid_skip_word(const Bufs &w, int pass);
 cudaError_t launch_grid_setup(const Geom &g, const Bufs &w, uint32_t *pi, cudaStream_t st);
 cudaError_t launch_grid_prep(const Geom &g, const Bufs &w, const uint32_t *pi, uint32_t *pin,
                              int pass, cudaStream_t st);
@@ -132,8 +135,10 @@ cudaError_t launch_deficit(const Geom &g, const Bufs &w, cudaStream_t st);
 cudaError_t launch_finalize(const Geom &g, const Bufs &w, uint32_t *pi, unsigned long long *jump,
                             cudaStream_t st);
 size_t finalize_extra_bytes(const Geom &g);
-// float32 key transform
-cudaError_t launch_float_keys(uint32_t *keys, size_t n, int inverse, cudaStream_t st);
+// float32 key transform; with `only`, a pass that the device leaves out unless
+// that word is set (elements from `tail` on at tail_keys, if given)
+cudaError_t launch_float_keys(uint32_t *keys, size_t n, int inverse, cudaStream_t st, const uint32_t *only = nullptr,
+                              size_t tail = 0, uint32_t *tail_keys = nullptr);
 // out-of-place LSD comparator
 cudaError_t launch_lsd_oop(void *keys, uint32_t *vals, void *keys_alt, uint32_t *vals_alt,
                            size_t n, int kb, int db, cudaStream_t st);

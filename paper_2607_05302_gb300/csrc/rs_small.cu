@@ -27,10 +27,6 @@ constexpr int SM_T = 512;            // threads per CTA
 constexpr int SM_ROWS = SM_T / 16;   // half-warps
 constexpr int SM_MAXC = 16;          // CTAs of the largest cluster
 
-// IEEE float32 bits <-> unsigned-orderable bits
-__device__ __forceinline__ uint32_t float_to_ordered(uint32_t x) { return x ^ ((x >> 31) ? 0xFFFFFFFFu : 0x80000000u); }
-__device__ __forceinline__ uint32_t ordered_to_float(uint32_t x) { return x ^ ((x >> 31) ? 0x80000000u : 0xFFFFFFFFu); }
-
 // ITEMS elements per thread; odd, so that the two half-warps of a warp read
 // different banks
 template <typename KT, bool HASV, int ITEMS> struct SmCfg {
