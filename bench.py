@@ -681,7 +681,7 @@ def main():
     roofline = {"bound": "hbm", "achieved": round(achieved, 1), "peak": hbm, "unit": "GB/s",
                 "frac": round(achieved / hbm, 4), "traffic": traffic,
                 "kernel": ("k_round (sortPhase, Alg. 5, chunk layout)" if lay == "chunks"
-                           else "k_lb_round (sortPhase, Alg. 5, grid layout)"),
+                           else "k_lb_round8 (sortPhase, Alg. 5, grid layout)"),
                 "algorithmic_bytes_per_launch": n * 2 * E, "peak_source": src,
                 "avg_launch_ms": round(avg_round, 4)}
     step_bytes = n * (4 * 2 * E) if kb == 4 and db == 8 else None

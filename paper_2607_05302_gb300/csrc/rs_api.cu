@@ -205,9 +205,9 @@ static void auto_plan_chunks(size_t n, int kb, int vb, int db, radsort_plan *pl)
 // the array's bytes (below about 2^26 elements no block size meets 2%: the
 // look-back ring and tables alone take ~2 MB; a quarter keeps the footprint
 // well below an out-of-place sort's).
-// Measured (u32 keys + values, us a sort): 2^20 b = 256 309, 512 259;
-// 2^22 506, 390; 2^24 1231, 820; 2^25 2233, 1398 -- blocks of 256 leave many
-// list entries per tile.
+// Measured (u32 keys + values, us a sort, b = 256, 512, 1024): 2^20 178, 149,
+// 136; 2^22 288, 246, 229; 2^24 762, 615, 572; 2^25 1294, 1148, 1037 -- small
+// blocks leave many copies and list entries per tile and many to permute.
 static void auto_plan(size_t n, int kb, int vb, int db, radsort_plan *pl)
 {
     if (pl->layout != RADSORT_LAYOUT_CHUNKS && n < (size_t(1) << 31)) {
