@@ -234,11 +234,19 @@ __device__ __forceinline__ uint32_t ld_cluster(uint32_t addr)
     asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
     return v;
 }
-__device__ __forceinline__ unsigned long long ld_cluster64(uint32_t addr)
+// 64 bits that another CTA may be storing meanwhile (st_relaxed64): relaxed
+// accesses that cover each other whole are single-copy atomic, so the load
+// returns one of the values stored; of a weak load that races with a store the
+// memory model says nothing, it may be half of each
+__device__ __forceinline__ unsigned long long ld_relaxed64(uint32_t addr)
 {
     unsigned long long v;
-    asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(addr) : "memory");
+    asm volatile("ld.relaxed.cluster.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(addr) : "memory");
     return v;
+}
+__device__ __forceinline__ void st_relaxed64(uint32_t addr, unsigned long long v)
+{
+    asm volatile("st.relaxed.cluster.shared::cluster.u64 [%0], %1;" ::"r"(addr), "l"(v) : "memory");
 }
 __device__ __forceinline__ uint32_t add_cluster(uint32_t addr, uint32_t v)
 {

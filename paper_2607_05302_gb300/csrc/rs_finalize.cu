@@ -352,12 +352,21 @@ template <bool MULTI> __device__ __forceinline__ void fz_plan(const FinArgs &a, 
         const uint32_t q = __umulhi(x, inv);
         return cluster_addr(sja + (x - q * per) * 8u, q);
     };
-    auto get = [&](uint32_t x) { return MULTI ? ld_cluster64(at(x)) : ld64(&sj[x]); };
+    // Entries are read while their owners rewrite them: every access is relaxed
+    // (volatile within a CTA) and covers the entry, so a read sees one state whole
+    auto get = [&](uint32_t x) { return MULTI ? ld_relaxed64(at(x)) : ld64(&sj[x]); };
     auto put = [&](uint32_t x, unsigned long long e) {
         if (MULTI)
-            st_cluster(at(x), e);
+            st_relaxed64(at(x), e);
         else
             st64(&sj[x], e);
+    };
+    auto own = [&](uint32_t i) { return MULTI ? ld_relaxed64(sja + i * 8u) : ld64(&sj[i]); }; // entry x0 + i
+    auto put_own = [&](uint32_t i, unsigned long long e) {
+        if (MULTI)
+            st_relaxed64(sja + i * 8u, e);
+        else
+            st64(&sj[i], e);
     };
     auto sync = [&]() {
         if (MULTI)
@@ -372,7 +381,7 @@ template <bool MULTI> __device__ __forceinline__ void fz_plan(const FinArgs &a, 
     if (tid < 2)
         s_cnt[tid] = 0u;
     for (uint32_t i = tid; i < mine; i += nt)
-        sj[i] = fz_entry(x0 + i, 0u, 0u, 0u);
+        put_own(i, fz_entry(x0 + i, 0u, 0u, 0u));
     sync();
     for (uint32_t q = gt; q < NL; q += gn) { // block at x moves to t
         const uint32_t x = a.pi[a.H + q], t = target_of(q, a.nA, a.nT);
@@ -388,7 +397,7 @@ template <bool MULTI> __device__ __forceinline__ void fz_plan(const FinArgs &a, 
             bool on[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) {
-                e[u] = i + u * nt < mine ? ld64(&sj[i + u * nt]) : 0ull;
+                e[u] = i + u * nt < mine ? own(i + u * nt) : 0ull;
                 on[u] = fz_min(e[u]) != 0u && fz_len(e[u]) < npi; // not to the path's end or round the cycle
             }
 #pragma unroll
@@ -402,7 +411,7 @@ template <bool MULTI> __device__ __forceinline__ void fz_plan(const FinArgs &a, 
                 const uint32_t mn = less ? fz_min(f[u]) : fz_min(e[u]);
                 const uint32_t dist = less ? fz_len(e[u]) + fz_dist(f[u]) : fz_dist(e[u]);
                 const uint32_t len = min(fz_len(e[u]) + fz_len(f[u]), FZ_LEN);
-                st64(&sj[i + u * nt], fz_entry(fz_next(f[u]), mn, dist, len));
+                put_own(i + u * nt, fz_entry(fz_next(f[u]), mn, dist, len));
                 more |= mn != 0u && len < npi;
             }
         }
@@ -466,7 +475,7 @@ template <bool MULTI> __device__ __forceinline__ void fz_plan(const FinArgs &a, 
         a.ctr[C_REC] = s_cnt[1];
     }
     for (uint32_t i = tid; i < mine; i += nt) { // order
-        const unsigned long long e = ld64(&sj[i]);
+        const unsigned long long e = own(i);
         unsigned long long hd = e;
         uint32_t r = 0;
         if (fz_len(e) == 0u)
