@@ -291,14 +291,15 @@ radsort_status radsort_lsd_oop_scratch_size(size_t n, int key_bytes, int value_b
  * workspace when their start is not 16-byte aligned.  With 8-bit digits those
  * that fit the workspace's alternate buffers together go out of place in
  * groups of up to 64, one launch per digit for a group; so do a few medium
- * segments (longer than 16384) where that takes no more workspace.  The others
+ * segments (longer than 16384) where that takes at most 1 MiB more workspace.  The others
  * are spread, longest first, over up to 4 library-owned streams (created on
  * the first call that has long segments on a device) that start after the
  * work already on `stream` and that `stream` waits for, each with its own part
  * of the workspace.  workspace: at least radsort_segmented_workspace_size() bytes,
  * or NULL to allocate stream-ordered.  With 8-bit digits a smaller caller
  * workspace, down to radsort_segmented_workspace_size_min() bytes, selects
- * the fastest of two low-memory plans that fits: (1) the medium segments
+ * the fastest of three plans that fits: the same without grouping those few
+ * medium segments; (1) the medium segments
  * longer than 16448 elements are sorted in place by Radsort itself on one
  * CTA each (Alg. 4-7 on blocks of 32 elements, with 2 sigma + 2 scratch
  * blocks per CTA, two CTAs per SM, one per SM on 7/8 of the SMs beside long

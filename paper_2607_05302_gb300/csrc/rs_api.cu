@@ -992,14 +992,15 @@ struct SegPlan {
 // level (8-bit digits, not oop): 0 the fastest plan; 1 medium segments
 // sorted in place (Radsort per CTA); 2 as 1, and long segments with an
 // unaligned start sorted in place too (their first elements merged back)
-// instead of out of place
+// instead of out of place; group_few: a few medium segments may be sorted with
+// the long ones, for up to 1 MiB more
 radsort_status seg_plan(const uint64_t *offh, size_t nseg, int kb, bool hasv, int db, bool oop, int level,
-                        SegPlan *sp)
+                        SegPlan *sp, bool group_few = true)
 {
     size_t large = 0, nlong = 0, nmed = 0;
     uint32_t med_max = 0, low_max = 0; // longest medium segment, and of those up to SEG_LOW
     SegGroup few{};                    // the medium segments longer than SEG_LOW
-    bool is_few = level == 0 && !oop && db == 8;
+    bool is_few = group_few && level == 0 && !oop && db == 8;
     const uint32_t small_max = seg_small_max(db);
     const size_t n = nseg ? offh[nseg] - offh[0] : 0;
     for (size_t s = 0; s < nseg; ++s) {
@@ -1288,7 +1289,7 @@ radsort_status radsort_segmented_workspace_size_min(const uint64_t *offsets_host
     radsort_status s = RADSORT_OK;
     for (int level = 0; level <= 2 && s == RADSORT_OK; ++level) {
         SegPlan sp;
-        s = seg_plan(offsets_host, num_segments, key_bytes, value_bytes == 4, digit_bits, false, level, &sp);
+        s = seg_plan(offsets_host, num_segments, key_bytes, value_bytes == 4, digit_bits, false, level, &sp, false);
         if (s == RADSORT_OK && (level == 0 || sp.total < best))
             best = sp.total;
     }
@@ -1313,6 +1314,10 @@ radsort_status radsort_sort_segmented(void *keys, uint32_t *values, const uint64
     SegPlan sp;
     radsort_status s = seg_plan(offsets_host, num_segments, key_bytes, hasv, digit_bits, false, 0, &sp);
     // a caller workspace below the fastest plan: the fastest one that fits
+    if (s == RADSORT_OK && workspace && workspace_bytes < sp.total) {
+        sp = SegPlan{};
+        s = seg_plan(offsets_host, num_segments, key_bytes, hasv, digit_bits, false, 0, &sp, false);
+    }
     for (int level = 1; s == RADSORT_OK && workspace && workspace_bytes < sp.total && digit_bits == 8 && level <= 2;
          ++level) {
         SegPlan lo;
