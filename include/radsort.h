@@ -133,10 +133,11 @@ radsort_status radsort_autotune(const void *keys, const uint32_t *values, size_t
                                 int digit_bits, void *stream, radsort_plan *plan);
 
 /*
- * radsort_autotune for both digit widths: tunes (or takes from the cache)
- * the plan for 8-bit and for 11-bit digits and returns the faster width in
- * *digit_bits with its plan (8 when the arrays are small enough that neither
- * is timed).  Pass both to radsort_sort_ex.  Same arguments, allocation,
+ * radsort_autotune and the digit width: tunes (or takes from the cache) the
+ * plan for 8-bit digits and returns 8 in *digit_bits, as a whole sort runs the
+ * same passes with both widths, except where the automatic plan is the chunk
+ * layout (2^31 elements and more): there 11-bit digits are tuned too and the
+ * faster width is returned with its plan.  Pass both to radsort_sort_ex.  Same arguments, allocation,
  * synchronisation and errors as radsort_autotune.
  */
 radsort_status radsort_autotune_digits(const void *keys, const uint32_t *values, size_t n, int key_bytes,

@@ -916,8 +916,17 @@ radsort_status radsort_autotune_digits(const void *keys, const uint32_t *values,
     radsort_plan p8{}, p11{};
     float m8, m11;
     radsort_status s = tune_one(keys, values, n, key_bytes, 8, stream, &p8, &m8);
-    if (s == RADSORT_OK)
-        s = tune_one(keys, values, n, key_bytes, 11, stream, &p11, &m11);
+    if (s != RADSORT_OK)
+        return s;
+    // Only the chunk layout sorts by the digits it is given: elsewhere a whole
+    // sort runs the same byte passes with both widths (digit_pass), and 11-bit
+    // digits cost more where a digit is sorted on its own (two passes each)
+    if (p8.layout != RADSORT_LAYOUT_CHUNKS) {
+        *digit_bits = 8;
+        *plan = p8;
+        return RADSORT_OK;
+    }
+    s = tune_one(keys, values, n, key_bytes, 11, stream, &p11, &m11);
     if (s != RADSORT_OK)
         return s;
     const bool eleven = m8 >= 0.f && m11 >= 0.f && m11 < m8;

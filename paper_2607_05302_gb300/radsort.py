@@ -159,7 +159,7 @@ def radsort_autotune(keys, values=None, *, digit_bits=8, stream=None):
 
 def radsort_autotune_digits(keys, values=None, *, stream=None):
     """(digit_bits, block_size, num_chunks, layout, shape) of the fastest plan
-    over both digit widths (timed on copies)."""
+    (timed on copies): 8-bit digits wherever both widths run the same passes."""
     p = Plan()
     d = ctypes.c_int(0)
     _ok(lib().radsort_autotune_digits(_ptr(keys), _ptr(values), keys.numel(), _key_bytes(keys),
