@@ -74,10 +74,11 @@ typedef enum {
  *    the alternate arrays inside the workspace, the paper's suggestion for
  *    arrays below Radsort's crossover (Sec. 5: use T as A').  The automatic
  *    plan takes it for n <= RADSORT_SCRATCH_MAX_N; radsort_sort_rounds never
- *    uses it.  Arrays of at most 155,648 elements of up to 8 bytes (106,496
- *    larger ones) are sorted in one launch in the shared memory of a
- *    thread-block cluster, with 8-bit digits whatever digit_bits says; they
- *    leave the workspace untouched and allocate none.
+ *    uses it.  Arrays of at most 155,648 elements of up to 8 bytes (larger
+ *    ones: 106,496 without a workspace, 57,344 with one) are sorted in one
+ *    launch in the shared memory of a thread-block cluster, with 8-bit digits
+ *    whatever digit_bits says; they leave the workspace untouched and allocate
+ *    none.
  */
 #define RADSORT_LAYOUT_AUTO 0u
 #define RADSORT_LAYOUT_CHUNKS 1u

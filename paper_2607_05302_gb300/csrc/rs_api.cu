@@ -669,7 +669,7 @@ static radsort_status sort_common(void *keys, uint32_t *values, size_t n, int ke
         bool own = false;
         if (ws && (workspace_bytes < need || !aligned16(ws)))
             return workspace_bytes < need ? RADSORT_ENOMEM : RADSORT_EINVAL;
-        if (n <= small_sort_max(key_bytes, hasv)) { // one launch, in shared memory (8-bit digits whatever the width)
+        if (n <= small_sort_max(key_bytes, hasv, ws != nullptr)) { // one launch, in shared memory (8-bit digits whatever the width)
             Scope sc(1, -1, st);
             const cudaError_t e = launch_small_sort(keys, values, static_cast<uint32_t>(n), key_bytes,
                                                     (flags & RADSORT_KEY_FLOAT32) != 0, st);

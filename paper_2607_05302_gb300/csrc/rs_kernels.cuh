@@ -157,9 +157,10 @@ struct SegGroup {
 };
 size_t lsd_group_bytes(const SegGroup &g, int kb, bool hasv);
 cudaError_t launch_lsd_group(void *keys, uint32_t *vals, const SegGroup &g, int kb, void *pool, cudaStream_t st);
-// a short array (n <= small_sort_max) sorted in one launch in a cluster's
-// shared memory; flt: keys are float32 bits, transformed on the way
-uint32_t small_sort_max(int kb, bool hasv);
+// a short array (n <= small_sort_max, which depends on whether the caller has
+// given a workspace) sorted in one launch in a cluster's shared memory; flt:
+// keys are float32 bits, transformed on the way
+uint32_t small_sort_max(int kb, bool hasv, bool workspace);
 cudaError_t launch_small_sort(void *keys, uint32_t *vals, uint32_t n, int kb, bool flt, cudaStream_t st);
 // batched segmented sort of the small and medium segments
 constexpr uint32_t SEG_MED = 1u << 18;

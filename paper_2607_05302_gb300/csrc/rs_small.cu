@@ -11,11 +11,14 @@
 // kernel does (half-warps, one word per digit), exchanges the CTAs' digit
 // counts through distributed shared memory, and scatters every element to its
 // place in the cluster's other buffer, on whichever CTA that is.
-// Measured (8-byte elements unless said otherwise, us a sort, workspace given;
-// before, through the round kernel: 55 at 1,000 and 65 from 10,000 to 155,648;
-// 12-byte elements 89 and 115-123): 1,000 9.7, 3,584 12.4, 10,000 16.5, 24,576
-// 20.6, 57,344 28.8, 106,496 43, 150,000 53; 12-byte 1,000 14.5, 24,576 41,
-// 106,496 94.  Past that the array no longer fits the cluster.
+// Measured (us; u32 + u32 with the copy of the input, workspace given, calls back
+// to back; boxes differ by a few percent): 1,000 24-26, 10,000 25, 24,576 29,
+// 57,344 39, 106,496 53, 130,000 62-66, 155,648 68 (the round kernel takes 72-81
+// from 155,649 to 200,003); u64 + u32 1,000 24-26, 24,576 57, 57,344 87, 57,345
+// 116, 106,496 134-136.  Replayed as graphs, without the copy, where launches cost
+// less: 12, 20, 24, 33, 48, 56-61, 63 (the round kernel 55-60) and 18, 52, 82,
+// 110, 129.  Past 155,648, and 106,496 of 12 bytes, the array no longer fits the
+// cluster; for the line with a workspace see small_sort_max.
 #include "rs_common.cuh"
 #include "rs_kernels.cuh"
 
@@ -313,7 +316,17 @@ cudaError_t small_dispatch(void *keys, uint32_t *vals, uint32_t n, int flt, cuda
 
 unsigned take_status_small() { return take_status_word(); }
 
-uint32_t small_sort_max(int kb, bool hasv) { return uint32_t(SM_MAXC * SM_T * small_items(kb, hasv)); }
+// The longest array sorted here.  12-byte elements scatter two words each across
+// the cluster, and past 7 a thread the round kernel is faster where it has its
+// workspace: 57,345 to 106,496 u64 + u32 111-118 us a call back to back against
+// 116-136 here, as graphs 82-88 against 110-130.  A call that has to allocate
+// the workspace still goes here: alone, after the pool has given its memory
+// back, 119-139 against 220-230.
+uint32_t small_sort_max(int kb, bool hasv, bool workspace)
+{
+    const int items = small_items(kb, hasv);
+    return uint32_t(SM_MAXC * SM_T * (items == 13 && workspace ? 7 : items));
+}
 
 cudaError_t launch_small_sort(void *keys, uint32_t *vals, uint32_t n, int kb, bool flt, cudaStream_t st)
 {
