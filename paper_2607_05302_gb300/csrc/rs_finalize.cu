@@ -320,11 +320,12 @@ __global__ void k_fz_order(FinArgs a)
 // rank in the sense of the kernels above.
 //
 // What bounds it is latency (about 16 dependent steps), so launches between
-// the steps cost most of it.  Finalize of 2^20 u32 + u32 (npi 3073) 45 us with
-// two passes in one CTA, 40 with this one; 2^22 (npi 9217) 70 and 60; 2^24 (npi
-// 33,793) 197 with 27 launches, 143 here.  The line at FZ_ONE_NPI: npi 2587
-// takes 33 us in one CTA and 37 in a cluster, 3073 and 5121 the same in both.
-// 16-bit fields set the line at FZ_PLAN_NPI.
+// the steps cost most of it.  Finalize of 2^20 u32 + u32 in blocks of 512 (npi
+// 3073) 45 us with two passes in one CTA, 40 with this one; in the blocks of 256
+// that the automatic plan takes (npi 5121, the cluster) 47; 2^22 (npi 9217) 70 and
+// 58; 2^24 (npi 33,793) 197 with 27 launches, 138 here.  The line at FZ_ONE_NPI:
+// npi 2587 takes 33 us in one CTA and 37 in a cluster, 3073 and 5121 the same in
+// both.  16-bit fields set the line at FZ_PLAN_NPI.
 constexpr uint32_t FZ_ONE_NPI = 4096, FZ_PLAN_NPI = 65534, FZ_CTAS = 8;
 constexpr uint32_t FZ_LEN = 0xFFFEu, FZ_HEAD = 0xFFFFu; // length field: longest, and the mark of a head's entry
 
@@ -352,21 +353,16 @@ template <bool MULTI> __device__ __forceinline__ void fz_plan(const FinArgs &a, 
         const uint32_t q = __umulhi(x, inv);
         return cluster_addr(sja + (x - q * per) * 8u, q);
     };
-    // Entries are read while their owners rewrite them: every access is relaxed
-    // (volatile within a CTA) and covers the entry, so a read sees one state whole
+    // Entries are read while their owners rewrite them: every access covers the
+    // entry and is relaxed -- volatile on the CTA's own (relaxed of system scope;
+    // relaxed accesses through the cluster's window took 2-3% longer), relaxed of
+    // cluster scope on others' -- so a read sees one state whole
     auto get = [&](uint32_t x) { return MULTI ? ld_relaxed64(at(x)) : ld64(&sj[x]); };
     auto put = [&](uint32_t x, unsigned long long e) {
         if (MULTI)
             st_relaxed64(at(x), e);
         else
             st64(&sj[x], e);
-    };
-    auto own = [&](uint32_t i) { return MULTI ? ld_relaxed64(sja + i * 8u) : ld64(&sj[i]); }; // entry x0 + i
-    auto put_own = [&](uint32_t i, unsigned long long e) {
-        if (MULTI)
-            st_relaxed64(sja + i * 8u, e);
-        else
-            st64(&sj[i], e);
     };
     auto sync = [&]() {
         if (MULTI)
@@ -381,7 +377,7 @@ template <bool MULTI> __device__ __forceinline__ void fz_plan(const FinArgs &a, 
     if (tid < 2)
         s_cnt[tid] = 0u;
     for (uint32_t i = tid; i < mine; i += nt)
-        put_own(i, fz_entry(x0 + i, 0u, 0u, 0u));
+        st64(&sj[i], fz_entry(x0 + i, 0u, 0u, 0u));
     sync();
     for (uint32_t q = gt; q < NL; q += gn) { // block at x moves to t
         const uint32_t x = a.pi[a.H + q], t = target_of(q, a.nA, a.nT);
@@ -397,7 +393,7 @@ template <bool MULTI> __device__ __forceinline__ void fz_plan(const FinArgs &a, 
             bool on[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) {
-                e[u] = i + u * nt < mine ? own(i + u * nt) : 0ull;
+                e[u] = i + u * nt < mine ? ld64(&sj[i + u * nt]) : 0ull;
                 on[u] = fz_min(e[u]) != 0u && fz_len(e[u]) < npi; // not to the path's end or round the cycle
             }
 #pragma unroll
@@ -411,7 +407,7 @@ template <bool MULTI> __device__ __forceinline__ void fz_plan(const FinArgs &a, 
                 const uint32_t mn = less ? fz_min(f[u]) : fz_min(e[u]);
                 const uint32_t dist = less ? fz_len(e[u]) + fz_dist(f[u]) : fz_dist(e[u]);
                 const uint32_t len = min(fz_len(e[u]) + fz_len(f[u]), FZ_LEN);
-                put_own(i + u * nt, fz_entry(fz_next(f[u]), mn, dist, len));
+                st64(&sj[i + u * nt], fz_entry(fz_next(f[u]), mn, dist, len));
                 more |= mn != 0u && len < npi;
             }
         }
@@ -475,7 +471,7 @@ template <bool MULTI> __device__ __forceinline__ void fz_plan(const FinArgs &a, 
         a.ctr[C_REC] = s_cnt[1];
     }
     for (uint32_t i = tid; i < mine; i += nt) { // order
-        const unsigned long long e = own(i);
+        const unsigned long long e = ld64(&sj[i]);
         unsigned long long hd = e;
         uint32_t r = 0;
         if (fz_len(e) == 0u)
