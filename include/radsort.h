@@ -310,7 +310,7 @@ radsort_status radsort_lsd_oop_scratch_size(size_t n, int key_bytes, int value_b
  * aligned has its first (at most 3) elements set aside, the rest sorted by
  * Radsort and those elements merged back, instead of the alternate buffers.
  * On 20,000 lognormal arrays (2^29 keys + values) the plans hold 9%, 3.4%
- * and 0.95% of the arrays' bytes; (1) and (2) run at about half the fastest
+ * and 1.3% of the arrays' bytes; (1) and (2) run at 43% of the fastest
  * plan's speed.  With a caller workspace the call
  * issues only kernel launches, memsets and event records / waits, so it can
  * be captured in a CUDA graph (make a first call with long segments before

@@ -205,9 +205,10 @@ static void auto_plan_chunks(size_t n, int kb, int vb, int db, radsort_plan *pl)
 // the array's bytes (below about 2^26 elements no block size meets 2%: the
 // look-back ring and tables alone take ~2 MB; a quarter keeps the footprint
 // well below an out-of-place sort's).
-// Measured (u32 keys + values, us a sort, b = 256, 512, 1024): 2^20 178, 149,
-// 136; 2^22 288, 246, 229; 2^24 762, 615, 572; 2^25 1294, 1148, 1037 -- small
-// blocks leave many copies and list entries per tile and many to permute.
+// Measured (u32 keys + values, us a sort alone, the GPU idle before it, b = 256,
+// 512, 1024): 2^20 178, 147, 138; 2^22 288, 246, 229; 2^24 763, 626, 576; 2^25
+// 1294, 1148, 1037 -- small blocks leave many copies and list entries per tile
+// and many to permute.
 static void auto_plan(size_t n, int kb, int vb, int db, radsort_plan *pl)
 {
     if (pl->layout != RADSORT_LAYOUT_CHUNKS && n < (size_t(1) << 31)) {
@@ -975,9 +976,9 @@ constexpr int SEG_STREAMS_ALT = 4;
 // the medium pass's scratch (one out-of-place buffer per CTA) is held to
 // this share of the arrays' bytes by running fewer CTAs (at least 16).
 // Measured on 20,000 lognormal arrays (2^29 keys + values, the longest
-// medium one near 2^18, long segments beside it on the library's streams):
-// 1.5% -> 7.1 Gkeys/s, 3% -> 13.5, 6% -> 24.0, no limit (2 CTAs per SM,
-// 14%) -> 20.7.  The low-memory plan (8-bit digits) sorts the medium
+// medium one near 2^18, long segments beside it in groups): 1.5% -> 18.2
+// Gkeys/s, 3% -> 34.3, 6% (127 CTAs) -> 43.6, no limit (a CTA on every SM,
+// 6.9%) -> 43.5.  The low-memory plan (8-bit digits) sorts the medium
 // segments in place instead, in a fixed 514 blocks of 32 elements per CTA.
 constexpr double SEG_MED_SHARE = 0.06;
 // few medium segments: those longer than SEG_LOW join the long ones when the
@@ -1061,10 +1062,12 @@ radsort_status seg_plan(const uint64_t *offh, size_t nseg, int kb, bool hasv, in
     sp->ip = level >= 1 && !oop && db == 8;
     // the in-place medium pass: two CTAs per SM, but one per SM on 7/8 of
     // the SMs when long segments run beside it, so that their sorts find SMs
-    // of their own (measured on 20,000 lognormal arrays, medium-in-place
-    // plan: 304 CTAs 17.0 Gkeys/s, 136 19.2, 120 17.3, 100 14.7; smallest
-    // plan: 304 13.7, 136 15.0, 120 15.6, 100 14.6; medium arrays alone: 304
-    // the fastest)
+    // of their own.  Set with the former round kernel (20,000 lognormal arrays,
+    // medium-in-place plan: 304 CTAs 17.0 Gkeys/s, 136 19.2; smallest plan: 13.7
+    // and 15.0).  With the present one, which needs the SMs for less long, 304
+    // would be faster (23.7 against 18.7; smallest plan 21.9 against 18.5) for
+    // 83 MB instead of 61 in the smallest plan; medium arrays alone: 304 the
+    // fastest (21.2, 133 CTAs 12.8)
     const size_t ip_ctas = nlong ? size_t(num_sms()) * 7 / 8 : size_t(seg_ip_ctas());
     sp->level = sp->ip ? level : 0;
     sp->med_ctas = !med_max ? 0
