@@ -12,7 +12,7 @@
 // counts through distributed shared memory, and scatters every element to its
 // place in the cluster's other buffer, on whichever CTA that is.
 // Measured (us; u32 + u32 with the copy of the input, workspace given, calls back
-// to back; boxes differ by a few percent): 1,000 24-26, 10,000 25, 24,576 29,
+// to back; machines differ by a few percent): 1,000 24-26, 10,000 25, 24,576 29,
 // 57,344 39, 106,496 53, 130,000 62-66, 155,648 68 (the round kernel takes 72-81
 // from 155,649 to 200,003); u64 + u32 1,000 24-26, 24,576 57, 57,344 87, 57,345
 // 116, 106,496 134-136.  Replayed as graphs, without the copy, where launches cost
